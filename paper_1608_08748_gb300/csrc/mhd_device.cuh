@@ -7,10 +7,9 @@
 // orderings and power-of-two scalings run on the integer pipes (inline PTX on the halves of the
 // doubles), quotients and roots take one Newton-Raphson step from the hardware seeds, and the
 // Riemann solver forms its speeds and eigenvector rows with few divisions and square roots.  The
-// PPM keeps the plain evaluation's edge values bit for bit outside the Step 4 blend (q6 is formed as
-// 6 q_c - 3 (q_L + q_R)); the FP64 build contracts a*b+c into one FMA.  The FP64 path agrees with a
-// plain evaluation to a few ulp per operation (about 1e-15 relative L1 after 50 steps of the 128^3
-// turbulence box).
+// parabolas are held as the deviations of their edges from the cell's value; the FP64 build contracts
+// a*b+c into one FMA.  The FP64 path agrees with a plain evaluation to a few ulp per operation (about
+// 1e-15 relative L1 after 50 steps of the 128^3 turbulence box).
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -143,60 +142,6 @@ struct Para {
   T L, R, d, q6;
 };
 
-// The limited slope of Sec. 2.1 Step 1 (the FP32 Eulerian pencils).  Selects, not branches, and
-// fmin for the minima (the operands are never NaN): the FP32 pencils are bound by instruction issue.
-template <typename T>
-__device__ __forceinline__ T slope_m(T qm, T q0, T qp) {
-  T dq = T(0.5) * (qp - qm);
-  T dp = qp - q0, dn = q0 - qm;
-  const T mn = fmin(fmin(fabs(dq), T(2) * fabs(dp)), T(2) * fabs(dn));
-  return dp * dn > T(0) ? copysign(mn, dq) : T(0);
-}
-
-// Steps 1-5 for cell i, evaluated as written, from q_{i-1}, q_i, q_{i+1}, the slopes of cells i - 1,
-// i, i + 1 and the second differences D+ = q_{i+2} - 2 q_{i+1} + q_i, D- = q_i - 2 q_{i-1} + q_{i-2}:
-// the FP32 Eulerian pencils take this form, carrying each slope to the next two cells (their bound
-// is instruction issue, and the form has no branches: the tests of Steps 2 and 4 are selects, the
-// division of eta is taken where it is not used, and the blend is q + hbar (q' - q)); ppm_lean
-// below serves the other parabolas.
-template <typename T>
-__device__ __forceinline__ Para<T> ppm_carried(T qm1, T qc, T qp1, T dmm, T dm0, T dmp, T Dp, T Dm) {
-  const T SIXTH = T(1.0 / 6.0);
-  T qL = T(0.5) * (qm1 + qc) - (dm0 - dmm) * SIXTH;
-  T qR = T(0.5) * (qc + qp1) - (dmp - dm0) * SIXTH;
-  T dq = qR - qL;
-  T q6 = T(6) * (qc - T(0.5) * (qL + qR));
-  {
-    const bool ext = (qL - qc) * (qc - qR) <= T(0);
-    const bool up = dq * q6 > dq * dq, dn = dq * q6 < -(dq * dq);
-    const T cL = T(3) * qc - T(2) * qR, cR = T(3) * qc - T(2) * qL;
-    const T nL = ext ? qc : (up ? cL : qL);
-    qR = ext ? qc : (!up && dn ? cR : qR);
-    qL = nL;
-  }
-  T qLp = qc - T(0.25) * dm0, qRp = qc + T(0.25) * dm0;
-  T dq2 = qp1 - qm1;
-  // min(|q_{i+1}|, |q_{i-1}|, |q_{i+1}| + |q_{i-1}|) is the smaller of the first two
-  const T mn = fmin(fabs(qp1), fabs(qm1));
-  const bool det = !(fabs(dq2) - T(0.01) * mn <= T(0) || Dp * Dm > T(0));
-  const T eta = (Dm - Dp) / (T(3) * dq2);  // discarded where det is false (dq2 may be 0 there)
-  const T hb = det ? fmax(fmin(T(20) * (eta - T(0.05)), T(1)), T(0)) : T(0);
-  qL = fma(hb, qLp - qL, qL);
-  qR = fma(hb, qRp - qR, qR);
-  Para<T> P;
-  P.L = qL;
-  P.R = qR;
-  P.d = qR - qL;
-  P.q6 = T(6) * (qc - T(0.5) * (qL + qR));
-  return P;
-}
-// the same parabola from q_{i-2} .. q_{i+2}
-template <typename T>
-__device__ __forceinline__ Para<T> ppm_direct(T qm2, T qm1, T qc, T qp1, T qp2) {
-  return ppm_carried(qm1, qc, qp1, slope_m(qm2, qm1, qc), slope_m(qm1, qc, qp1), slope_m(qc, qp1, qp2),
-                     qp2 - T(2) * qp1 + qc, qc - T(2) * qm1 + qm2);
-}
-
 // 2^(j/32) for j = 0 .. 31, correctly rounded (the table of the exponential exp_tang below)
 __device__ const double kExp2Frac32[32] = {
     0x1.0000000000000p+0, 0x1.059b0d3158574p+0, 0x1.0b5586cf9890fp+0, 0x1.11301d0125b51p+0,
@@ -283,16 +228,6 @@ __device__ __forceinline__ bool sign_bit_b(double x) {
   return r != 0;
 }
 __device__ __forceinline__ bool sign_bit_b(float x) { return signbit(x); }
-
-// Ordered key of a double: the signed 64-bit order of the keys is the order of the values, with
-// -0 below +0 (the magnitude bits of a negative value flipped).  Comparisons of keys run on the
-// integer pipe.
-__device__ __forceinline__ long long okey(double x) {
-  long long k;
-  asm("{\n\t.reg .s64 m;\n\tmov.b64 %0, %1;\n\tshr.s64 m, %0, 63;\n\t"
-      "and.b64 m, m, 0x7fffffffffffffff;\n\txor.b64 %0, %0, m;\n\t}" : "=l"(k) : "d"(x));
-  return k;
-}
 
 // x 2^-K (K = 1, 2) on the integer pipe: the exponent field lowered by K.  Equal to the FP64
 // product wherever that is a normal double, a zero, an infinity or a NaN; a product below the
@@ -384,6 +319,9 @@ __device__ __forceinline__ double sqrt_nr(double x) {
   if (__builtin_expect(!gt_nn(2.2250738585072014e-308, x), 1)) return x * rsqrt_nr(x);
   return sqrt(x);
 }
+// 1/sqrt of a positive normal value in the bulk type (FP64: the step above)
+__device__ __forceinline__ double rsqrt_n(double x) { return rsqrt_nr(x); }
+__device__ __forceinline__ float rsqrt_n(float x) { return rsqrtf(x); }
 // bulk-type forms: FP64 by the steps above; FP32 by the plain operations (the FP32 build already
 // takes the hardware-approximate division and square root)
 __device__ __forceinline__ double rcp_t(double x) { return rcp_nr(x); }
@@ -421,181 +359,182 @@ __device__ __forceinline__ double exp_tang(double x) {
   return scale_pow2(y, k >> 5);
 }
 
+// Sums and products of the bulk type where no FMA takes both (the face kernels write their FMAs out).
+template <typename T>
+__device__ __forceinline__ T add_t(T a, T b) { return a + b; }
+template <typename T>
+__device__ __forceinline__ T sub_t(T a, T b) { return a - b; }
+template <typename T>
+__device__ __forceinline__ T mul_t(T a, T b) { return a * b; }
+
+// The bit pattern of a double as two 32-bit words and back, and the powers of two that the limiter
+// takes on the integer pipe for magnitudes of normal doubles: 2 |x| (|x| + |x| for every finite
+// |x| from the normal range on) and |x| / 4 (below 2^-1020 the exponent is held at zero: a value
+// under the normal range, as good as the zero it stands for).
+__device__ __forceinline__ int hi_of(double x) {
+#ifdef __CUDA_ARCH__
+  return __double2hiint(x);
+#else
+  long long k;
+  __builtin_memcpy(&k, &x, 8);
+  return (int)(k >> 32);
+#endif
+}
+__device__ __forceinline__ double with_hi(double x, int hi) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(hi, __double2loint(x));
+#else
+  long long k;
+  __builtin_memcpy(&k, &x, 8);
+  k = (long long)(((unsigned long long)(unsigned)hi << 32) | ((unsigned long long)k & 0xffffffffull));
+  __builtin_memcpy(&x, &k, 8);
+  return x;
+#endif
+}
+__device__ __forceinline__ double twice_b(double x) { return with_hi(x, hi_of(x) + (1 << 20)); }
+__device__ __forceinline__ float twice_b(float x) { return x + x; }
+__device__ __forceinline__ double quarter_nn(double x) {
+  const int h = hi_of(x) - (2 << 20);
+  return with_hi(x, h > 0 ? h : 0);
+}
+__device__ __forceinline__ float quarter_nn(float x) { return 0.25f * x; }
+
 // Half the limited slope of Sec. 2.1 Step 1 for a cell with differences dn = q_0 - q_-1,
 // dp = q_1 - q_0 and s = q_1 - q_-1: the slope is min(|s|/2, 2|dp|, 2|dn|) with the sign of s where
-// dn and dp have one sign, else 0; halving it is exact, and saves the doublings.
+// dn and dp have one sign, else 0; halving it is exact, and saves the doublings.  Selects, not
+// branches (in FP64 on the integer pipe; in FP32 the minima are single instructions).
 template <typename T>
 __device__ __forceinline__ T half_slope(T s, T dn, T dp) {
-  if (!same_sign(dn, dp)) return T(0);
-  T m = min_nn(min_nn(scale_down_b<2>(abs_b(s)), abs_b(dp)), abs_b(dn));
-  return with_sign_b(m, s);
+  const T m = min_nn(min_nn(quarter_nn(abs_b(s)), abs_b(dp)), abs_b(dn));
+  return same_sign(dn, dp) ? with_sign_b(m, s) : T(0);
 }
 
-// Steps 2-5 from the Step 1 edge values qL, qR of cell i (value qc, halved slope h0), the second
-// differences D+ and D-, s0 = q_{i+1} - q_{i-1} and q_{i+1}, q_{i-1}.  Steps 2 and 5 are taken by
-// selects, not branches: partly taken branches leave FP64 lanes idle, and the FP64 pipe is the
-// bound.
+// Sec. 2.1 in deviations.  A cell's parabola is held as its value q and A = 2 (q - q^L),
+// B = 2 (q^R - q), twice the deviations of its edges.  With the halved slopes h and the difference
+// d = q_{j+1} - q_j the edge between the cells j and j+1 (Step 1) gives B_j = d - (2/3)(h_{j+1} - h_j)
+// and A_{j+1} = d + (2/3)(h_{j+1} - h_j): one subtraction and two FMAs for both.  In A and B the rest
+// of the method is short:
+//   Step 2: an extremum is A B <= 0 (then A = B = 0); Delta q q6 > (Delta q)^2 is |A| > 2 |B|, and its
+//           fix q^L = 3 q - 2 q^R is A = 2 B; the mirrored case is |B| > 2 |A|, B = 2 A.  No sum or
+//           product: comparisons and doublings.
+//   Step 4: the flattened edges q -+ (slope)/4 are A = B = h, so the blend is A += hbar (h - A),
+//           B += hbar (h - B).
+//   Step 5: Delta q = (A + B)/2 and q6 = 3 (A - B)/2 are not formed: the averages of Sec. 2.4 over
+//           the fraction y next to the right or the left edge are
+//             q + y u A/2 + u^2 B/2   and   q - u^2 A/2 - y u B/2   with u = 1 - y.
+// On the FP64 pipe, the bound of the FP64 faces, a streamed parabola takes 7 instructions besides
+// Step 4's blend (with edge values, Delta q and q6 it took 17), and an average the same two FMAs; on
+// the FP32 path it takes about half the instructions.  The deviations also round less: no edge value
+// is formed from which q is subtracted again.  With the Riemann solve below, one step of the turbulence
+// box went from 25.6 to 19.4 ms at 128^3 in FP64 (Eulerian faces 16.2 -> 12.8, Lagrangian 8.7 -> 5.6 ms)
+// and from 15.9 to 14.5 ms at 256^3 in FP32 (5.2 -> 4.5, 4.1 -> 3.4 ms).
 template <typename T>
-__device__ __forceinline__ Para<T> ppm_limit(T qL, T qR, T qc, T h0, T Dp, T Dm, T s0, T qp1, T qm1) {
-  // 6 q_c once per parabola (FP64); 3 q_c = (6 q_c) / 2 exactly
-  const T six_qc = T(6) * qc;
-  // Step 2: monotonicity
-  {
-    const T dq = qR - qL;
-    const T q6 = six_qc - T(3) * (qL + qR);
-    bool ext, up, dn;
-    if constexpr (sizeof(T) == 8) {
-      // the tests as orderings of the values on the integer pipe: (q_L - q_c)(q_c - q_R) > 0 is q_c
-      // strictly between q_L and q_R; dq q6 > dq^2 is q6 beyond dq on the side of its sign, and
-      // -dq q6 > dq^2 is q6 beyond -dq on the other side (exact comparisons instead of rounded
-      // products: the fixes are continuous at the ties, q_L = 3 q_c - 2 q_R there)
-      const long long kL = okey(qL), kc = okey(qc), kR = okey(qR);
-      ext = !((kL > kc && kc > kR) || (kL < kc && kc < kR));
-      const long long kd = okey(dq), k6 = okey(q6), kmd = okey(neg_b(dq));
-      const bool dpos = kd > 0, dneg = kd < -1;  // dq > 0, dq < 0 (keys of +0 and -0: 0 and -1)
-      up = (dpos && k6 > kd) || (dneg && k6 < kd);
-      dn = (dpos && k6 < kmd) || (dneg && k6 > kmd);
-    } else {
-      ext = !same_sign(qL - qc, qc - qR);
-      const T a = dq * q6, b = dq * dq;
-      up = gt_nn(a, b);
-      dn = !up && gt_nn(neg_b(a), b);
-    }
-    // the two overshoot fixes are exclusive: one candidate 3 qc - 2 q from the opposite edge
-    const T cand = scale_down_b<1>(six_qc) - T(2) * (up ? qR : qL);
-    const T qLm = ext ? qc : (up ? cand : qL);
-    const T qRm = ext ? qc : (dn ? cand : qR);
-    qL = qLm;
-    qR = qRm;
-  }
-  // Step 4: discontinuity detector
-  const T mn = min_nn(abs_b(qp1), abs_b(qm1));
-  if constexpr (sizeof(T) == 4) {
-    // FP32 (bound by instruction issue): selects, not branches; eta is divided out everywhere and
-    // discarded where the detector is off (s0 may be 0 there), and the blend is q + hbar (q' - q)
-    const bool det = gt_nn(abs_b(s0), T(0.01) * mn) && !same_sign(Dp, Dm);
-    const T eta = (Dm - Dp) / (T(3) * s0);
-    const T hb = det ? fmaxf(fminf(T(20) * (eta - T(0.05)), T(1)), T(0)) : T(0);
-    qL = fma(hb, (qc - T(0.5) * h0) - qL, qL);
-    qR = fma(hb, (qc + T(0.5) * h0) - qR, qR);
-  } else if (gt_nn(abs_b(s0), T(0.01) * mn) && !same_sign(Dp, Dm)) {
-    // eta = num / den with den = 3 s0 != 0 here; num_s = num sgn(den)
-    const T num = Dm - Dp;
-    const T num_s = sign_bit_b(s0) ? neg_b(num) : num;
-    const T qLp = qc - T(0.5) * h0, qRp = qc + T(0.5) * h0;
-    // eta > 1/20 as num_s > |den| / 20 = 0.15 |s0| and eta > 1/10 as num_s / 2 > 0.15 |s0| (halving is
-    // exact): one product serves both tests (at the two thresholds hbar is continuous, so their
-    // rounding cannot move the result)
-    const T ad20 = T(0.15) * abs_b(s0);
-    if (sizeof(T) == 8 && gt_nn(scale_down_b<1>(num_s), ad20)) {
-      // eta > 1/10: hbar = 1, the flattened values themselves (no FP64 division; in FP32 the
-      // division is cheaper than the branch)
-      qL = qLp;
-      qR = qRp;
-    } else if (gt_nn(num_s, ad20)) {
-      if constexpr (sizeof(T) == 8) {
-        // hbar = 20 (eta - 1/20) = 20 num / (3 s0) - 1 by the Newton-Raphson reciprocal (den is
-        // nonzero here).  hbar lies in (0, 1] here up to rounding: the clamp and the test compare
-        // on the integer pipe (a negative hbar orders below both 1 and 0), and the blend
-        // hbar q' + (1 - hbar) q is taken as q + hbar (q' - q)
-        T hb = fma(T(20) * num, rcp_nr(T(3) * s0), T(-1));
-        hb = min_nn(hb, T(1));
-        if (gt_nn(hb, T(0))) {
-          qL = fma(hb, qLp - qL, qL);
-          qR = fma(hb, qRp - qR, qR);
-        }
-      } else {
-        const T eta = num / (T(3) * s0);
-        T hb = T(20) * (eta - T(0.05));
-        hb = hb < T(1) ? hb : T(1);
-        if (hb > T(0)) {
-          qL = hb * qLp + (T(1) - hb) * qL;
-          qR = hb * qRp + (T(1) - hb) * qR;
-        }
-      }
+struct Dev {
+  T A, B;
+};
+
+// Steps 2 and 4 for a cell with unlimited deviations A, B, halved slope h0, second differences D+ and
+// D-, s0 = q_{+1} - q_{-1} and the two neighbours' values.  Step 4's eta = -(D+ - D-)/(3 s0) acts where
+// |s0| > min(|q_{+1}|, |q_{-1}|)/100 (the smaller of the paper's three values is one of the two) and
+// D+ D- <= 0; hbar = 20 (eta - 1/20) = (20/3)(D- - D+)/s0 - 1, clamped to [0, 1].
+__device__ __forceinline__ Dev<double> dev_limit(double A, double B, double h0, double Dp, double Dm, double s0,
+                                                 double qp1, double qm1) {
+  const bool mono = same_sign(A, B);
+  // comparisons of magnitudes on the integer pipe; where mono holds neither is zero
+  const double aA = abs_b(A), aB = abs_b(B), A2 = twice_b(A), B2 = twice_b(B);
+  const bool up = gt_nn(aA, abs_b(B2)), dn = gt_nn(aB, abs_b(A2));
+  A = mono ? (up ? B2 : A) : 0.0;
+  B = mono ? (dn ? A2 : B) : 0.0;
+  const double as0 = abs_b(s0);
+  if (gt_nn(as0, mul_t(0.01, min_nn(abs_b(qp1), abs_b(qm1)))) && !same_sign(Dp, Dm)) {
+    const double num = sub_t(Dm, Dp);
+    const double num_s = sign_bit_b(s0) ? neg_b(num) : num;
+    // eta > 1/20 as num sgn(s0) > 3 |s0| / 20 (hbar is continuous there, so the test's rounding cannot
+    // move the result); below it hbar = 0 and the division is not taken
+    if (gt_nn(num_s, mul_t(0.15, as0))) {
+      double hb = fma(mul_t(20.0 / 3.0, num), rcp_nr(s0), -1.0);
+      hb = min_nn(hb, 1.0);
+      hb = sign_bit_b(hb) ? 0.0 : hb;  // negative only by rounding
+      A = fma(hb, sub_t(h0, A), A);
+      B = fma(hb, sub_t(h0, B), B);
     }
   }
-  // Step 5
-  Para<T> P;
-  P.L = qL;
-  P.R = qR;
-  P.d = qR - qL;
-  P.q6 = six_qc - T(3) * (qL + qR);
-  return P;
+  return Dev<double>{A, B};
+}
+// FP32: bound by instruction issue, so selects instead of branches, and the reciprocal is taken
+// everywhere and discarded where the detector is off (s0 may be 0 there); the clamp is the FMA's own
+// saturation.
+__device__ __forceinline__ float saturate_f(float x) {
+#ifdef __CUDA_ARCH__
+  return __saturatef(x);
+#else
+  return x > 0.0f ? (x < 1.0f ? x : 1.0f) : 0.0f;
+#endif
+}
+__device__ __forceinline__ Dev<float> dev_limit(float A, float B, float h0, float Dp, float Dm, float s0, float qp1,
+                                                float qm1) {
+  const bool mono = A * B > 0.0f;
+  const float mA = min_nn(abs_b(A), 2.0f * abs_b(B)), mB = min_nn(abs_b(B), 2.0f * abs_b(A));
+  A = mono ? with_sign_b(mA, A) : 0.0f;
+  B = mono ? with_sign_b(mB, B) : 0.0f;
+  const bool det = gt_nn(abs_b(s0), 0.01f * min_nn(abs_b(qp1), abs_b(qm1))) && !(Dp * Dm > 0.0f);
+  const float hb = det ? saturate_f(fma((20.0f / 3.0f) * (Dm - Dp), rcp_t(s0), -1.0f)) : 0.0f;
+  return Dev<float>{fma(hb, h0 - A, A), fma(hb, h0 - B, B)};
 }
 
-// Sec. 2.1 Steps 1-5 for cell i from q_{i-2} .. q_{i+2}, with the Step 4 weights in the reading
-// where hbar weighs the flattened values q -+ delta_m q / 4 (the amendment acts in
-// discontinuities).  Written for few FP64 operations: the slopes are carried halved, the
-// differences q_{i+1} - q_{i-1} and the second differences are formed once, min(|q_{i+1}|,
-// |q_{i-1}|, |q_{i+1}| + |q_{i-1}|) is min(|q_{i+1}|, |q_{i-1}|), and eta = -(D+ - D-) / (3 dq) is
-// divided out only where it lies between 1/20 and 1/10 (below, hbar = 0 and Step 4 changes
-// nothing; above, hbar = 1 and the flattened values replace the edges; hbar = 20 (eta - 1/20)
-// clamped to [0, 1] is continuous at both ends, so the tests' rounding cannot move the result).
+// the deviations of the cell in the middle of q_{-2} .. q_{+2}
 template <typename T>
-__device__ __forceinline__ Para<T> ppm_lean(T qm2, T qm1, T qc, T qp1, T qp2) {
-  const T THIRD = T(1.0 / 3.0);  // twice 1/6, exactly
-  const T d0 = qm1 - qm2, d1 = qc - qm1, d2 = qp1 - qc, d3 = qp2 - qp1;
-  const T sm = qc - qm2, s0 = qp1 - qm1, sp = qp2 - qc;
+__device__ __forceinline__ Dev<T> dev_of(T qm2, T qm1, T qc, T qp1, T qp2) {
+  const T d0 = sub_t(qm1, qm2), d1 = sub_t(qc, qm1), d2 = sub_t(qp1, qc), d3 = sub_t(qp2, qp1);
+  const T sm = sub_t(qc, qm2), s0 = sub_t(qp1, qm1), sp = sub_t(qp2, qc);
   const T hm = half_slope(sm, d0, d1), h0 = half_slope(s0, d1, d2), hp = half_slope(sp, d2, d3);
-  // Step 1: edge values (dm0 - dmm) / 6 = (h0 - hm) / 3
-  const T qL = scale_down_b<1>(qm1 + qc) - (h0 - hm) * THIRD;
-  const T qR = scale_down_b<1>(qc + qp1) - (hp - h0) * THIRD;
-  // second differences D+ = q_{i+2} - 2 q_{i+1} + q_i, D- = q_i - 2 q_{i-1} + q_{i-2}: in FP64 as
-  // differences of the first differences (one instruction each, as the stream forms them)
-  T Dp, Dm;
-  if constexpr (sizeof(T) == 8) {
-    Dp = d3 - d2;
-    Dm = d1 - d0;
-  } else {
-    Dp = (qp2 - T(2) * qp1) + qc;
-    Dm = (qc - T(2) * qm1) + qm2;
-  }
-  return ppm_limit(qL, qR, qc, h0, Dp, Dm, s0, qp1, qm1);
+  const T A = fma(T(2.0 / 3.0), sub_t(h0, hm), d1), B = fma(T(-2.0 / 3.0), sub_t(hp, h0), d2);
+  return dev_limit(A, B, h0, sub_t(d3, d2), sub_t(d1, d0), s0, qp1, qm1);
 }
 
-// The parabolas of consecutive cells j, j+1, ... along a line, each from the quantities ppm_lean
-// forms for it (so bit for bit the same), where the difference q_{j+1} - q_j, the halved slope, the
-// edge value between two cells and the second difference centred on a cell are formed once and
-// shared by the neighbours that use them.  Prime with q_{J-2} .. q_{J+1}; each next(q_{j+2}) then
-// returns the parabola of the next cell j = J, J+1, ...
+// The deviations of consecutive cells j, j+1, ... along a line, each from the quantities dev_of forms
+// for it (so bit for bit the same), where the difference q_{j+1} - q_j, the halved slope, the edge and
+// the second difference centred on a cell are formed once and shared by the neighbours that use them.
+// Prime with q_{J-2} .. q_{J+1}; each next(q_{j+2}) then returns cell j = J, J+1, ..., whose value is
+// left in qm.  FP32 forms the differences dp and s0 again instead of carrying them (two instructions
+// against two registers).
 template <typename T>
-struct PPMStream {
+struct DevStream {
   T qm, q0, qp;  // q_{j-1}, q_j, q_{j+1}
   T dp;          // q_{j+1} - q_j
   T h0;          // halved slope of cell j
-  T eL;          // edge value between j-1 and j
+  T A;           // unlimited A of cell j
   T Cm, C0;      // second differences centred on j-1 and j
   T s0;          // q_{j+1} - q_{j-1}
 
   __device__ __forceinline__ void prime(T qa, T qb, T qc, T qd) {  // q_{J-2} .. q_{J+1}
-    const T THIRD = T(1.0 / 3.0);
-    const T d0 = qb - qa, d1 = qc - qb, d2 = qd - qc;
-    const T hm = half_slope(qc - qa, d0, d1);
-    s0 = qd - qb;
+    const T d0 = sub_t(qb, qa), d1 = sub_t(qc, qb), d2 = sub_t(qd, qc);
+    const T hm = half_slope(sub_t(qc, qa), d0, d1);
+    s0 = sub_t(qd, qb);
     h0 = half_slope(s0, d1, d2);
-    eL = scale_down_b<1>(qb + qc) - (h0 - hm) * THIRD;
-    Cm = d1 - d0;
-    C0 = d2 - d1;
+    A = fma(T(2.0 / 3.0), sub_t(h0, hm), d1);
+    Cm = sub_t(d1, d0);
+    C0 = sub_t(d2, d1);
     qm = qb;
     q0 = qc;
     qp = qd;
     dp = d2;
   }
-  __device__ __forceinline__ Para<T> next(T qn) {  // qn = q_{j+2}
-    const T THIRD = T(1.0 / 3.0);
-    const T d2 = qn - qp;
-    const T s1 = qn - q0;
+  __device__ __forceinline__ Dev<T> next(T qn) {  // qn = q_{j+2}
+    if constexpr (sizeof(T) == 4) {
+      dp = qp - q0;
+      s0 = qp - qm;
+    }
+    const T d2 = sub_t(qn, qp), s1 = sub_t(qn, q0);
     const T h1 = half_slope(s1, dp, d2);
-    const T C1 = d2 - dp;
-    const T eR = scale_down_b<1>(q0 + qp) - (h1 - h0) * THIRD;
-    Para<T> P = ppm_limit(eL, eR, q0, h0, C1, Cm, s0, qp, qm);
+    const T C1 = sub_t(d2, dp), t = sub_t(h1, h0);
+    const Dev<T> P = dev_limit(A, fma(T(-2.0 / 3.0), t, dp), h0, C1, Cm, s0, qp, qm);
+    A = fma(T(2.0 / 3.0), t, dp);
     qm = q0;
     q0 = qp;
     qp = qn;
     dp = d2;
     h0 = h1;
-    eL = eR;
     Cm = C0;
     C0 = C1;
     s0 = s1;
@@ -603,167 +542,212 @@ struct PPMStream {
   }
 };
 
-// Sec. 2.4: parabola averages over the domain of dependence of a wave of |speed| y h / tau
+// The parabola by its edge values, Delta q = q^R - q^L and q6 (the paper's own form), from the value
+// and the deviations, and the forms that return it; the kernels take the deviations.
 template <typename T>
-__device__ __forceinline__ T avg_right_end(const Para<T>& P, T y) {
-  const T TWO_THIRDS = T(2.0 / 3.0);
-  return P.R - T(0.5) * y * (P.d - P.q6 * (T(1) - TWO_THIRDS * y));
+__device__ __forceinline__ Para<T> para_of(T q, Dev<T> P) {
+  return Para<T>{q - T(0.5) * P.A, q + T(0.5) * P.B, T(0.5) * (P.A + P.B), T(1.5) * (P.A - P.B)};
 }
 template <typename T>
-__device__ __forceinline__ T avg_left_end(const Para<T>& P, T y) {
-  const T TWO_THIRDS = T(2.0 / 3.0);
-  return P.L + T(0.5) * y * (P.d + P.q6 * (T(1) - TWO_THIRDS * y));
+__device__ __forceinline__ Para<T> ppm_lean(T qm2, T qm1, T qc, T qp1, T qp2) {
+  return para_of(qc, dev_of(qm2, qm1, qc, qp1, qp2));
 }
+template <typename T>
+struct PPMStream : DevStream<T> {
+  __device__ __forceinline__ Para<T> next(T qn) {
+    const Dev<T> P = DevStream<T>::next(qn);
+    return para_of(this->qm, P);
+  }
+};
+// ... from the slopes of the cells i - 1, i, i + 1 and the second differences around them
+template <typename T>
+__device__ __forceinline__ T slope_m(T qm, T q0, T qp) {
+  return T(2) * half_slope(qp - qm, q0 - qm, qp - q0);
+}
+template <typename T>
+__device__ __forceinline__ Para<T> ppm_carried(T qm1, T qc, T qp1, T dmm, T dm0, T dmp, T Dp, T Dm) {
+  const T A = fma(T(1.0 / 3.0), dm0 - dmm, qc - qm1), B = fma(T(-1.0 / 3.0), dmp - dm0, qp1 - qc);
+  return para_of(qc, dev_limit(A, B, T(0.5) * dm0, Dp, Dm, qp1 - qm1, qp1, qm1));
+}
+template <typename T>
+__device__ __forceinline__ Para<T> ppm_direct(T qm2, T qm1, T qc, T qp1, T qp2) {
+  return ppm_carried(qm1, qc, qp1, slope_m(qm2, qm1, qc), slope_m(qm1, qc, qp1), slope_m(qc, qp1, qp2),
+                     qp2 - T(2) * qp1 + qc, qc - T(2) * qm1 + qm2);
+}
+
+// the coefficients of A and B in the averages over the fraction y (Sec. 2.4): y u / 2 and u^2 / 2
+template <typename T>
+struct AvgCoef {
+  T p, r;
+};
+template <typename T>
+__device__ __forceinline__ AvgCoef<T> avg_coef(T y) {
+  const T u = sub_t(T(1), y), hu = fma(T(-0.5), y, T(0.5));
+  return AvgCoef<T>{mul_t(y, hu), mul_t(u, hu)};
+}
+// the average next to the right edge of a cell less the cell's value, and the average next to the left
+// edge of a cell of value d
+template <typename T>
+__device__ __forceinline__ T inc_right(Dev<T> P, AvgCoef<T> k) { return fma(k.r, P.B, mul_t(k.p, P.A)); }
+template <typename T>
+__device__ __forceinline__ T inc_left(T d, Dev<T> P, AvgCoef<T> k) { return fma(-k.r, P.A, fma(-k.p, P.B, d)); }
 
 // ------------------------------------------------------------------------------------------------
 // Sec. 2.4 + App. A: Roe-type face state, eigenvectors and the characteristic Riemann solution.
-// wl/wr = (rho, p, gamma, B_t1, B_t2, sqrt(rho)) of the left/right cell; Bn the face field.
-// qs = (V_n, V_t1, V_t2, B_t1, B_t2, P).
+// Of each side: w = (rho, p, gamma, B_t1, B_t2, sqrt(rho)) of the cell, and the values and deviations of
+// its parabolas of (v_n, v_t1, v_t2, B_t1, B_t2, p).  Bn is the face field.  qs = (V_n, V_t1, V_t2, B_t1, B_t2, P).
+template <typename T>
+struct FaceSide {
+  T w[6];
+  T q[6];
+  Dev<T> P[6];
+};
+
+// The speeds, alpha factors and eigenvector entries are those of App. A in few FP64 instructions:
+//   one reciprocal of the weight sum; 1/sqrt(rho) gives 1/rho, sqrt(rho) and c_a = |B_n| / sqrt(rho);
+//   c_f^2 = (c^2 + c_a^2 + b_perp^2 + sq)/2 with sq = c_f^2 - c_s^2 =
+//     sqrt((c^2 - c_a^2)^2 + b_perp^2 (2 c^2 + 2 c_a^2 + b_perp^2)), sums of non-negative terms, and
+//     c_s = c c_a / c_f;
+//   with Z = c^2 - c_a^2 - b_perp^2: alpha_f^2 = (c^2 - c_s^2)/sq = (1 + Z/sq)/2 and alpha_s^2 =
+//     (c_f^2 - c^2)/sq = (1 - Z/sq)/2.  The larger of the two is formed from |Z|, without
+//     cancellation, and the other from alpha_f alpha_s = c b_perp / sq, with the one reciprocal square
+//     root of the larger: exactly 0 where B_perp = 0;
+//   1/sq comes with the square root of sq^2, |B_perp| with 1/|B_perp|.
+// The rows of the fast and the slow waves see v_t and B_t only through their components along B_perp,
+// and those of the Alfven waves only through the ones across it.  The components along B_perp
+// are taken of the parabolas' coefficients once per face, so the four magnetosonic waves average and
+// sum four variables instead of six and their rows have four entries; each pair +-c shares y and its
+// rows up to the sign of the velocity entries (s_+ from the left cell's right end, s_- from the right
+// cell's left end; R s_+ + (S R) s_- is R (s_+ - s_-) on the velocities and R (s_+ + s_-) on B_t, P).
 //
-// The speeds, alpha factors and eigenvector entries are those of App. A with 10 divisions and
-// square roots instead of 29: one reciprocal of the weight sum, 1/sqrt(rho) (giving 1/rho,
-// sqrt(rho), c_a = |B_n| / sqrt(rho) and the 1/sqrt(2 rho) of the Alfven rows), 1/c (giving c and
-// the 1/(2c^2), 1/(2 sqrt(rho) c) factors of L), 1/c_f (giving c_f and c_s = c c_a / c_f, from
-// c_f^2 c_s^2 = c^2 c_a^2) and 1/|B_perp|.  The left and right waves of each pair share their
-// rows up to the sign of the velocity components, so the rows are formed once.
+// All waves act on the averages less the left cell's values q_l, and q* = q_l + sum R s: with R L = I that
+// is the sum over the averages themselves, at the same count of instructions, and its rounding is that
+// of the differences between the cells, not of their values.
+template <typename T>
+__device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>& r, T Bn, T tau_h, T qs[6]) {
+  const T INV_SQRT2 = T(0.70710678118654752440), HALF = T(0.5);
+  const T iden = rcp_t(add_t(l.w[5], r.w[5]));
+  const T al = mul_t(l.w[5], iden), ar = mul_t(r.w[5], iden);  // the normalised weights
+  const T rho = fma(al, l.w[0], mul_t(ar, r.w[0]));
+  const T p = fma(al, l.w[1], mul_t(ar, r.w[1]));
+  const T gam = fma(al, l.w[2], mul_t(ar, r.w[2]));
+  const T Bt1 = fma(al, r.w[3], mul_t(ar, l.w[3]));  // crossed weights for B
+  const T Bt2 = fma(al, r.w[4], mul_t(ar, l.w[4]));
+
+  const T rs = rsqrt_n(rho);  // 1 / sqrt(rho)
+  const T irho = mul_t(rs, rs), sqr = mul_t(rho, rs);
+  const T gp = mul_t(gam, p);
+  const T c2 = mul_t(gp, irho);
+  const T ca2 = mul_t(mul_t(Bn, Bn), irho);
+  const T bp2 = fma(Bt1, Bt1, mul_t(Bt2, Bt2));
+  const T b2 = mul_t(bp2, irho);  // b_perp^2
+  const T X = sub_t(c2, ca2), s2 = add_t(c2, ca2), s = add_t(s2, b2);
+  const T sq2 = fma(X, X, mul_t(b2, fma(T(2), s2, b2)));
+  // the directions of B_perp; the degenerate case keeps |B_perp| itself
+  T by = INV_SQRT2, bz = INV_SQRT2, bper;
+  if (gt_nn(bp2, T(1e-24) * rho * s)) {
+    const T ib = rsqrt_n(bp2);
+    by = mul_t(Bt1, ib);
+    bz = mul_t(Bt2, ib);
+    bper = mul_t(bp2, ib);
+  } else {
+    bper = sqrt_t(bp2);
+  }
+  const T rc = rsqrt_n(c2), c = mul_t(c2, rc);
+  T sq = T(0), af = INV_SQRT2, as = INV_SQRT2;
+  {
+    const T isq = rsqrt_n(sq2), sqn = mul_t(sq2, isq);
+    if (gt_nn(sqn, T(1e-12) * s)) {
+      sq = sqn;
+      const T Z = sub_t(X, b2);
+      const T big2 = fma(mul_t(HALF, abs_b(Z)), isq, HALF);  // in [1/2, 1]
+      const T rb = rsqrt_n(big2), big = mul_t(big2, rb);
+      const T small = mul_t(mul_t(mul_t(c, bper), mul_t(rs, isq)), rb);
+      const bool fast = !sign_bit_b(Z);
+      af = fast ? big : small;
+      as = fast ? small : big;
+    }
+  }
+  const T cf2 = mul_t(HALF, add_t(s, sq));
+  const T rcf = rsqrt_n(cf2);
+  const T cf = mul_t(cf2, rcf), ca = mul_t(abs_b(Bn), rs);
+  const T cs = mul_t(mul_t(c, ca), rcf);
+  const bool neg = sign_bit_b(Bn) && gt_nn(abs_b(Bn), T(0));  // sign(0) = +1
+  const T bys = neg ? neg_b(by) : by, bzs = neg ? neg_b(bz) : bz;
+
+  const AvgCoef<T> ka = avg_coef(mul_t(ca, tau_h)), kf = avg_coef(mul_t(cf, tau_h)), ks = avg_coef(mul_t(cs, tau_h));
+
+  // the right cell's values less the left cell's
+  T d[6];
+#pragma unroll
+  for (int m = 0; m < 6; ++m) d[m] = sub_t(r.q[m], l.q[m]);
+  // the Alfven waves, on the components across B_perp: v = -bz v_t1 + by v_t2 (times sgn(B_n)),
+  // b = (bz B_t1 - by B_t2) / sqrt(rho); first, so that the tangential coefficients are not needed
+  // beyond their components along B_perp
+  T hv, hb;
+  {
+    T ql[5], qr[5];
+#pragma unroll
+    for (int m = 1; m < 5; ++m) {
+      ql[m] = inc_right(l.P[m], ka);
+      qr[m] = inc_left(d[m], r.P[m], ka);
+    }
+    const T vl = fma(bys, ql[2], -mul_t(bzs, ql[1])), vr = fma(bys, qr[2], -mul_t(bzs, qr[1]));
+    const T bl = fma(bz, ql[3], -mul_t(by, ql[4])), br = fma(bz, qr[3], -mul_t(by, qr[4]));
+    const T sp = fma(rs, bl, vl), sm = fma(-rs, br, vr);
+    hv = mul_t(HALF, add_t(sp, sm));
+    hb = mul_t(mul_t(HALF, sqr), sub_t(sp, sm));
+  }
+  // the magnetosonic waves on (v_n, v_par sgn(B_n), B_par, p): the +c_f wave has
+  // L = (lf, -ls, as i2sc, af i2r), R = (af cf, -as cs, as sc, af gp), the +c_s wave
+  // L = (ls, lf, -af i2sc, as i2r), R = (as cs, af cf, -af sc, as gp)
+  auto along = [&](T a, T b) { return fma(by, a, mul_t(bz, b)); };
+  auto along_s = [&](T a, T b) { return fma(bys, a, mul_t(bzs, b)); };
+  const Dev<T> lv = {along_s(l.P[1].A, l.P[2].A), along_s(l.P[1].B, l.P[2].B)};
+  const Dev<T> lb = {along(l.P[3].A, l.P[4].A), along(l.P[3].B, l.P[4].B)};
+  const Dev<T> rv = {along_s(r.P[1].A, r.P[2].A), along_s(r.P[1].B, r.P[2].B)};
+  const Dev<T> rb = {along(r.P[3].A, r.P[4].A), along(r.P[3].B, r.P[4].B)};
+  const T dv = along_s(d[1], d[2]), db = along(d[3], d[4]);
+  const T af_cf = mul_t(af, cf), as_cs = mul_t(as, cs);
+  const T i2c2 = mul_t(mul_t(HALF, rc), rc), i2sc = mul_t(mul_t(HALF, rs), rc), i2r = mul_t(i2c2, irho);
+  const T lf = mul_t(af_cf, i2c2), ls = mul_t(as_cs, i2c2);
+  auto pair = [&](AvgCoef<T> k, T l0, T l1, T l2, T l3, T& dif, T& sum) {
+    const T sp = fma(l0, inc_right(l.P[0], k),
+                     fma(l1, inc_right(lv, k), fma(l2, inc_right(lb, k), mul_t(l3, inc_right(l.P[5], k)))));
+    const T sm = fma(-l0, inc_left(d[0], r.P[0], k),
+                     fma(-l1, inc_left(dv, rv, k), fma(l2, inc_left(db, rb, k), mul_t(l3, inc_left(d[5], r.P[5], k)))));
+    dif = sub_t(sp, sm);
+    sum = add_t(sp, sm);
+  };
+  T difF, sumF, difS, sumS;
+  pair(kf, lf, -ls, mul_t(as, i2sc), mul_t(af, i2r), difF, sumF);
+  pair(ks, ls, lf, -mul_t(af, i2sc), mul_t(as, i2r), difS, sumS);
+  const T vpar = fma(af_cf, difS, -mul_t(as_cs, difF));
+  const T bpar = mul_t(mul_t(sqr, c), fma(as, sumF, -mul_t(af, sumS)));
+  qs[0] = fma(af_cf, difF, fma(as_cs, difS, l.q[0]));
+  qs[1] = fma(bys, vpar, fma(-bzs, hv, l.q[1]));
+  qs[2] = fma(bzs, vpar, fma(bys, hv, l.q[2]));
+  qs[3] = fma(by, bpar, fma(bz, hb, l.q[3]));
+  qs[4] = fma(bz, bpar, fma(-by, hb, l.q[4]));
+  qs[5] = fma(gp, fma(af, sumF, mul_t(as, sumS)), l.q[5]);
+}
+// the same from parabolas in the paper's form, whose values are L + A/2 with A = Delta q + q6/3 and
+// B = Delta q - q6/3
 template <typename T>
 __device__ __forceinline__ void riemann(const T wl[6], const T wr[6], T Bn, const Para<T> pl[6],
                                         const Para<T> pr[6], T tau_h, T qs[6]) {
-  const T INV_SQRT2 = T(0.70710678118654752440);
-  const T sl = wl[5], sr = wr[5];
-  const T iden = rcp_t(sl + sr);
-  const T al = sl * iden, ar = sr * iden;  // the normalised weights
-  const T rho = al * wl[0] + ar * wr[0];
-  const T p = al * wl[1] + ar * wr[1];
-  const T gam = al * wl[2] + ar * wr[2];
-  const T Bt1 = al * wr[3] + ar * wl[3];  // crossed weights for B
-  const T Bt2 = al * wr[4] + ar * wl[4];
-
-  const T rs = rsqrt_t(rho);  // 1 / sqrt(rho)
-  const T irho = rs * rs;
-  const T gp = gam * p;
-  const T c2 = gp * irho;
-  const T ca2 = (Bn * Bn) * irho;
-  const T bp2 = Bt1 * Bt1 + Bt2 * Bt2;
-  const T bp2r = bp2 * irho;
-  const T s = c2 + (ca2 + bp2r);
-  // fast and slow speeds without cancellation: with X = c^2 - c_a^2 and b_perp^2 = B_perp^2 / rho,
-  //   c_f^2 - c_s^2 = sqrt(X^2 + b_perp^2 (2 c^2 + 2 c_a^2 + b_perp^2)),
-  //   (c^2 - c_s^2)(c_f^2 - c^2) = c^2 b_perp^2,
-  // so alpha_s (or alpha_f) is exactly 0 where B_perp = 0; dcs = c^2 - c_s^2, dfc = c_f^2 - c^2
-  const T X = c2 - ca2;
-  const T sq = sqrt_t(X * X + bp2r * ((T(2) * c2 + T(2) * ca2) + bp2r));
-  // the larger of the two differences from the sum, the other from their product
-  T dcs, dfc;
-  if constexpr (sizeof(T) == 8) {
-    // one FP64 division for both signs of X, so a warp with both signs does not take two
-    const bool xpos = !sign_bit_b(X);  // at X = 0 either form holds
-    // (|X| + sq - bp2r) / 2 for X >= 0, (|X| + sq + bp2r) / 2 for X < 0
-    T big = scale_down_b<1>((abs_b(X) + sq) - (xpos ? bp2r : neg_b(bp2r)));
-    big = sign_bit_b(big) ? T(0) : big;
-    const T other = !gt_nn(T(2.2250738585072014e-308), big) ? (c2 * bp2r) * rcp_t(big)
-                    : gt_nn(big, T(0)) ? c2 * bp2r / big : T(0);
-    dcs = xpos ? big : other;
-    dfc = xpos ? other : big;
-  } else {
-    // the same selects in FP32, where they save the branch
-    const bool xpos = X >= T(0);
-    T big = T(0.5) * ((fabs(X) + sq) - (xpos ? bp2r : -bp2r));
-    big = fmax(big, T(0));
-    const T other = big > T(0) ? c2 * bp2r / big : T(0);
-    dcs = xpos ? big : other;
-    dfc = xpos ? other : big;
-  }
-  const T cf2 = c2 + dfc;
-  const T rc = rsqrt_t(c2), rcf = rsqrt_t(cf2);
-  const T c = c2 * rc, cf = cf2 * rcf, ca = abs_b(Bn) * rs;
-  const T cs = (c * ca) * rcf;
-  T af, as;
-  if (gt_nn(sq, T(1e-12) * s)) {
-    const T isq = rcp_t(sq);
-    af = sqrt_t(dcs * isq);
-    as = sqrt_t(dfc * isq);
-  } else {
-    af = INV_SQRT2;
-    as = INV_SQRT2;
-  }
-  T by, bz;
-  if (gt_nn(bp2, T(1e-24) * rho * s)) {
-    const T ibp = rsqrt_t(bp2);
-    by = Bt1 * ibp;
-    bz = Bt2 * ibp;
-  } else {
-    by = INV_SQRT2;
-    bz = INV_SQRT2;
-  }
-  const T sg = (sign_bit_b(Bn) && gt_nn(abs_b(Bn), T(0))) ? T(-1) : T(1);  // sign(0) = +1
-  const T sqr = rho * rs, sc = sqr * c, sr2 = sqr * INV_SQRT2;
-  const T i2c2 = scale_down_b<1>(rc * rc), i2sc = scale_down_b<1>(rs * rc), i2rc2 = i2c2 * irho;
-  const T isr2 = rs * INV_SQRT2;
-
-  // App. A rows of the +c_f and +c_s waves; the -c waves negate the v_n, v_t1, v_t2 entries
-  const T afcf = af * cf, ascs = as * cs, bys = by * sg, bzs = bz * sg;
-  const T Rf[6] = {afcf, -(ascs * bys), -(ascs * bzs), as * sc * by, as * sc * bz, af * gp};
-  const T Lf[6] = {afcf * i2c2, -(ascs * bys) * i2c2, -(ascs * bzs) * i2c2, as * by * i2sc,
-                   as * bz * i2sc, af * i2rc2};
-  const T Rs[6] = {ascs, afcf * bys, afcf * bzs, -(af * sc * by), -(af * sc * bz), as * gp};
-  const T Ls[6] = {ascs * i2c2, afcf * bys * i2c2, afcf * bzs * i2c2, -(af * by * i2sc),
-                   -(af * bz * i2sc), as * i2rc2};
-  // Alfven rows: v_t1, v_t2 entries shared, B_t1, B_t2 entries negated for the -c_a wave
-  const T Av[2] = {-(bzs * INV_SQRT2), bys * INV_SQRT2};
-  const T AL[2] = {bz * isr2, -(by * isr2)};
-  const T AR[2] = {sr2 * bz, -(sr2 * by)};
-
-#pragma unroll
-  for (int m = 0; m < 6; ++m) qs[m] = T(0);
-  const T TWO_THIRDS = T(2.0 / 3.0);
-  // s_k = L_k . qbar_k (qbar_k the domain-of-dependence average on the upwind side), q* = sum R_k s_k.
-  // The +c and -c waves of a pair share y, and their rows up to the sign S of the velocity entries:
-  // with s_+ = L . qbar_+ (left cell, right end) and s_- = (S L) . qbar_- (right cell, left end),
-  // R s_+ + (S R) s_- is R (s_+ - s_-) on v_n, v_t1, v_t2 and R (s_+ + s_-) on B_t1, B_t2, P.
-  auto magnetosonic_pair = [&](const T L[6], const T R[6], T speed) {
-    const T y = speed * tau_h;
-    const T hy = scale_down_b<1>(y), w = T(1) - TWO_THIRDS * y;
-    T pa = T(0), pb = T(0), ma = T(0), mb = T(0);
-#pragma unroll
+  auto side = [](const T w[6], const Para<T> P[6]) {
+    FaceSide<T> f;
     for (int m = 0; m < 6; ++m) {
-      // avg_right_end of the left cell, avg_left_end of the right cell (Sec. 2.4)
-      const T qp = pl[m].R - hy * (pl[m].d - pl[m].q6 * w);
-      const T qm = pr[m].L + hy * (pr[m].d + pr[m].q6 * w);
-      if (m < 3) {
-        pa = pa + L[m] * qp;
-        ma = ma + L[m] * qm;
-      } else {
-        pb = pb + L[m] * qp;
-        mb = mb + L[m] * qm;
-      }
+      f.w[m] = w[m];
+      f.P[m].A = P[m].d + P[m].q6 * T(1.0 / 3.0);
+      f.P[m].B = P[m].d - P[m].q6 * T(1.0 / 3.0);
+      f.q[m] = P[m].L + T(0.5) * f.P[m].A;
     }
-    const T sp = pa + pb, sm = mb - ma;
-    const T dif = sp - sm, sum = sp + sm;
-#pragma unroll
-    for (int m = 0; m < 6; ++m) qs[m] = qs[m] + R[m] * (m < 3 ? dif : sum);
+    return f;
   };
-  // Alfven pair: the v_t rows are shared, the B_t rows change sign
-  auto alfven_pair = [&]() {
-    const T y = ca * tau_h;
-    const T hy = scale_down_b<1>(y), w = T(1) - TWO_THIRDS * y;
-    T qp[5], qm[5];
-#pragma unroll
-    for (int m = 1; m < 5; ++m) {
-      qp[m] = pl[m].R - hy * (pl[m].d - pl[m].q6 * w);
-      qm[m] = pr[m].L + hy * (pr[m].d + pr[m].q6 * w);
-    }
-    const T sp = (Av[0] * qp[1] + Av[1] * qp[2]) + (AL[0] * qp[3] + AL[1] * qp[4]);
-    const T sm = (Av[0] * qm[1] + Av[1] * qm[2]) - (AL[0] * qm[3] + AL[1] * qm[4]);
-    const T sum = sp + sm, dif = sp - sm;
-    qs[1] = qs[1] + Av[0] * sum;
-    qs[2] = qs[2] + Av[1] * sum;
-    qs[3] = qs[3] + AR[0] * dif;
-    qs[4] = qs[4] + AR[1] * dif;
-  };
-  magnetosonic_pair(Lf, Rf, cf);  // waves 1, 2: +-c_f
-  magnetosonic_pair(Ls, Rs, cs);  // waves 3, 4: +-c_s
-  alfven_pair();                  // waves 5, 6: +-c_a
+  FaceSide<T> l = side(wl, pl), r = side(wr, pr);
+  riemann(l, r, Bn, tau_h, qs);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -199,9 +199,9 @@ __global__ void __launch_bounds__(512) kb_prim(const Box<T>* __restrict__ boxes,
 template <typename T>
 __host__ __device__ constexpr bool euler_streams() { return sizeof(T) == 8; }
 
-// The Eulerian pencils that stream their parabolas keep each primitive's PPMStream in this thread's
-// slots of dynamic shared memory between faces (9 values x 6 primitives; value k of primitive v at
-// [(9 v + k) blockDim.x + threadIdx.x], so a warp's accesses are consecutive).
+// The FP64 Eulerian pencils keep each primitive's DevStream in this thread's slots of dynamic shared
+// memory between faces (9 values x 6 primitives; value k of primitive v at [(9 v + k) blockDim.x +
+// threadIdx.x], so a warp's accesses are consecutive).
 template <typename T>
 __device__ __forceinline__ T& stream_slot(int v, int k) {
   extern __shared__ __align__(16) unsigned char stream_smem_raw[];
@@ -209,26 +209,26 @@ __device__ __forceinline__ T& stream_slot(int v, int k) {
   return sm[(9 * v + k) * blockDim.x + threadIdx.x];
 }
 template <typename T>
-__device__ __forceinline__ void stream_save(const PPMStream<T>& S, int v) {
+__device__ __forceinline__ void stream_save(const DevStream<T>& S, int v) {
   stream_slot<T>(v, 0) = S.qm;
   stream_slot<T>(v, 1) = S.q0;
   stream_slot<T>(v, 2) = S.qp;
   stream_slot<T>(v, 3) = S.dp;
   stream_slot<T>(v, 4) = S.h0;
-  stream_slot<T>(v, 5) = S.eL;
+  stream_slot<T>(v, 5) = S.A;
   stream_slot<T>(v, 6) = S.Cm;
   stream_slot<T>(v, 7) = S.C0;
   stream_slot<T>(v, 8) = S.s0;
 }
 template <typename T>
-__device__ __forceinline__ PPMStream<T> stream_load(int v) {
-  PPMStream<T> S;
+__device__ __forceinline__ DevStream<T> stream_load(int v) {
+  DevStream<T> S;
   S.qm = stream_slot<T>(v, 0);
   S.q0 = stream_slot<T>(v, 1);
   S.qp = stream_slot<T>(v, 2);
   S.dp = stream_slot<T>(v, 3);
   S.h0 = stream_slot<T>(v, 4);
-  S.eL = stream_slot<T>(v, 5);
+  S.A = stream_slot<T>(v, 5);
   S.Cm = stream_slot<T>(v, 6);
   S.C0 = stream_slot<T>(v, 7);
   S.s0 = stream_slot<T>(v, 8);
@@ -240,23 +240,22 @@ __device__ __forceinline__ PPMStream<T> stream_load(int v) {
 // two EMF contributions E = B x U of Sec. 2.5.
 template <typename T>
 __device__ __forceinline__ void store_face_fluxes(const FaceOut<T>& fo, idx_t f, T Bn, const T qs[6]) {
-  T Vn = qs[0], Vt1 = qs[1], Vt2 = qs[2], Bt1 = qs[3], Bt2 = qs[4], P = qs[5];
-  T pstar = P + T(0.5) * (Bn * Bn + Bt1 * Bt1 + Bt2 * Bt2);
-  fo.f[0][f] = pstar - Bn * Bn;
-  fo.f[1][f] = -(Bn * Bt1);
-  fo.f[2][f] = -(Bn * Bt2);
-  fo.f[3][f] = pstar * Vn - Bn * (Bn * Vn + Bt1 * Vt1 + Bt2 * Vt2);
+  const T Vn = qs[0], Vt1 = qs[1], Vt2 = qs[2], Bt1 = qs[3], Bt2 = qs[4], P = qs[5];
+  const T Bn2 = mul_t(Bn, Bn);
+  const T pstar = fma(T(0.5), fma(Bt1, Bt1, fma(Bt2, Bt2, Bn2)), P);
+  fo.f[0][f] = sub_t(pstar, Bn2);
+  fo.f[1][f] = -mul_t(Bn, Bt1);
+  fo.f[2][f] = -mul_t(Bn, Bt2);
+  fo.f[3][f] = fma(pstar, Vn, -mul_t(Bn, fma(Bn, Vn, fma(Bt1, Vt1, mul_t(Bt2, Vt2)))));
   fo.f[4][f] = Vn;
-  fo.f[5][f] = Bn * Vt1 - Bt1 * Vn;
-  fo.f[6][f] = Bt2 * Vn - Bn * Vt2;
+  fo.f[5][f] = fma(Bn, Vt1, -mul_t(Bt1, Vn));
+  fo.f[6][f] = fma(Bt2, Vn, -mul_t(Bn, Vt2));
 }
 
-// The FP32 Eulerian pencil: the five-cell stencil of each of the six primitives slides along the
-// pencil in registers (register moves; the loop over the faces stays rolled, since eight unrolled
-// copies of the Riemann solve overflow the instruction cache), and the left cell's density, gamma
-// and sqrt(rho) are carried from the previous face: ten loads per face instead of forty-three.
-// Each cell's limited slope is formed once and carried to the parabolas of the next two cells
-// (ppm_carried; the same operations on the same numbers as the five-point ppm_direct).  Where all
+// The FP32 Eulerian pencil: each of the six primitives streams along the pencil in registers (a
+// DevStream of seven values; the loop over the faces stays rolled, since eight unrolled copies of the
+// Riemann solve overflow the instruction cache), and the left cell's deviations, density, gamma and
+// sqrt(rho) are carried from the previous face: ten loads per face instead of forty-three.  Where all
 // cells f0 - 3 .. f1 + 1 of the pencil lie inside the grid they are addressed as base + i * stride
 // without the boundary map.
 //
@@ -305,28 +304,23 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, idx_t p, co
       for (int v = 0; v < 6; ++v) out[v] = qv[v][q];
     }
   };
-  T w[6][5];  // cells j - 2 .. j + 2 of the parabola of cell j
+  DevStream<T> S[6];
+  FaceSide<T> l, r;  // the face's two cells; l carries the previous face's right cell
+  {
+    T col[5][6];
 #pragma unroll
-  for (int o = 0; o < 5; ++o) {
-    T col[6];
-    load6(f0 - 3 + o, col);
+    for (int o = 0; o < 5; ++o) load6(f0 - 3 + o, col[o]);
 #pragma unroll
-    for (int v = 0; v < 6; ++v) w[v][o] = col[v];
+    for (int v = 0; v < 6; ++v) {
+      S[v].prime(col[0][v], col[1][v], col[2][v], col[3][v]);
+      l.P[v] = S[v].next(col[4][v]);  // cell f0 - 1
+    }
   }
-  Para<T> pl[6], pr[6];
-  T sa[6], sb[6];  // the slopes of cells i - 1 and i, carried to the parabola of cell i
-#pragma unroll
-  for (int v = 0; v < 6; ++v) {
-    pl[v] = ppm_direct(w[v][0], w[v][1], w[v][2], w[v][3], w[v][4]);  // cell f0 - 1
-    sa[v] = slope_m(w[v][1], w[v][2], w[v][3]);
-    sb[v] = slope_m(w[v][2], w[v][3], w[v][4]);
-  }
-  T rl, gl, sl;  // density, gamma and sqrt(rho) of the face's left cell
   {
     const idx_t q = cell_at(f0 - 1);
-    rl = B.s.rho[q];
-    gl = B.w.g[q];
-    sl = B.w.sr[q];
+    l.w[0] = B.s.rho[q];
+    l.w[2] = B.w.g[q];
+    l.w[5] = B.w.sr[q];
   }
   // the loads of a face are issued one face ahead, so that their latency overlaps the previous
   // face's Riemann solve: the new stencil cell i + 2 and the right cell i (density, gamma,
@@ -344,17 +338,16 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, idx_t p, co
   for (int k = 0; k < pencil_len<T>(); ++k) {
     if (k < nfp) {
       const int i = f0 + k;
-      // the left cell's p, B_t1, B_t2 are the centre of the window before it slides
-      const T pL = w[5][2], b1L = w[3][2], b2L = w[4][2];
 #pragma unroll
       for (int v = 0; v < 6; ++v) {
-        w[v][0] = w[v][1];
-        w[v][1] = w[v][2];
-        w[v][2] = w[v][3];
-        w[v][3] = w[v][4];
-        w[v][4] = nq[v];
+        l.q[v] = S[v].qm;  // cell i - 1
+        r.P[v] = S[v].next(nq[v]);  // cell i
+        r.q[v] = S[v].qm;
       }
-      const T rr = nr, gr = ng, sr = ns, Bn = nb;
+      r.w[0] = nr;
+      r.w[2] = ng;
+      r.w[5] = ns;
+      const T Bn = nb;
       if (k + 1 < nfp) {
         const idx_t cr = cell_at(i + 1);
         load6(i + 3, nq);
@@ -363,28 +356,16 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, idx_t p, co
         ns = B.w.sr[cr];
         nb = B.s.b[D][cr];
       }
-#pragma unroll
-      for (int v = 0; v < 6; ++v) {  // cell i
-        const T sc = slope_m(w[v][2], w[v][3], w[v][4]);
-        pr[v] = ppm_carried(w[v][1], w[v][2], w[v][3], sa[v], sb[v], sc, w[v][4] - T(2) * w[v][3] + w[v][2],
-                            w[v][2] - T(2) * w[v][1] + w[v][0]);
-        sa[v] = sb[v];
-        sb[v] = sc;
-      }
-      const T wl[6] = {rl, pL, gl, b1L, b2L, sl};
-      const T wr[6] = {rr, w[5][2], gr, w[3][2], w[4][2], sr};
+      l.w[1] = l.q[5];
+      l.w[3] = l.q[3];
+      l.w[4] = l.q[4];
+      r.w[1] = r.q[5];
+      r.w[3] = r.q[3];
+      r.w[4] = r.q[4];
       T qs[6];
-      riemann(wl, wr, Bn, pl, pr, tau_h, qs);
+      riemann(l, r, Bn, tau_h, qs);
       store_face_fluxes(B.fo[D], MHD_LATTICE(g, fbase + k * fstride), Bn, qs);
-#pragma unroll
-      for (int v = 0; v < 6; ++v) {
-        pl[v].R = pr[v].L + pr[v].d;  // q^R of cell i again, so that it need not live across the solve
-        pl[v].d = pr[v].d;
-        pl[v].q6 = pr[v].q6;
-      }
-      rl = rr;
-      gl = gr;
-      sl = sr;
+      l = r;
     }
   }
 }
@@ -394,7 +375,7 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, idx_t p, co
 // other two indices in [0, n)); each cell's parabolas are built once and serve both its faces.
 // Per face: the PPM parabolas of (v_n, v_t1, v_t2, B_t1, B_t2, p) of the two cells, the Riemann
 // solve, and the non-advective fluxes with the two EMF contributions E = B x U (Sec. 2.5).  The
-// FP64 form streams the parabolas (PPMStream in shared memory); the FP32 form slides the stencil.
+// FP64 form keeps the streams in shared memory, the FP32 form in registers.
 template <typename T, int D>
 __device__ __forceinline__ void euler_pencil(const Box<T>& B, idx_t p) {
   if constexpr (!euler_streams<T>()) {
@@ -417,50 +398,49 @@ __device__ __forceinline__ void euler_pencil(const Box<T>& B, idx_t p) {
     cc[D] = i;
     return cmap(g, cc[0], cc[1], cc[2]);
   };
-  Para<T> pl[6], pr[6];
+  FaceSide<T> l, r;  // the face's two cells; l.P carries the previous face's right cell
   {
     idx_t cell[5];
 #pragma unroll
     for (int o = 0; o < 5; ++o) cell[o] = cell_at(f0 - 3 + o);
 #pragma unroll
     for (int v = 0; v < 6; ++v) {
-      PPMStream<T> S;
+      DevStream<T> S;
       S.prime(qv[v][cell[0]], qv[v][cell[1]], qv[v][cell[2]], qv[v][cell[3]]);
-      pl[v] = S.next(qv[v][cell[4]]);  // cell f0 - 1
+      l.P[v] = S.next(qv[v][cell[4]]);  // cell f0 - 1
       stream_save(S, v);
     }
   }
   for (int i = f0; i < f1; ++i) {
-    idx_t cell[5];
-#pragma unroll
-    for (int o = 0; o < 5; ++o) cell[o] = cell_at(i - 2 + o);
+    const idx_t cl = cell_at(i - 1), cr = cell_at(i), cn = cell_at(i + 2);
 #pragma unroll
     for (int v = 0; v < 6; ++v) {
-      PPMStream<T> S = stream_load<T>(v);
-      pr[v] = S.next(qv[v][cell[4]]);  // cell i
+      DevStream<T> S = stream_load<T>(v);
+      l.q[v] = S.qm;               // cell i - 1
+      r.P[v] = S.next(qv[v][cn]);  // cell i
+      r.q[v] = S.qm;
       stream_save(S, v);
     }
-    idx_t cl = cell[1], cr = cell[2];
-    T wl[6] = {B.s.rho[cl], B.w.p[cl], B.w.g[cl], B.w.B[D1][cl], B.w.B[D2][cl], B.w.sr[cl]};
-    T wr[6] = {B.s.rho[cr], B.w.p[cr], B.w.g[cr], B.w.B[D1][cr], B.w.B[D2][cr], B.w.sr[cr]};
-    T Bn = B.s.b[D][cr];
+    l.w[0] = B.s.rho[cl];
+    l.w[1] = l.q[5];
+    l.w[2] = B.w.g[cl];
+    l.w[3] = l.q[3];
+    l.w[4] = l.q[4];
+    l.w[5] = B.w.sr[cl];
+    r.w[0] = B.s.rho[cr];
+    r.w[1] = r.q[5];
+    r.w[2] = B.w.g[cr];
+    r.w[3] = r.q[3];
+    r.w[4] = r.q[4];
+    r.w[5] = B.w.sr[cr];
+    const T Bn = B.s.b[D][cr];
     T qs[6];
-    riemann(wl, wr, Bn, pl, pr, tau_h, qs);
-    T Vn = qs[0], Vt1 = qs[1], Vt2 = qs[2], Bt1 = qs[3], Bt2 = qs[4], P = qs[5];
-    T pstar = P + T(0.5) * (Bn * Bn + Bt1 * Bt1 + Bt2 * Bt2);
+    riemann(l, r, Bn, tau_h, qs);
     int cf[3] = {c[0], c[1], c[2]};
     cf[D] = i;
-    idx_t f = fidx(g, cf[0], cf[1], cf[2]);
-    const FaceOut<T>& fo = B.fo[D];
-    fo.f[0][f] = pstar - Bn * Bn;
-    fo.f[1][f] = -(Bn * Bt1);
-    fo.f[2][f] = -(Bn * Bt2);
-    fo.f[3][f] = pstar * Vn - Bn * (Bn * Vn + Bt1 * Vt1 + Bt2 * Vt2);
-    fo.f[4][f] = Vn;
-    fo.f[5][f] = Bn * Vt1 - Bt1 * Vn;
-    fo.f[6][f] = Bt2 * Vn - Bn * Vt2;
+    store_face_fluxes(B.fo[D], fidx(g, cf[0], cf[1], cf[2]), Bn, qs);
 #pragma unroll
-    for (int v = 0; v < 6; ++v) pl[v] = pr[v];
+    for (int v = 0; v < 6; ++v) l.P[v] = r.P[v];
   }
 }
 
@@ -727,18 +707,20 @@ __device__ __forceinline__ void lag_face(const Box<T>& B, idx_t t) {
   T rl = B.s.rho[cl], rr = B.s.rho[cr];
   T isl = rsqrt_t(rl), isr = rsqrt_t(rr);
   T vn = (B.s.m[D][cl] * isl + B.s.m[D][cr] * isr) * rcp_t(rl * isl + rr * isr);
-  T y = fabs(vn) * tau_h;
+  const AvgCoef<T> k = avg_coef(T(fabs(vn) * tau_h));
   const T* q[7] = {B.s.rho, B.s.m[0], B.s.m[1], B.s.m[2], B.s.E, B.s.eint, B.s.rh2};
   idx_t f = fidx(g, c[0], c[1], c[2]);
   const int o0 = vn >= T(0) ? 0 : 1;  // upwind cell: stencil cells o0 .. o0 + 4
+  // the upwind average as q + kA A + kB B on either side
+  const T kA = o0 == 0 ? k.p : -k.r, kB = o0 == 0 ? k.r : -k.p;
   const int nv = B.nv;
   idx_t st[5];
 #pragma unroll
   for (int o = 0; o < 5; ++o) st[o] = o0 == 0 ? cell[o] : cell[o + 1];
   auto flux = [&](const T* a, int v) {
-    Para<T> P = ppm_lean(a[st[0]], a[st[1]], a[st[2]], a[st[3]], a[st[4]]);
-    T qb = o0 == 0 ? avg_right_end(P, y) : avg_left_end(P, y);
-    B.fo[D].f[v][f] = vn * qb;
+    const T qc = a[st[2]];
+    const Dev<T> P = dev_of(a[st[0]], a[st[1]], qc, a[st[3]], a[st[4]]);
+    B.fo[D].f[v][f] = vn * fma(kB, P.B, fma(kA, P.A, qc));
   };
 #pragma unroll
   for (int v = 0; v < 7; ++v) {
@@ -775,7 +757,6 @@ __device__ __forceinline__ void lag_pencil(const Box<T>& B, idx_t p) {
   const int f0 = c[D] * pencil_len<T>();
   const int nfp = (f0 + pencil_len<T>() < nf ? f0 + pencil_len<T>() : nf) - f0;
   const T tau_h = (T)B.sc->tau_h;
-  const T TWO_THIRDS = T(2.0 / 3.0);
   auto cell_at = [&](int i) {
     int cc[3] = {c[0], c[1], c[2]};
     cc[D] = i;
@@ -785,35 +766,32 @@ __device__ __forceinline__ void lag_pencil(const Box<T>& B, idx_t p) {
   cf[D] = f0;
   const idx_t fbase = fidx(g, cf[0], cf[1], cf[2]);
   const idx_t fstride = D == 0 ? 1 : (D == 1 ? (idx_t)(g.n[0] + 1) : (idx_t)(g.n[0] + 1) * (g.n[1] + 1));
-  // per face: v_n, and the average over the upwind fraction y = |v_n| tau / h written as
-  // E + shy (d + sgn q6 w) with E = q^R of the left cell (v_n >= 0, sgn = -1) or q^L of the right
-  // cell (sgn = +1), shy = sgn y / 2 and w = 1 - 2y/3 (the two forms of Sec. 2.4)
-  T vn[pencil_len<T>()], shy[pencil_len<T>()], w[pencil_len<T>()];
+  // per face: v_n and the coefficients of the average over the upwind fraction y = |v_n| tau / h,
+  // q + p A + r B of the left cell (v_n >= 0) or q - r A - p B of the right cell: with (X, Z) = (A, B)
+  // or (-B, -A) both are q + p X + r Z
+  T vn[pencil_len<T>()];
+  AvgCoef<T> kc[pencil_len<T>()];
   // v_n = (v_l sqrt(rho_l) + v_r sqrt(rho_r)) / (sqrt(rho_l) + sqrt(rho_r)) from the per-cell
   // m / sqrt(rho) and rho / sqrt(rho) = sqrt(rho), each formed once and carried to the next face
   T al, bl;
   {
     const idx_t c0 = cell_at(f0 - 1);
-    const T r0 = B.s.rho[c0], is0 = rsqrt_t(r0);
-    al = B.s.m[D][c0] * is0;
-    bl = r0 * is0;
+    const T r0 = B.s.rho[c0], is0 = rsqrt_n(r0);
+    al = mul_t(B.s.m[D][c0], is0);
+    bl = mul_t(r0, is0);
   }
 #pragma unroll
   for (int k = 0; k < pencil_len<T>(); ++k) {
     vn[k] = T(0);
-    shy[k] = T(0);
-    w[k] = T(1);
+    kc[k].p = kc[k].r = T(0);
     if (k < nfp) {
       const idx_t cr = cell_at(f0 + k);
-      const T rr = B.s.rho[cr], isr = rsqrt_t(rr);
-      const T ar = B.s.m[D][cr] * isr, br = rr * isr;
-      vn[k] = (al + ar) * rcp_t(bl + br);
+      const T rr = B.s.rho[cr], isr = rsqrt_n(rr);
+      const T ar = mul_t(B.s.m[D][cr], isr), br = mul_t(rr, isr);
+      vn[k] = mul_t(add_t(al, ar), rcp_t(add_t(bl, br)));
       al = ar;
       bl = br;
-      const T y = abs_b(vn[k]) * tau_h;
-      const T hy = scale_down_b<1>(y);
-      shy[k] = sign_bit_b(vn[k]) ? hy : neg_b(hy);  // v_n = -0 has y = 0
-      w[k] = T(1) - TWO_THIRDS * y;
+      kc[k] = avg_coef(mul_t(abs_b(vn[k]), tau_h));
     }
   }
   const int nv = B.nv;
@@ -822,18 +800,18 @@ __device__ __forceinline__ void lag_pencil(const Box<T>& B, idx_t p) {
     const T* a = v == 0 ? B.s.rho : v < 4 ? B.s.m[v - 1] : v == 4 ? B.s.E : v == 5 ? B.s.eint
                  : (IONS && v == 7) ? B.s.rhp : B.s.rh2;
     T* out = B.fo[D].f[v] + fbase;
-    PPMStream<T> S;
+    DevStream<T> S;
     S.prime(a[cell_at(f0 - 3)], a[cell_at(f0 - 2)], a[cell_at(f0 - 1)], a[cell_at(f0)]);
-    Para<T> Pl = S.next(a[cell_at(f0 + 1)]);  // cell f0 - 1
+    Dev<T> Pl = S.next(a[cell_at(f0 + 1)]);  // cell f0 - 1
 #pragma unroll
     for (int k = 0; k < pencil_len<T>(); ++k) {
       if (k < nfp) {
-        const Para<T> Pr = S.next(a[cell_at(f0 + k + 2)]);  // cell f0 + k
+        const T ql = S.qm;
+        const Dev<T> Pr = S.next(a[cell_at(f0 + k + 2)]);  // cell f0 + k
         const bool left = !sign_bit_b(vn[k]);  // v_n = -0: a zero flux either way
-        const T E = left ? Pl.R : Pr.L;
-        const T d = left ? Pl.d : Pr.d;
-        const T q6 = left ? neg_b(Pl.q6) : Pr.q6;
-        out[MHD_LATTICE(g, fbase + k * fstride) - fbase] = vn[k] * (E + shy[k] * (d + q6 * w[k]));
+        const T q = left ? ql : S.qm;
+        const T X = left ? Pl.A : neg_b(Pr.B), Z = left ? Pl.B : neg_b(Pr.A);
+        out[MHD_LATTICE(g, fbase + k * fstride) - fbase] = mul_t(vn[k], fma(kc[k].r, Z, fma(kc[k].p, X, q)));
         Pl = Pr;
       }
     }
