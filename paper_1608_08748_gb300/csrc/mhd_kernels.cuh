@@ -168,7 +168,7 @@ __device__ __forceinline__ void prim_cell(const Box<T>& B, idx_t c) {
   T Bc[3], m[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    Bc[d] = T(0.5) * (B.s.b[d][c] + B.s.b[d][up[d]]);
+    Bc[d] = mul_t(T(0.5), add_t(B.s.b[d][c], B.s.b[d][up[d]]));
     m[d] = B.s.m[d][c];
   }
   const T eint = B.s.eint[c];
@@ -179,8 +179,8 @@ __device__ __forceinline__ void prim_cell(const Box<T>& B, idx_t c) {
 #pragma unroll
   for (int d = 0; d < 3; ++d) B.w.B[d][c] = Bc[d];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) B.w.v[d][c] = m[d] * irho;
-  B.w.p[c] = (gmt - T(1)) * eint;
+  for (int d = 0; d < 3; ++d) B.w.v[d][c] = mul_t(m[d], irho);
+  B.w.p[c] = mul_t(sub_t(gmt, T(1)), eint);
   B.w.g[c] = gmt;
   B.w.sr[c] = sqrt_t(rho);
 }
@@ -536,13 +536,13 @@ __device__ __forceinline__ void edges_point(const Box<T>& B, idx_t t) {
     a[d2] = wrap(c[d2], g.n[d2], g.bc[d2]);
     int alo[3] = {c[0], c[1], c[2]};
     alo[d2] = wrap(c[d2] - 1, g.n[d2], g.bc[d2]);
-    T f1 = B.fo[d1].f[5][fidx(g, alo[0], alo[1], alo[2])] + B.fo[d1].f[5][fidx(g, a[0], a[1], a[2])];
+    const T f1 = add_t(B.fo[d1].f[5][fidx(g, alo[0], alo[1], alo[2])], B.fo[d1].f[5][fidx(g, a[0], a[1], a[2])]);
     int b[3] = {c[0], c[1], c[2]};
     b[d1] = wrap(c[d1], g.n[d1], g.bc[d1]);
     int blo[3] = {c[0], c[1], c[2]};
     blo[d1] = wrap(c[d1] - 1, g.n[d1], g.bc[d1]);
-    T f2 = B.fo[d2].f[6][fidx(g, blo[0], blo[1], blo[2])] + B.fo[d2].f[6][fidx(g, b[0], b[1], b[2])];
-    e[d] = T(0.25) * (f1 + f2);
+    const T f2 = add_t(B.fo[d2].f[6][fidx(g, blo[0], blo[1], blo[2])], B.fo[d2].f[6][fidx(g, b[0], b[1], b[2])]);
+    e[d] = mul_t(T(0.25), add_t(f1, f2));
   }
 #pragma unroll
   for (int d = 0; d < 3; ++d)
@@ -565,7 +565,10 @@ __global__ void __launch_bounds__(512) kb_edges(const Box<T>* __restrict__ boxes
 // by the FP64 pipe, so the constants are folded.)
 template <typename T>
 __device__ __forceinline__ T rk_value(T q, T q0, T a, T b, T gthS, int r) {
-  return r == 0 ? q + gthS : (a * q0 + b * q) + gthS;
+  if constexpr (sizeof(T) == 8)
+    return r == 0 ? add_t(q, gthS) : fma(a, q0, fma(b, q, gthS));
+  else
+    return r == 0 ? q + gthS : (a * q0 + b * q) + gthS;
 }
 
 // The cell kernels (primitives, edge EMFs, and the two updates in FP32) issue every load of a cell
@@ -592,22 +595,25 @@ __device__ __forceinline__ void euler_update_cell(const Box<T>& B, idx_t c, int 
   const T a = (T)RK3_A(r), bb = (T)RK3_B(r), gth = rk_gth(B, r);
   idx_t f0 = fidx(g, q[0], q[1], q[2]);
   idx_t fup[3] = {fidx(g, q[0] + 1, q[1], q[2]), fidx(g, q[0], q[1] + 1, q[2]), fidx(g, q[0], q[1], q[2] + 1)};
-  // -0 + x is x for every x, so the first addition to each sum folds away
-  T acc[5] = {T(-0.0), T(-0.0), T(-0.0), T(-0.0), T(-0.0)};  // m_x, m_y, m_z, rho E, -h div V
+  T acc[5];  // m_x, m_y, m_z, rho E, -h div V
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const int d1 = (d + 1) % 3, d2 = (d + 2) % 3;
     const FaceOut<T>& o = B.fo[d];
-    acc[d] = acc[d] + (o.f[0][f0] - o.f[0][fup[d]]);
-    acc[d1] = acc[d1] + (o.f[1][f0] - o.f[1][fup[d]]);
-    acc[d2] = acc[d2] + (o.f[2][f0] - o.f[2][fup[d]]);
-    acc[3] = acc[3] + (o.f[3][f0] - o.f[3][fup[d]]);
-    acc[4] = acc[4] + (o.f[4][f0] - o.f[4][fup[d]]);
+    auto sum = [&](T& a, int v) {
+      const T df = sub_t(o.f[v][f0], o.f[v][fup[d]]);
+      a = d == 0 ? df : add_t(a, df);
+    };
+    sum(acc[d], 0);
+    sum(acc[d1], 1);
+    sum(acc[d2], 2);
+    sum(acc[3], 3);
+    sum(acc[4], 4);
   }
   T Rv[5];  // h R: the flux-difference sums, and -(gamma - 1) rho eps h div V
 #pragma unroll
   for (int v = 0; v < 4; ++v) Rv[v] = acc[v];
-  Rv[4] = ((B.w.g[c] - T(1)) * B.s.eint[c]) * acc[4];
+  Rv[4] = mul_t(mul_t(sub_t(B.w.g[c], T(1)), B.s.eint[c]), acc[4]);
   if (GRAV) {
     // self-gravity (Sec. 2): -rho grad Phi and -rho v . grad Phi, central differences of the
     // potential of the step (periodic box); a separate instance, so that the update without
@@ -627,7 +633,7 @@ __device__ __forceinline__ void euler_update_cell(const Box<T>& B, idx_t c, int 
   // Flux-CT: d b_d / dt = -(curl E)_d on the face i_d - 1/2 of this cell
   auto curl_of = [&](int d) {
     const int d1 = (d + 1) % 3, d2 = (d + 2) % 3;
-    return (B.e[d1][fup[d2]] - B.e[d1][f0]) - (B.e[d2][fup[d1]] - B.e[d2][f0]);
+    return sub_t(sub_t(B.e[d1][fup[d2]], B.e[d1][f0]), sub_t(B.e[d2][fup[d1]], B.e[d2][f0]));
   };
   if constexpr (update_loads_first<T>()) {
     T qv[5], q0v[5], bv[3], b0v[3], curl[3];
@@ -645,26 +651,26 @@ __device__ __forceinline__ void euler_update_cell(const Box<T>& B, idx_t c, int 
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       if (r == 0) q0[v][c] = qv[v];
-      qq[v][c] = rk_value(qv[v], q0v[v], a, bb, gth * Rv[v], r);
+      qq[v][c] = rk_value(qv[v], q0v[v], a, bb, mul_t(gth, Rv[v]), r);
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       if (r == 0) B.s0.b[d][c] = bv[d];
-      B.s.b[d][c] = rk_value(bv[d], b0v[d], a, bb, gth * curl[d], r);
+      B.s.b[d][c] = rk_value(bv[d], b0v[d], a, bb, mul_t(gth, curl[d]), r);
     }
   } else {
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const T qv = qq[v][c], q0v = r ? q0[v][c] : T(0);
       if (r == 0) q0[v][c] = qv;
-      qq[v][c] = rk_value(qv, q0v, a, bb, gth * Rv[v], r);
+      qq[v][c] = rk_value(qv, q0v, a, bb, mul_t(gth, Rv[v]), r);
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const T curl = curl_of(d);
       const T bv = B.s.b[d][c], b0v = r ? B.s0.b[d][c] : T(0);
       if (r == 0) B.s0.b[d][c] = bv;
-      B.s.b[d][c] = rk_value(bv, b0v, a, bb, gth * curl, r);
+      B.s.b[d][c] = rk_value(bv, b0v, a, bb, mul_t(gth, curl), r);
     }
   }
 }
@@ -844,9 +850,12 @@ __device__ __forceinline__ void lag_update_cell(const Box<T>& B, idx_t c, int r)
   const int nv = B.nv;
   constexpr int NV = IONS ? 8 : 7;
   auto sum_of = [&](int v) {
-    T acc = T(-0.0);  // -0 + x is x: the first addition folds away
+    T acc = T(0);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) acc = acc + (B.fo[d].f[v][f0] - B.fo[d].f[v][fup[d]]);
+    for (int d = 0; d < 3; ++d) {
+      const T df = sub_t(B.fo[d].f[v][f0], B.fo[d].f[v][fup[d]]);
+      acc = d == 0 ? df : add_t(acc, df);
+    }
     return acc;
   };
   if constexpr (update_loads_first<T>()) {
@@ -872,7 +881,7 @@ __device__ __forceinline__ void lag_update_cell(const Box<T>& B, idx_t c, int r)
         const int v = h * H + i;
         if (v < NV && v < nv) {
           if (r == 0) q0[v][c] = qv[i];
-          qq[v][c] = rk_value(qv[i], q0v[i], a, bb, gth * acc[i], r);
+          qq[v][c] = rk_value(qv[i], q0v[i], a, bb, mul_t(gth, acc[i]), r);
         }
       }
     }
@@ -884,7 +893,7 @@ __device__ __forceinline__ void lag_update_cell(const Box<T>& B, idx_t c, int r)
       const T acc = sum_of(v);
       const T qv = qq[v][c], q0v = r ? q0[v][c] : T(0);
       if (r == 0) q0[v][c] = qv;
-      qq[v][c] = rk_value(qv, q0v, a, bb, gth * acc, r);
+      qq[v][c] = rk_value(qv, q0v, a, bb, mul_t(gth, acc), r);
     }
   }
 }
