@@ -254,7 +254,7 @@ def fp32_leg(M, I, torch, n=256, steps=10, warm=3, err_steps=100):
     dominant = max((k for k in kernels if k != "small"), key=lambda k: kernels[k])
     roof = None
     if FP32_FLOPS_PER_EULER_FACE:
-        faces = (n + 1) * n * n
+        faces = 3 * (n + 1) * n * n  # one launch takes the three directions
         launch_s = prof["euler_face"]["ms_total"] / prof["euler_face"]["launches"] * 1e-3
         measured = M.probe_fma_peak(fp64=False)
         achieved = FP32_FLOPS_PER_EULER_FACE * faces / launch_s / 1e12
@@ -539,7 +539,7 @@ def run_ours(args):
         v["share"] = v["ms_total"] / tot
     roofline = None
     if kernels:
-        faces_per_launch = (N_GRID + 1) * N_GRID * N_GRID
+        faces_per_launch = 3 * (N_GRID + 1) * N_GRID * N_GRID  # one launch takes the three directions
         avg_launch_s = kernels["euler_face"]["ms_total"] / kernels["euler_face"]["launches"] * 1e-3
         achieved = FLOPS_PER_EULER_FACE * faces_per_launch / avg_launch_s / 1e12
         measured = M.probe_fma_peak(fp64=True)

@@ -709,9 +709,9 @@ int mhd_check_flags(int clear, unsigned* flags) {
 
 int mhd_launches_per_step(mhd_sim* S) {
   if (!valid(S)) return fail(MHD_EINVAL, "mhd_launches_per_step: null sim");
-  // begin + 3 x (primitives, 3 faces, edges, update) + 3 x (3 faces) + 2 updates + the last
-  // update with the post stage + end (the first update of each stage stores its RK register Q^n)
-  return 1 + 3 * 6 + 3 * 3 + 2 + 1 + 1;
+  // begin + 3 x (primitives, faces, edges, update) + 3 x faces + 2 updates + the last update with the
+  // post stage + end (the first update of each stage stores its RK register Q^n)
+  return 1 + 3 * 4 + 3 + 2 + 1 + 1;
 }
 
 int mhd_profile(mhd_sim* S, double cfl, int steps, double* out_ms, int64_t* out_launches) {

@@ -43,48 +43,38 @@ struct Box {
   FaceOut<T> fo[3];  // Eulerian face outputs; the Lagrangian fluxes reuse fo[d].f[0..nv-1]
   T* e[3];
   int nv;            // advected fields of the Lagrangian stage (6; 7 with rho_H2; 8 with rho_H+)
+  int plen;          // faces of a pencil (set by the executor, choose_pencils)
+  int seg[3];        // pencils along each axis
   const T* phi;      // gravitational potential of the step (nullptr: no self-gravity)
   int* hflags;       // host-mapped copy of the error flags, written at the end of every step
 };
 
 struct Tiles {
-  const int* box;    // box of tile t
-  const int* start;  // first element of tile t inside its box
+  const int* box;    // box of tile t; its direction (of the face tables) in the bits from TILE_DIR_SHIFT on
+  const int* start;  // first element of tile t inside its box (and direction)
   int n;             // number of tiles
 };
+constexpr int TILE_DIR_SHIFT = 28;
 
-// domains of the tile tables
-enum { DOM_CELLS = 0, DOM_FACE_X = 1, DOM_FACE_Y = 2, DOM_FACE_Z = 3, DOM_LATTICE = 4,
-       DOM_PENCIL_X = 5, DOM_PENCIL_Y = 6, DOM_PENCIL_Z = 7, NDOM = 8 };
+// domains of the tile tables; those of faces and pencils hold the three directions one after another,
+// so one launch covers the three sweeps of a stage
+enum { DOM_CELLS = 0, DOM_FACES = 1, DOM_LATTICE = 2, DOM_PENCILS = 3, NDOM = 4 };
 
-// Faces are solved in pencils of pencil_len<T>() consecutive faces along the sweep direction: the
-// thread carries the parabolas (or the stencil) of the left cell from one face to the next, so
-// every cell's parabolas are built once per direction (plus one extra cell per pencil).  Measured
-// on the 256^3 FP32 and 128^3 FP64 steps: 12 faces for the float pencils (Eulerian faces 7.10 ms
-// against 7.40 with 8 and 7.15 with 16), 8 for the double ones (16.6 ms against 17.0 with 12 and
-// 17.6 with 16; their register files hold the stream of each face).
+// Faces are solved in pencils of consecutive faces along the sweep direction: the thread carries the
+// stream of the left cell from one face to the next, so every cell's parabolas are built once per
+// direction (plus one extra cell and the stream's priming per pencil).  pencil_len<T>() is the longest
+// pencil: on the 256^3 FP32 step 6 faces measured fastest (4.41 ms of Eulerian faces; 4.83 with 4, 4.55
+// with 8 and with 12), on the 128^3 FP64 one 8.  Small grids take shorter pencils, see
+// choose_pencils.
 template <typename T>
-__host__ __device__ constexpr int pencil_len() { return sizeof(T) == 4 ? 12 : 8; }
-template <typename T>
-__host__ __device__ __forceinline__ int pencil_segments(int n) { return (n + 1 + pencil_len<T>() - 1) / pencil_len<T>(); }
+__host__ __device__ constexpr int pencil_len() { return sizeof(T) == 4 ? 6 : 8; }
 
-// decode a cell index / a face index of direction D / a lattice index
-__device__ __forceinline__ void decode(idx_t t, int e0, int e1, int c[3]) {
-  c[0] = t % e0;
-  idx_t r = t / e0;
-  c[1] = (int)(r % e1);
-  c[2] = (int)(r / e1);
-}
-// the same with the grid's precomputed divisors (t >= 0): a cell index (cells), a face index of
-// direction D (D = 0, 1, 2) or a lattice index (D = 3)
-template <int D>
-__device__ __forceinline__ void decode_fast(const Geom& g, idx_t t, int c[3]) {
-  const FastDiv f0 = D == 0 || D == 3 ? g.dn1[0] : g.dn[0];
-  const FastDiv f1 = D == 1 || D == 3 ? g.dn1[1] : g.dn[1];
-  const unsigned r = fdiv((unsigned)t, f0);
-  c[0] = (int)((unsigned)t - r * f0.d);
-  const unsigned q = fdiv(r, f1);
-  c[1] = (int)(r - q * f1.d);
+// a lattice index with the grid's precomputed divisors (t >= 0)
+__device__ __forceinline__ void decode_lattice(const Geom& g, idx_t t, int c[3]) {
+  const unsigned r = fdiv((unsigned)t, g.dn1[0]);
+  c[0] = (int)((unsigned)t - r * g.dn1[0].d);
+  const unsigned q = fdiv(r, g.dn1[1]);
+  c[1] = (int)(r - q * g.dn1[1].d);
   c[2] = (int)q;
 }
 // a cell index with the precomputed divisors of n_x and n_y
@@ -96,21 +86,61 @@ __device__ __forceinline__ void decode_cell(const Geom& g, idx_t t, int c[3]) {
   c[2] = (int)q;
 }
 
-// pencil p of direction D -> (segment along D, the other two indices) in c.  In the FP64 x sweep
-// the y index runs fastest, so the threads of a warp share one segment and its face count (the last
-// segment of a row is shorter; the FP64 pipe, not the memory system, bounds those kernels); the
-// FP32 x sweep keeps the segment fastest for coalescing (the y-fastest order measured 12.9 against
-// 8.1 ms per 256^3 step there), and the y and z sweeps run x fastest as the cells do.
-template <typename T, int D>
-__device__ __forceinline__ void decode_pencil(idx_t p, const int ext[3], int c[3]) {
-  if (D == 0 && sizeof(T) == 8) {
-    c[1] = p % ext[1];
-    const idx_t r = p / ext[1];
-    c[0] = (int)(r % ext[0]);
-    c[2] = (int)(r / ext[0]);
-  } else {
-    decode(p, ext[0], ext[1], c);
+// A pencil of direction D: its faces f0 .. f0 + nfp - 1 along the axis, and the cells and faces of its
+// line (cell i at base + i stride, face i at fbase + i fstride).
+struct Line {
+  idx_t base, stride, fbase, fstride;
+  int n, bc;
+  int f0, nfp;
+  __device__ __forceinline__ idx_t cell(const Geom& g, int i) const {
+    return MHD_CELL(g, base + wrap(i, n, bc) * stride);
   }
+  __device__ __forceinline__ idx_t face(const Geom& g, int i) const { return MHD_LATTICE(g, fbase + i * fstride); }
+};
+// Pencil p of direction D.  In the FP64 x sweep the y index runs fastest, so the threads of a warp
+// share one segment and its face count (the last segment of a row is shorter; the FP64 pipe, not the
+// memory system, bounds those kernels); the FP32 x sweep keeps the segment fastest for coalescing (the
+// y-fastest order measured 12.9 against 8.1 ms per 256^3 step there), and the y and z sweeps run x
+// fastest as the cells do.  D is a run-time value, the same for the whole block: one body serves the
+// three sweeps (three instances in one kernel spilled 364 bytes of registers in FP32, against 72).
+template <typename T>
+__device__ __forceinline__ Line line_of_pencil(const Box<T>& B, int D, idx_t p) {
+  const Geom& g = B.g;
+  const int S = B.seg[D], nx = g.n[0], ny = g.n[1];
+  int seg, i = 0, j = 0, k = 0;
+  if (D == 0) {
+    if (sizeof(T) == 8) {
+      j = p % ny;
+      p /= ny;
+      seg = p % S;
+      k = p / S;
+    } else {
+      seg = p % S;
+      p /= S;
+      j = p % ny;
+      k = p / ny;
+    }
+  } else {
+    i = p % nx;
+    p /= nx;
+    if (D == 1) {
+      seg = p % S;
+      k = p / S;
+    } else {
+      j = p % ny;
+      seg = p / ny;
+    }
+  }
+  Line L;
+  L.n = g.n[D];
+  L.bc = g.bc[D];
+  L.base = (k * ny + j) * nx + i;
+  L.stride = D == 0 ? 1 : D == 1 ? nx : nx * ny;
+  L.fbase = (k * (ny + 1) + j) * (nx + 1) + i;
+  L.fstride = D == 0 ? 1 : D == 1 ? nx + 1 : (nx + 1) * (ny + 1);
+  L.f0 = seg * B.plen;
+  L.nfp = min(B.plen, L.n + 1 - L.f0);
+  return L;
 }
 
 #define MHD_TILE_LOOP(tl) for (int t_ = blockIdx.x; t_ < (tl).n; t_ += gridDim.x)
@@ -262,40 +292,24 @@ __device__ __forceinline__ void store_face_fluxes(const FaceOut<T>& fo, idx_t f,
 // STG (the x sweep only): the six window primitives of the pencil's row are read from shared memory,
 // srow[v * fs + x] for x in [0, n_x), where the block staged them (kb_euler_x_staged); the boundary map
 // then only wraps or clamps x within the row.
-template <typename T, int D, bool STG = false>
-__device__ __forceinline__ void euler_pencil_window(const Box<T>& B, idx_t p, const T* srow = nullptr,
+template <typename T, bool STG = false>
+__device__ __forceinline__ void euler_pencil_window(const Box<T>& B, int D, idx_t p, const T* srow = nullptr,
                                                     int fs = 0) {
-  static_assert(!STG || D == 0, "rows are staged for the x sweep only");
-  constexpr int D1 = (D + 1) % 3, D2 = (D + 2) % 3;
+  const int D1 = D == 2 ? 0 : D + 1, D2 = D == 0 ? 2 : D - 1;
   const Geom& g = B.g;
-  int ext[3] = {g.n[0], g.n[1], g.n[2]};
-  const int n = g.n[D], nf = n + 1;
-  ext[D] = pencil_segments<T>(n);
-  int c[3];
-  decode_pencil<T, D>(p, ext, c);
-  const int f0 = c[D] * pencil_len<T>();
-  const int nfp = (f0 + pencil_len<T>() < nf ? f0 + pencil_len<T>() : nf) - f0;
+  const Line L = line_of_pencil(B, D, p);
+  const int f0 = L.f0, nfp = L.nfp;
   const T tau_h = (T)B.sc->tau_h;
-  const bool inside = f0 >= 3 && f0 + nfp + 2 <= n;
-  int c0[3] = {c[0], c[1], c[2]};
-  c0[D] = 0;
-  const idx_t base = cidx(g, c0[0], c0[1], c0[2]);
-  const idx_t stride = D == 0 ? 1 : (D == 1 ? g.n[0] : g.n[0] * g.n[1]);
+  const bool inside = f0 >= 3 && f0 + nfp + 2 <= L.n;
   auto cell_at = [&](int i) -> idx_t {
-    if (inside) return MHD_CELL(g, base + i * stride);
-    int cc[3] = {c[0], c[1], c[2]};
-    cc[D] = i;
-    return cmap(g, cc[0], cc[1], cc[2]);
+    if (inside) return MHD_CELL(g, L.base + i * L.stride);
+    return L.cell(g, i);
   };
-  int cf[3] = {c[0], c[1], c[2]};
-  cf[D] = f0;
-  const idx_t fbase = fidx(g, cf[0], cf[1], cf[2]);
-  const idx_t fstride = D == 0 ? 1 : (D == 1 ? (idx_t)(g.n[0] + 1) : (idx_t)(g.n[0] + 1) * (g.n[1] + 1));
   const T* qv[6] = {B.w.v[D], B.w.v[D1], B.w.v[D2], B.w.B[D1], B.w.B[D2], B.w.p};
   // the six window primitives of cell i along the pencil
   auto load6 = [&](int i, T out[6]) {
     if constexpr (STG) {
-      const int x = inside ? i : wrap(i, n, g.bc[0]);
+      const int x = inside ? i : wrap(i, L.n, L.bc);
 #pragma unroll
       for (int v = 0; v < 6; ++v) out[v] = srow[v * fs + x];
     } else {
@@ -335,8 +349,8 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, idx_t p, co
     nb = B.s.b[D][cr];
   }
 #pragma unroll 1
-  for (int k = 0; k < pencil_len<T>(); ++k) {
-    if (k < nfp) {
+  for (int k = 0; k < nfp; ++k) {
+    {
       const int i = f0 + k;
 #pragma unroll
       for (int v = 0; v < 6; ++v) {
@@ -364,40 +378,31 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, idx_t p, co
       r.w[4] = r.q[4];
       T qs[6];
       riemann(l, r, Bn, tau_h, qs);
-      store_face_fluxes(B.fo[D], MHD_LATTICE(g, fbase + k * fstride), Bn, qs);
+      store_face_fluxes(B.fo[D], L.face(g, i), Bn, qs);
       l = r;
     }
   }
 }
 
 // Eulerian faces of direction D (Sec. 2.4): the face i_D - 1/2 lies between cells i_D - 1 and i_D.
-// One thread takes the faces i_D in [s P, min((s+1) P, n_D + 1)), P = pencil_len<T>(), of one pencil s (the
+// One thread takes the faces i_D in [s P, min((s+1) P, n_D + 1)), P = plen, of one pencil s (the
 // other two indices in [0, n)); each cell's parabolas are built once and serve both its faces.
 // Per face: the PPM parabolas of (v_n, v_t1, v_t2, B_t1, B_t2, p) of the two cells, the Riemann
 // solve, and the non-advective fluxes with the two EMF contributions E = B x U (Sec. 2.5).  The
 // FP64 form keeps the streams in shared memory, the FP32 form in registers.
-template <typename T, int D>
-__device__ __forceinline__ void euler_pencil(const Box<T>& B, idx_t p) {
+template <typename T>
+__device__ __forceinline__ void euler_pencil(const Box<T>& B, int D, idx_t p) {
   if constexpr (!euler_streams<T>()) {
-    euler_pencil_window<T, D>(B, p);
+    euler_pencil_window<T>(B, D, p);
     return;
   }
-  constexpr int D1 = (D + 1) % 3, D2 = (D + 2) % 3;
+  const int D1 = D == 2 ? 0 : D + 1, D2 = D == 0 ? 2 : D - 1;
   const Geom& g = B.g;
-  int ext[3] = {g.n[0], g.n[1], g.n[2]};
-  const int nf = g.n[D] + 1;
-  ext[D] = pencil_segments<T>(g.n[D]);
-  int c[3];
-  decode_pencil<T, D>(p, ext, c);
-  const int f0 = c[D] * pencil_len<T>();
-  const int f1 = f0 + pencil_len<T>() < nf ? f0 + pencil_len<T>() : nf;
+  const Line L = line_of_pencil(B, D, p);
+  const int f0 = L.f0, f1 = L.f0 + L.nfp;
   const T tau_h = (T)B.sc->tau_h;
   const T* qv[6] = {B.w.v[D], B.w.v[D1], B.w.v[D2], B.w.B[D1], B.w.B[D2], B.w.p};
-  auto cell_at = [&](int i) {
-    int cc[3] = {c[0], c[1], c[2]};
-    cc[D] = i;
-    return cmap(g, cc[0], cc[1], cc[2]);
-  };
+  auto cell_at = [&](int i) { return L.cell(g, i); };
   FaceSide<T> l, r;  // the face's two cells; l.P carries the previous face's right cell
   {
     idx_t cell[5];
@@ -436,9 +441,7 @@ __device__ __forceinline__ void euler_pencil(const Box<T>& B, idx_t p) {
     const T Bn = B.s.b[D][cr];
     T qs[6];
     riemann(l, r, Bn, tau_h, qs);
-    int cf[3] = {c[0], c[1], c[2]};
-    cf[D] = i;
-    store_face_fluxes(B.fo[D], fidx(g, cf[0], cf[1], cf[2]), Bn, qs);
+    store_face_fluxes(B.fo[D], L.face(g, i), Bn, qs);
 #pragma unroll
     for (int v = 0; v < 6; ++v) l.P[v] = r.P[v];
   }
@@ -453,7 +456,7 @@ __device__ __forceinline__ void euler_pencil(const Box<T>& B, idx_t p) {
 // need n_x a multiple of 4 (16-byte rows) and the launch's dynamic shared memory to hold them
 // (16 bytes of barrier, then [primitive][row][x]): the launcher takes this kernel only where every
 // box qualifies, and a tile that does not (which the launcher rules out) is flagged, not solved.
-// The results are those of kb_euler_pencil<T, 0> bit for bit.  It is opt-in (MHD_OPT_X_STAGE): on
+// The results are those of kb_euler_pencil bit for bit.  It is opt-in (MHD_OPT_X_STAGE): on
 // GB300 the x sweep measured slower with it (119 against 111 us per 128^3 launch), since the shared
 // memory takes L1 capacity from the sweep's other strided accesses (L1 hit rate 38 -> 16 %), and
 // staging all ten input fields as well (72 KB per block) kept the concurrent y and z sweeps' blocks
@@ -468,8 +471,8 @@ __global__ void __launch_bounds__(256, 2) kb_euler_x_staged(const Box<T>* __rest
   __syncthreads();
   unsigned parity = 0;
   MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    const int nx = B.g.n[0], S = pencil_segments<T>(nx);
+    const Box<T>& B = boxes[tl.box[t_] & ((1 << TILE_DIR_SHIFT) - 1)];
+    const int nx = B.g.n[0], S = B.seg[0];
     const idx_t total = (idx_t)S * B.g.n[1] * B.g.n[2];
     const idx_t p0 = tl.start[t_], p = p0 + (idx_t)threadIdx.x;
     const idx_t pe = p0 + (idx_t)blockDim.x < total ? p0 + (idx_t)blockDim.x : total;
@@ -502,19 +505,29 @@ __global__ void __launch_bounds__(256, 2) kb_euler_x_staged(const Box<T>* __rest
       mbar_wait_bounded(bar, phase);
       return;
     }
-    if (p < total) euler_pencil_window<T, 0, true>(B, p, rows + (int)(p / S - r_lo) * nx, nrows * nx);
+    if (p < total) euler_pencil_window<T, true>(B, 0, p, rows + (int)(p / S - r_lo) * nx, nrows * nx);
   }
 }
 
-template <typename T, int D>
+// The three sweeps in one launch: they read the same cells and write separate arrays, so a sweep's
+// last wave overlaps the next sweep's first, and the small grids pay one launch instead of three.
+template <typename T>
+__device__ __forceinline__ const Box<T>& box_of_tile(const Box<T>* boxes, int code, int& dir) {
+  dir = code >> TILE_DIR_SHIFT;
+  return boxes[code & ((1 << TILE_DIR_SHIFT) - 1)];
+}
+template <typename T>
+__device__ __forceinline__ idx_t pencil_count(const Box<T>& B, int dir) {
+  return (idx_t)(dir == 0 ? B.seg[0] : B.g.n[0]) * (dir == 1 ? B.seg[1] : B.g.n[1]) * (dir == 2 ? B.seg[2] : B.g.n[2]);
+}
+
+template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) kb_euler_pencil(const Box<T>* __restrict__ boxes, Tiles tl) {
   MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    idx_t p = tl.start[t_] + (idx_t)threadIdx.x;
-    idx_t total = (idx_t)(D == 0 ? pencil_segments<T>(B.g.n[0]) : B.g.n[0]) *
-                      (D == 1 ? pencil_segments<T>(B.g.n[1]) : B.g.n[1]) *
-                      (D == 2 ? pencil_segments<T>(B.g.n[2]) : B.g.n[2]);
-    if (p < total) euler_pencil<T, D>(B, p);
+    int dir;
+    const Box<T>& B = box_of_tile(boxes, tl.box[t_], dir);
+    const idx_t p = tl.start[t_] + (idx_t)threadIdx.x;
+    if (p < pencil_count(B, dir)) euler_pencil<T>(B, dir, p);
   }
 }
 
@@ -525,7 +538,7 @@ template <typename T>
 __device__ __forceinline__ void edges_point(const Box<T>& B, idx_t t) {
   const Geom& g = B.g;
   int c[3];
-  decode_fast<3>(g, t, c);
+  decode_lattice(g, t, c);
   T e[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -687,45 +700,46 @@ __global__ void __launch_bounds__(512) kb_euler_update(const Box<T>* __restrict_
 // ------------------------------------------------------------------------------------------------
 // Sec. 2.6 Lagrangian face flux for direction D: F = v_n q(-|v_n| tau) (v_n >= 0, left cell) or
 // v_n q(|v_n| tau) (right cell) with v_n the sqrt(rho)-weighted mean of the cell velocities.
-template <typename T, int D, bool IONS>
-__device__ __forceinline__ void lag_face(const Box<T>& B, idx_t t) {
+template <typename T, bool IONS>
+__device__ __forceinline__ void lag_face(const Box<T>& B, int D, idx_t t) {
   const Geom& g = B.g;
-  int c[3];
-  decode_fast<D>(g, t, c);
+  // face t of direction D: x runs over n_x (+ 1 in the x sweep) values, y over n_y (+ 1 in the y sweep)
+  const FastDiv d0 = D == 0 ? g.dn1[0] : g.dn[0], d1 = D == 1 ? g.dn1[1] : g.dn[1];
+  const unsigned r0 = fdiv((unsigned)t, d0);
+  const int i = (int)((unsigned)t - r0 * d0.d), k = (int)fdiv(r0, d1), j = (int)(r0 - (unsigned)k * d1.d);
   const T tau_h = (T)B.sc->tau_h;
+  const int nx = g.n[0], ny = g.n[1], n = g.n[D];
+  const int a = D == 0 ? i : D == 1 ? j : k;
+  const idx_t stride = D == 0 ? 1 : (D == 1 ? nx : nx * ny);
+  const idx_t cc = (k * ny + j) * nx + i;
   idx_t cell[6];
-  if (c[D] >= 3 && c[D] + 2 < g.n[D]) {
+  if (a >= 3 && a + 2 < n) {
     // the whole stencil inside the grid: a stride from this face's right cell, no boundary map
-    const idx_t stride = D == 0 ? 1 : (D == 1 ? g.n[0] : g.n[0] * g.n[1]);
-    const idx_t cc = cidx(g, c[0], c[1], c[2]);
 #pragma unroll
     for (int o = 0; o < 6; ++o) cell[o] = MHD_CELL(g, cc + (o - 3) * stride);
   } else {
+    const idx_t line = cc - a * stride;
 #pragma unroll
-    for (int o = 0; o < 6; ++o) {
-      int cc[3] = {c[0], c[1], c[2]};
-      cc[D] += o - 3;
-      cell[o] = cmap(g, cc[0], cc[1], cc[2]);
-    }
+    for (int o = 0; o < 6; ++o) cell[o] = MHD_CELL(g, line + wrap(a + o - 3, n, g.bc[D]) * stride);
   }
   idx_t cl = cell[2], cr = cell[3];
   // v_l sqrt(rho_l) = m_l / sqrt(rho_l) and sqrt(rho) = rho / sqrt(rho): two 1/sqrt and a division
   T rl = B.s.rho[cl], rr = B.s.rho[cr];
   T isl = rsqrt_t(rl), isr = rsqrt_t(rr);
   T vn = (B.s.m[D][cl] * isl + B.s.m[D][cr] * isr) * rcp_t(rl * isl + rr * isr);
-  const AvgCoef<T> k = avg_coef(T(fabs(vn) * tau_h));
+  const AvgCoef<T> kc = avg_coef(T(fabs(vn) * tau_h));
   const T* q[7] = {B.s.rho, B.s.m[0], B.s.m[1], B.s.m[2], B.s.E, B.s.eint, B.s.rh2};
-  idx_t f = fidx(g, c[0], c[1], c[2]);
+  const idx_t f = fidx(g, i, j, k);
   const int o0 = vn >= T(0) ? 0 : 1;  // upwind cell: stencil cells o0 .. o0 + 4
   // the upwind average as q + kA A + kB B on either side
-  const T kA = o0 == 0 ? k.p : -k.r, kB = o0 == 0 ? k.r : -k.p;
+  const T kA = o0 == 0 ? kc.p : -kc.r, kB = o0 == 0 ? kc.r : -kc.p;
   const int nv = B.nv;
   idx_t st[5];
 #pragma unroll
   for (int o = 0; o < 5; ++o) st[o] = o0 == 0 ? cell[o] : cell[o + 1];
-  auto flux = [&](const T* a, int v) {
-    const T qc = a[st[2]];
-    const Dev<T> P = dev_of(a[st[0]], a[st[1]], qc, a[st[3]], a[st[4]]);
+  auto flux = [&](const T* u, int v) {
+    const T qc = u[st[2]];
+    const Dev<T> P = dev_of(u[st[0]], u[st[1]], qc, u[st[3]], u[st[4]]);
     B.fo[D].f[v][f] = vn * fma(kB, P.B, fma(kA, P.A, qc));
   };
 #pragma unroll
@@ -739,39 +753,27 @@ __device__ __forceinline__ void lag_face(const Box<T>& B, idx_t t) {
   }
 }
 
-template <typename T, int D, bool IONS>
+template <typename T, bool IONS>
 __global__ void __launch_bounds__(256) kb_lag_face(const Box<T>* __restrict__ boxes, Tiles tl) {
   MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    idx_t t = tl.start[t_] + (idx_t)threadIdx.x;
-    idx_t total = (idx_t)(B.g.n[0] + (D == 0)) * (B.g.n[1] + (D == 1)) * (B.g.n[2] + (D == 2));
-    if (t < total) lag_face<T, D, IONS>(B, t);
+    int dir;
+    const Box<T>& B = box_of_tile(boxes, tl.box[t_], dir);
+    const idx_t t = tl.start[t_] + (idx_t)threadIdx.x;
+    if (t < (idx_t)(B.g.n[0] + (dir == 0)) * (B.g.n[1] + (dir == 1)) * (B.g.n[2] + (dir == 2)))
+      lag_face<T, IONS>(B, dir, t);
   }
 }
 
 // The same fluxes for the faces i_D - 1/2, i_D in [s P, min((s+1) P, n_D + 1)), of one
 // pencil s: the face velocities first, then field by field the parabolas of the pencil's cells in
 // one PPMStream along D, each face taking the average of its upwind cell.
-template <typename T, int D, bool IONS>
-__device__ __forceinline__ void lag_pencil(const Box<T>& B, idx_t p) {
+template <typename T, bool IONS>
+__device__ __forceinline__ void lag_pencil(const Box<T>& B, int D, idx_t p) {
   const Geom& g = B.g;
-  int ext[3] = {g.n[0], g.n[1], g.n[2]};
-  const int nf = g.n[D] + 1;
-  ext[D] = pencil_segments<T>(g.n[D]);
-  int c[3];
-  decode_pencil<T, D>(p, ext, c);
-  const int f0 = c[D] * pencil_len<T>();
-  const int nfp = (f0 + pencil_len<T>() < nf ? f0 + pencil_len<T>() : nf) - f0;
+  const Line L = line_of_pencil(B, D, p);
+  const int f0 = L.f0, nfp = L.nfp;
   const T tau_h = (T)B.sc->tau_h;
-  auto cell_at = [&](int i) {
-    int cc[3] = {c[0], c[1], c[2]};
-    cc[D] = i;
-    return cmap(g, cc[0], cc[1], cc[2]);
-  };
-  int cf[3] = {c[0], c[1], c[2]};
-  cf[D] = f0;
-  const idx_t fbase = fidx(g, cf[0], cf[1], cf[2]);
-  const idx_t fstride = D == 0 ? 1 : (D == 1 ? (idx_t)(g.n[0] + 1) : (idx_t)(g.n[0] + 1) * (g.n[1] + 1));
+  auto cell_at = [&](int i) { return L.cell(g, i); };
   // per face: v_n and the coefficients of the average over the upwind fraction y = |v_n| tau / h,
   // q + p A + r B of the left cell (v_n >= 0) or q - r A - p B of the right cell: with (X, Z) = (A, B)
   // or (-B, -A) both are q + p X + r Z
@@ -805,7 +807,7 @@ __device__ __forceinline__ void lag_pencil(const Box<T>& B, idx_t p) {
   for (int v = 0; v < nv; ++v) {
     const T* a = v == 0 ? B.s.rho : v < 4 ? B.s.m[v - 1] : v == 4 ? B.s.E : v == 5 ? B.s.eint
                  : (IONS && v == 7) ? B.s.rhp : B.s.rh2;
-    T* out = B.fo[D].f[v] + fbase;
+    T* out = B.fo[D].f[v];
     DevStream<T> S;
     S.prime(a[cell_at(f0 - 3)], a[cell_at(f0 - 2)], a[cell_at(f0 - 1)], a[cell_at(f0)]);
     Dev<T> Pl = S.next(a[cell_at(f0 + 1)]);  // cell f0 - 1
@@ -817,22 +819,20 @@ __device__ __forceinline__ void lag_pencil(const Box<T>& B, idx_t p) {
         const bool left = !sign_bit_b(vn[k]);  // v_n = -0: a zero flux either way
         const T q = left ? ql : S.qm;
         const T X = left ? Pl.A : neg_b(Pr.B), Z = left ? Pl.B : neg_b(Pr.A);
-        out[MHD_LATTICE(g, fbase + k * fstride) - fbase] = mul_t(vn[k], fma(kc[k].r, Z, fma(kc[k].p, X, q)));
+        out[L.face(g, f0 + k)] = mul_t(vn[k], fma(kc[k].r, Z, fma(kc[k].p, X, q)));
         Pl = Pr;
       }
     }
   }
 }
 
-template <typename T, int D, bool IONS>
+template <typename T, bool IONS>
 __global__ void __launch_bounds__(256, 1) kb_lag_pencil(const Box<T>* __restrict__ boxes, Tiles tl) {
   MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    idx_t p = tl.start[t_] + (idx_t)threadIdx.x;
-    idx_t total = (idx_t)(D == 0 ? pencil_segments<T>(B.g.n[0]) : B.g.n[0]) *
-                      (D == 1 ? pencil_segments<T>(B.g.n[1]) : B.g.n[1]) *
-                      (D == 2 ? pencil_segments<T>(B.g.n[2]) : B.g.n[2]);
-    if (p < total) lag_pencil<T, D, IONS>(B, p);
+    int dir;
+    const Box<T>& B = box_of_tile(boxes, tl.box[t_], dir);
+    const idx_t p = tl.start[t_] + (idx_t)threadIdx.x;
+    if (p < pencil_count(B, dir)) lag_pencil<T, IONS>(B, dir, p);
   }
 }
 

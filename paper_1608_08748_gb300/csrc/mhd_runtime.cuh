@@ -56,21 +56,21 @@ inline int profile_class(int kc) {
 // profiler tags: PROF_KC_BASE + kernel class for the tiled kernels, MHD_K_SMALL for the rest
 constexpr int PROF_KC_BASE = 100;
 inline int report_class(int tag) { return tag >= PROF_KC_BASE ? profile_class(tag - PROF_KC_BASE) : tag; }
-// domain of the tiles of each kernel class (per-direction kernels: first of three domains)
+// domain of the tiles of each kernel class
 // The Lagrangian faces run in pencils (kb_lag_pencil) where the parabolas are FP64: sharing the
 // differences, slopes and edge values of neighbouring cells saves FP64 instructions, the bound of
 // that path; the FP32 path keeps one thread per face (kb_lag_face).
 template <typename T>
 constexpr bool lag_in_pencils() { return sizeof(T) == 8; }
 
-// shared memory per thread of the Eulerian pencils: six PPMStreams where they stream
+// shared memory per thread of the FP64 Eulerian pencils: six DevStreams
 template <typename T>
 constexpr size_t euler_pencil_smem() { return euler_streams<T>() ? 6 * 9 * sizeof(T) : 0; }
 
 template <typename T>
 inline int class_domain(int kc) {
-  const int lag = lag_in_pencils<T>() ? DOM_PENCIL_X : DOM_FACE_X;
-  const int m[NKC] = {DOM_CELLS, DOM_PENCIL_X, DOM_LATTICE, DOM_CELLS, lag, DOM_CELLS, DOM_CELLS};
+  const int lag = lag_in_pencils<T>() ? DOM_PENCILS : DOM_FACES;
+  const int m[NKC] = {DOM_CELLS, DOM_PENCILS, DOM_LATTICE, DOM_CELLS, lag, DOM_CELLS, DOM_CELLS};
   return m[kc];
 }
 
@@ -86,6 +86,7 @@ inline int tile_slot(int block) { return block == 64 ? 0 : block == 128 ? 1 : bl
 struct TileTable {
   int* d = nullptr;  // [box..., start...] in one allocation
   int n = 0;
+  int first[4] = {0, 0, 0, 0};  // face tables: the tiles of direction q are first[q] .. first[q + 1]
 };
 
 // CUDA event pairs around launches while profiling
@@ -127,41 +128,39 @@ struct Exec {
   Profiler* prof = nullptr;
   bool ions = false;      // some box has H+ (reactions 5-8): the kernels with the ion code
   bool x_stage = false;   // the FP32 x sweep may stage its rows in shared memory (kb_euler_x_staged)
-  // The three directional sweeps of a stage are independent (each reads the cells and writes its
-  // own face arrays): the y and z sweeps run on two side streams forked from and joined to the
-  // launching stream, so that each sweep's tail overlaps the others' work.  In a captured step the
-  // fork and join become graph edges.
-  cudaStream_t side[2] = {nullptr, nullptr};
-  cudaEvent_t fork_ev = nullptr, join_ev[2] = {nullptr, nullptr};
 };
 
+// elements of a box in a domain (the face domains: of direction dir)
 template <typename T>
-long long domain_size(const Box<T>& B, int dom) {
+long long domain_size(const Box<T>& B, int dom, int dir) {
   const Geom& g = B.g;
+  long long e[3] = {g.n[0], g.n[1], g.n[2]};
   switch (dom) {
     case DOM_CELLS: return g.N;
-    case DOM_FACE_X: return (long long)(g.n[0] + 1) * g.n[1] * g.n[2];
-    case DOM_FACE_Y: return (long long)g.n[0] * (g.n[1] + 1) * g.n[2];
-    case DOM_FACE_Z: return (long long)g.n[0] * g.n[1] * (g.n[2] + 1);
-    case DOM_PENCIL_X: return (long long)pencil_segments<T>(g.n[0]) * g.n[1] * g.n[2];
-    case DOM_PENCIL_Y: return (long long)g.n[0] * pencil_segments<T>(g.n[1]) * g.n[2];
-    case DOM_PENCIL_Z: return (long long)g.n[0] * g.n[1] * pencil_segments<T>(g.n[2]);
+    case DOM_FACES: e[dir] += 1; break;
+    case DOM_PENCILS: e[dir] = B.seg[dir]; break;
     default: return g.NF;
   }
+  return e[0] * e[1] * e[2];
 }
 
 template <typename T>
 cudaError_t ensure_table(Exec<T>& X, int dom, int block) {
   TileTable& t = X.tab[dom][tile_slot(block)];
   if (t.d) return cudaSuccess;
+  const int ndir = dom == DOM_FACES || dom == DOM_PENCILS ? 3 : 1;
   std::vector<int> bx, st;
-  for (int b = 0; b < X.nb; ++b) {
-    long long n = domain_size(X.h[b], dom);
-    for (long long s = 0; s < n; s += block) {
-      bx.push_back(b);
-      st.push_back((int)s);
+  for (int q = 0; q < ndir; ++q) {
+    t.first[q] = (int)bx.size();
+    for (int b = 0; b < X.nb; ++b) {
+      const long long n = domain_size(X.h[b], dom, q);
+      for (long long s = 0; s < n; s += block) {
+        bx.push_back(b | (q << TILE_DIR_SHIFT));
+        st.push_back((int)s);
+      }
     }
   }
+  for (int q = ndir; q < 4; ++q) t.first[q] = (int)bx.size();
   t.n = (int)bx.size();
   if (t.n == 0) return cudaSuccess;
   cudaError_t e = cudaMalloc(&t.d, sizeof(int) * 2 * (size_t)t.n);
@@ -174,12 +173,8 @@ cudaError_t ensure_table(Exec<T>& X, int dom, int block) {
 template <typename T>
 cudaError_t ensure_tables(Exec<T>& X) {
   for (int kc = 0; kc < NKC; ++kc) {
-    int dom = class_domain<T>(kc);
-    int ndom = (dom == DOM_FACE_X || dom == DOM_PENCIL_X) ? 3 : 1;
-    for (int q = 0; q < ndom; ++q) {
-      cudaError_t e = ensure_table(X, dom + q, X.cfg[kc].block);
-      if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = ensure_table(X, class_domain<T>(kc), X.cfg[kc].block);
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -191,6 +186,16 @@ Tiles tiles_of(const Exec<T>& X, int dom, int block) {
   r.box = t.d;
   r.start = t.d + t.n;
   r.n = t.n;
+  return r;
+}
+// the tiles of the directions q0 .. q1 - 1 of a face table
+template <typename T>
+Tiles tiles_of_dirs(const Exec<T>& X, int dom, int block, int q0, int q1) {
+  const TileTable& t = X.tab[dom][tile_slot(block)];
+  Tiles r;
+  r.box = t.d + t.first[q0];
+  r.start = t.d + t.n + t.first[q0];
+  r.n = t.first[q1] - t.first[q0];
   return r;
 }
 
@@ -229,7 +234,7 @@ size_t euler_x_stage_bytes(const Exec<T>& X, int block) {
   for (int b = 0; b < X.nb; ++b) {
     const int nx = X.h[b].g.n[0];
     if (nx % 4 != 0) return 0;
-    const size_t rows = (size_t)((block - 1) / pencil_segments<T>(nx) + 2);
+    const size_t rows = (size_t)((block - 1) / X.h[b].seg[0] + 2);
     const size_t need = 16 + rows * 6 * (size_t)nx * sizeof(T);
     m = need > m ? need : m;
   }
@@ -246,14 +251,33 @@ cudaError_t prepare_kernels() {
     return cudaFuncSetAttribute(kb_euler_x_staged<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXStageMax);
   if constexpr (euler_pencil_smem<T>() > 0) {
     const int bytes = (int)(256 * euler_pencil_smem<T>());
-    cudaError_t e = cudaFuncSetAttribute(kb_euler_pencil<T, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kb_euler_pencil<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kb_euler_pencil<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    return e;
+    return cudaFuncSetAttribute(kb_euler_pencil<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   }
   return cudaSuccess;
+}
+
+// The length of the pencils: the longest of 1, 2, 4, ... faces (up to pencil_len<T>()) at which the
+// three sweeps of the boxes still have kPencilWarps warps per SM.  A pencil's own cost (one more cell
+// and the priming of its streams) falls with its length; a grid with fewer warps leaves the pipes idle
+// while each thread walks its pencil alone.  The faces' results do not depend on the length.  Measured
+// with 1 / 2 / 4 / 8 faces, ms per FP64 step: 128x4x4 0.24 / 0.31 / 0.43 / 0.69, 32^3 0.65 / 0.61 / 0.60 / 0.72,
+// 64^3 4.0 / 3.3 / 3.1 / 2.9; with 1 / 2 / 6 / 12 in FP32: 32^3 0.117 / 0.111 / 0.120 / 0.142, 256^3 19.0 / 16.4 /
+// 14.6 / 14.8.  (One launch per direction and pencils of 8 and 12 faces took 0.72 ms for 128x4x4 and
+// 0.154 ms for the FP32 32^3.)
+constexpr int kPencilWarps = 4;
+template <typename T>
+void choose_pencils(Exec<T>& X) {
+  int plen = pencil_len<T>();
+  for (; plen > 1; plen /= 2) {
+    long long pencils = 0;
+    for (const Box<T>& b : X.h)
+      for (int q = 0; q < 3; ++q) pencils += b.g.N / b.g.n[q] * ((b.g.n[q] + plen) / plen);
+    if (pencils >= 32ll * kPencilWarps * X.nsm) break;
+  }
+  for (Box<T>& b : X.h) {
+    b.plen = plen;
+    for (int q = 0; q < 3; ++q) b.seg[q] = (b.g.n[q] + plen) / plen;
+  }
 }
 
 template <typename T>
@@ -262,19 +286,10 @@ cudaError_t exec_init(Exec<T>& X, const std::vector<Box<T>>& boxes) {
   X.nb = (int)boxes.size();
   X.ions = false;
   for (const Box<T>& b : boxes) X.ions = X.ions || (b.ph.chem && b.ph.ions);
-  if (!X.side[0]) {
-    for (int k = 0; k < 2; ++k) {
-      cudaError_t es = cudaStreamCreateWithFlags(&X.side[k], cudaStreamNonBlocking);
-      if (es != cudaSuccess) return es;
-      es = cudaEventCreateWithFlags(&X.join_ev[k], cudaEventDisableTiming);
-      if (es != cudaSuccess) return es;
-    }
-    cudaError_t es = cudaEventCreateWithFlags(&X.fork_ev, cudaEventDisableTiming);
-    if (es != cudaSuccess) return es;
-  }
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&X.nsm, cudaDevAttrMultiProcessorCount, dev);
+  choose_pencils(X);
   cudaError_t e = prepare_kernels<T>();
   if (e != cudaSuccess) return e;
   default_cfgs(X);
@@ -297,14 +312,6 @@ void exec_free(Exec<T>& X) {
   X.d = nullptr;
   X.nb = 0;
   X.h.clear();
-  for (int k = 0; k < 2; ++k) {
-    if (X.side[k]) cudaStreamDestroy(X.side[k]);
-    if (X.join_ev[k]) cudaEventDestroy(X.join_ev[k]);
-    X.side[k] = nullptr;
-    X.join_ev[k] = nullptr;
-  }
-  if (X.fork_ev) cudaEventDestroy(X.fork_ev);
-  X.fork_ev = nullptr;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -316,13 +323,13 @@ void launch_ks(Exec<T>& X, cudaStream_t st, int kc, int dom, size_t smem_per_thr
   PScope p(X.prof, st, PROF_KC_BASE + kc);  // the profiler records the kernel class
   kernel<<<grid_of(t, c, X.nsm), c.block, smem_per_thread * c.block, st>>>(X.d, t, args...);
 }
-// the same with the block's dynamic shared memory given in bytes
-template <typename T, typename K, typename... A>
-void launch_kb(Exec<T>& X, cudaStream_t st, int kc, int dom, size_t bytes, K kernel, A... args) {
+// the directions q0 .. q1 - 1 of a face table, with the block's dynamic shared memory in bytes
+template <typename T, typename K>
+void launch_dirs(Exec<T>& X, cudaStream_t st, int kc, int dom, int q0, int q1, size_t bytes, K kernel) {
   const LaunchCfg& c = X.cfg[kc];
-  Tiles t = tiles_of(X, dom, c.block);
+  Tiles t = tiles_of_dirs(X, dom, c.block, q0, q1);
   PScope p(X.prof, st, PROF_KC_BASE + kc);
-  kernel<<<grid_of(t, c, X.nsm), c.block, bytes, st>>>(X.d, t, args...);
+  kernel<<<grid_of(t, c, X.nsm), c.block, bytes, st>>>(X.d, t);
 }
 template <typename T, typename K, typename... A>
 void launch_k(Exec<T>& X, cudaStream_t st, int kc, int dom, K kernel, A... args) {
@@ -341,26 +348,6 @@ void launch_small(Exec<T>& X, cudaStream_t st, int which, double cfl = 0, double
   if (which == 3) kb_zero_dmax<T><<<g, 128, 0, st>>>(X.d, X.nb);
 }
 
-// the x, y, z sweeps sw(dir, stream): forked onto the side streams, or in order on st while the
-// per-class profiler runs (its events bracket launches on st)
-template <typename T, typename F>
-void launch_sweeps(Exec<T>& X, cudaStream_t st, F sw) {
-  if (!X.side[0] || (X.prof && X.prof->on)) {
-    for (int d = 0; d < 3; ++d) sw(d, st);
-    return;
-  }
-  cudaEventRecord(X.fork_ev, st);
-  cudaStreamWaitEvent(X.side[0], X.fork_ev, 0);
-  cudaStreamWaitEvent(X.side[1], X.fork_ev, 0);
-  sw(0, st);
-  sw(1, X.side[0]);
-  sw(2, X.side[1]);
-  for (int k = 0; k < 2; ++k) {
-    cudaEventRecord(X.join_ev[k], X.side[k]);
-    cudaStreamWaitEvent(st, X.join_ev[k], 0);
-  }
-}
-
 template <typename T>
 void launch_euler_stage(Exec<T>& X, cudaStream_t st) {
   NvtxRange range("Eulerian stage with Flux-CT (Sec. 2.4, 2.5)");
@@ -371,20 +358,16 @@ void launch_euler_stage(Exec<T>& X, cudaStream_t st) {
       launch_k(X, st, KC_PRIM, DOM_CELLS, kb_prim<T, true>);
     else
       launch_k(X, st, KC_PRIM, DOM_CELLS, kb_prim<T, false>);
-    launch_sweeps(X, st, [&](int d, cudaStream_t s) {
-      if (d == 0) {
-        if constexpr (!euler_streams<T>()) {
-          const size_t xs = X.x_stage ? euler_x_stage_bytes(X, X.cfg[KC_EFACE].block) : 0;
-          if (xs > 0) {
-            launch_kb(X, s, KC_EFACE, DOM_PENCIL_X, xs, kb_euler_x_staged<T>);
-            return;
-          }
-        }
-        launch_ks(X, s, KC_EFACE, DOM_PENCIL_X, euler_pencil_smem<T>(), kb_euler_pencil<T, 0>);
+    size_t xs = 0;
+    if constexpr (!euler_streams<T>()) xs = X.x_stage ? euler_x_stage_bytes(X, X.cfg[KC_EFACE].block) : 0;
+    if (xs > 0) {
+      if constexpr (!euler_streams<T>()) {
+        launch_dirs(X, st, KC_EFACE, DOM_PENCILS, 0, 1, xs, kb_euler_x_staged<T>);
+        launch_dirs(X, st, KC_EFACE, DOM_PENCILS, 1, 3, 0, kb_euler_pencil<T>);
       }
-      if (d == 1) launch_ks(X, s, KC_EFACE, DOM_PENCIL_Y, euler_pencil_smem<T>(), kb_euler_pencil<T, 1>);
-      if (d == 2) launch_ks(X, s, KC_EFACE, DOM_PENCIL_Z, euler_pencil_smem<T>(), kb_euler_pencil<T, 2>);
-    });
+    } else {
+      launch_ks(X, st, KC_EFACE, DOM_PENCILS, euler_pencil_smem<T>(), kb_euler_pencil<T>);
+    }
     launch_k(X, st, KC_EDGES, DOM_LATTICE, kb_edges<T>);
     if (grav)
       launch_k(X, st, KC_EUPD, DOM_CELLS, kb_euler_update<T, true>, r);
@@ -399,31 +382,13 @@ template <typename T>
 void launch_lag_stage(Exec<T>& X, cudaStream_t st, bool fuse_last) {
   NvtxRange range("Lagrangian stage (Sec. 2.6)");
   for (int r = 0; r < 3; ++r) {
-    launch_sweeps(X, st, [&](int d, cudaStream_t s) {
-      if constexpr (lag_in_pencils<T>()) {
-        const int dom = DOM_PENCIL_X + d;
-        if (X.ions) {
-          if (d == 0) launch_k(X, s, KC_LFACE, dom, kb_lag_pencil<T, 0, true>);
-          if (d == 1) launch_k(X, s, KC_LFACE, dom, kb_lag_pencil<T, 1, true>);
-          if (d == 2) launch_k(X, s, KC_LFACE, dom, kb_lag_pencil<T, 2, true>);
-        } else {
-          if (d == 0) launch_k(X, s, KC_LFACE, dom, kb_lag_pencil<T, 0, false>);
-          if (d == 1) launch_k(X, s, KC_LFACE, dom, kb_lag_pencil<T, 1, false>);
-          if (d == 2) launch_k(X, s, KC_LFACE, dom, kb_lag_pencil<T, 2, false>);
-        }
-      } else {
-        const int dom = DOM_FACE_X + d;
-        if (X.ions) {
-          if (d == 0) launch_k(X, s, KC_LFACE, dom, kb_lag_face<T, 0, true>);
-          if (d == 1) launch_k(X, s, KC_LFACE, dom, kb_lag_face<T, 1, true>);
-          if (d == 2) launch_k(X, s, KC_LFACE, dom, kb_lag_face<T, 2, true>);
-        } else {
-          if (d == 0) launch_k(X, s, KC_LFACE, dom, kb_lag_face<T, 0, false>);
-          if (d == 1) launch_k(X, s, KC_LFACE, dom, kb_lag_face<T, 1, false>);
-          if (d == 2) launch_k(X, s, KC_LFACE, dom, kb_lag_face<T, 2, false>);
-        }
-      }
-    });
+    if constexpr (lag_in_pencils<T>()) {
+      if (X.ions) launch_k(X, st, KC_LFACE, DOM_PENCILS, kb_lag_pencil<T, true>);
+      else launch_k(X, st, KC_LFACE, DOM_PENCILS, kb_lag_pencil<T, false>);
+    } else {
+      if (X.ions) launch_k(X, st, KC_LFACE, DOM_FACES, kb_lag_face<T, true>);
+      else launch_k(X, st, KC_LFACE, DOM_FACES, kb_lag_face<T, false>);
+    }
     if (r == 2 && fuse_last) break;
     if (X.ions)
       launch_k(X, st, KC_LUPD, DOM_CELLS, kb_lag_update<T, true>, r);
