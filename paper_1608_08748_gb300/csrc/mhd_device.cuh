@@ -474,29 +474,35 @@ struct Dev {
 // D-, s0 = q_{+1} - q_{-1} and the two neighbours' values.  Step 4's eta = -(D+ - D-)/(3 s0) acts where
 // |s0| > min(|q_{+1}|, |q_{-1}|)/100 (the smaller of the paper's three values is one of the two) and
 // D+ D- <= 0; hbar = 20 (eta - 1/20) = (20/3)(D- - D+)/s0 - 1, clamped to [0, 1].
-__device__ __forceinline__ Dev<double> dev_limit(double A, double B, double h0, double Dp, double Dm, double s0,
-                                                 double qp1, double qm1) {
+// In FP64: Step 2 by comparisons of magnitudes on the integer pipe (where the signs agree neither is 0).
+__device__ __forceinline__ Dev<double> dev_monotone(double A, double B) {
   const bool mono = same_sign(A, B);
-  // comparisons of magnitudes on the integer pipe; where mono holds neither is zero
   const double aA = abs_b(A), aB = abs_b(B), A2 = twice_b(A), B2 = twice_b(B);
   const bool up = gt_nn(aA, abs_b(B2)), dn = gt_nn(aB, abs_b(A2));
-  A = mono ? (up ? B2 : A) : 0.0;
-  B = mono ? (dn ? A2 : B) : 0.0;
-  const double as0 = abs_b(s0);
-  if (gt_nn(as0, mul_t(0.01, min_nn(abs_b(qp1), abs_b(qm1)))) && !same_sign(Dp, Dm)) {
-    const double num = sub_t(Dm, Dp);
-    const double num_s = sign_bit_b(s0) ? neg_b(num) : num;
-    // eta > 1/20 as num sgn(s0) > 3 |s0| / 20 (hbar is continuous there, so the test's rounding cannot
-    // move the result); below it hbar = 0 and the division is not taken
-    if (gt_nn(num_s, mul_t(0.15, as0))) {
-      double hb = fma(mul_t(20.0 / 3.0, num), rcp_nr(s0), -1.0);
-      hb = min_nn(hb, 1.0);
-      hb = sign_bit_b(hb) ? 0.0 : hb;  // negative only by rounding
-      A = fma(hb, sub_t(h0, A), A);
-      B = fma(hb, sub_t(h0, B), B);
-    }
-  }
-  return Dev<double>{A, B};
+  return Dev<double>{mono ? (up ? B2 : A) : 0.0, mono ? (dn ? A2 : B) : 0.0};
+}
+// Whether Step 4 may act (num = D- - D+, mn = min(|q_{+1}|, |q_{-1}|)): D+ D- <= 0 exactly, and hbar > 0,
+// |s0| > mn / 100 on the high words, which are e + f for 2^e (1 + f) and lie at most 0.0861 below the
+// base-2 logarithm: hbar > 0 is log2 |num| > log2 |s0| - 2.7370 with the sign of s0, |s0| > mn / 100 is
+// log2 |s0| > log2 mn - 6.6439.  It never misses a cell where Step 4 acts; step4 makes the exact test.
+__device__ __forceinline__ bool step4_candidate(double Dp, double Dm, double num, double s0, double mn) {
+  const int hn = hi_of(abs_b(num)), hs = hi_of(abs_b(s0));
+  return same_sign(num, s0) && !same_sign(Dp, Dm) && hn > hs - (int)(2.83 * (1 << 20)) &&
+         hs > hi_of(mn) - (int)(6.74 * (1 << 20));
+}
+// Step 4's blend.  hbar = 20 eta - 1 is continuous where it crosses 0 and 1, so the clamps' rounding
+// cannot move the result.
+__device__ __forceinline__ Dev<double> step4(Dev<double> P, double h0, double num, double s0, double mn) {
+  double hb = fma(mul_t(in_register(20.0 / 3.0), num), rcp_nr(s0), -in_register(1.0));
+  hb = min_nn(hb, 1.0);
+  if (sign_bit_b(hb) || !gt_nn(abs_b(s0), mul_t(in_register(0.01), mn))) hb = 0.0;
+  return Dev<double>{fma(hb, sub_t(h0, P.A), P.A), fma(hb, sub_t(h0, P.B), P.B)};
+}
+__device__ __forceinline__ Dev<double> dev_limit(double A, double B, double h0, double Dp, double Dm, double s0,
+                                                 double qp1, double qm1) {
+  const Dev<double> P = dev_monotone(A, B);
+  const double num = sub_t(Dm, Dp), mn = min_nn(abs_b(qp1), abs_b(qm1));
+  return step4_candidate(Dp, Dm, num, s0, mn) ? step4(P, h0, num, s0, mn) : P;
 }
 // FP32: bound by instruction issue, so selects instead of branches, and the reciprocal is taken
 // everywhere and discarded where the detector is off (s0 may be 0 there); the clamp is the FMA's own
@@ -557,7 +563,10 @@ struct DevStream {
     qp = qd;
     dp = d2;
   }
-  __device__ __forceinline__ Dev<T> next(T qn) {  // qn = q_{j+2}
+  // The unlimited deviations A, B of cell j and what the limits take besides: limit(A, B, h0, Dp, Dm,
+  // s0, q_{j+1}, q_{j-1}).  Moves on to cell j + 1.
+  template <typename F>
+  __device__ __forceinline__ void next(T qn, F limit) {  // qn = q_{j+2}
     if constexpr (sizeof(T) == 4) {
       dp = qp - q0;
       s0 = qp - qm;
@@ -565,7 +574,7 @@ struct DevStream {
     const T d2 = sub_t(qn, qp), s1 = sub_t(qn, q0);
     const T h1 = half_slope(s1, dp, d2);
     const T C1 = sub_t(d2, dp), t = sub_t(h1, h0);
-    const Dev<T> P = dev_limit(A, fma(-in_register(T(2.0 / 3.0)), t, dp), h0, C1, Cm, s0, qp, qm);
+    limit(A, fma(-in_register(T(2.0 / 3.0)), t, dp), h0, C1, Cm, s0, qp, qm);
     A = fma(in_register(T(2.0 / 3.0)), t, dp);
     qm = q0;
     q0 = qp;
@@ -575,6 +584,10 @@ struct DevStream {
     Cm = C0;
     C0 = C1;
     s0 = s1;
+  }
+  __device__ __forceinline__ Dev<T> next(T qn) {
+    Dev<T> P;
+    next(qn, [&](T a, T b, T h, T Dp, T Dm, T s, T qp1, T qm1) { P = dev_limit(a, b, h, Dp, Dm, s, qp1, qm1); });
     return P;
   }
 };

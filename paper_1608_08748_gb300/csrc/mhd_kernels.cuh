@@ -29,6 +29,11 @@ struct FaceOut {
 };
 
 // ------------------------------------------------------------------------------------------------
+// faces of a pencil and pencils along each axis
+struct Pencils {
+  int len[3], seg[3];
+};
+
 // Batched execution.  Every step kernel walks a table of tiles; a tile is blockDim.x consecutive
 // elements (cells, faces of one direction, or lattice points) of one box, so a warp never spans
 // two boxes.  Grid-stride over tiles: a grid smaller than the tile count makes the launch
@@ -43,8 +48,7 @@ struct Box {
   FaceOut<T> fo[3];  // Eulerian face outputs; the Lagrangian fluxes reuse fo[d].f[0..nv-1]
   T* e[3];
   int nv;            // advected fields of the Lagrangian stage (6; 7 with rho_H2; 8 with rho_H+)
-  int plen;          // faces of a pencil (set by the executor, choose_pencils)
-  int seg[3];        // pencils along each axis
+  Pencils pe, pl;    // the Eulerian and the FP64 Lagrangian pencils (set by the executor, choose_pencils)
   const T* phi;      // gravitational potential of the step (nullptr: no self-gravity)
   int* hflags;       // host-mapped copy of the error flags, written at the end of every step
 };
@@ -58,14 +62,13 @@ constexpr int TILE_DIR_SHIFT = 28;
 
 // domains of the tile tables; those of faces and pencils hold the three directions one after another,
 // so one launch covers the three sweeps of a stage
-enum { DOM_CELLS = 0, DOM_FACES = 1, DOM_LATTICE = 2, DOM_PENCILS = 3, NDOM = 4 };
+enum { DOM_CELLS = 0, DOM_FACES = 1, DOM_LATTICE = 2, DOM_PENCILS = 3, DOM_LAG_PENCILS = 4, NDOM = 5 };
 
 // Faces are solved in pencils of consecutive faces along the sweep direction: the thread carries the
 // stream of the left cell from one face to the next, so every cell's parabolas are built once per
 // direction (plus one extra cell and the stream's priming per pencil).  pencil_len<T>() is the longest
 // pencil: on the 256^3 FP32 step 6 faces measured fastest (4.41 ms of Eulerian faces; 4.83 with 4, 4.55
-// with 8 and with 12), on the 128^3 FP64 one 8.  Small grids take shorter pencils, see
-// choose_pencils.
+// with 8 and with 12), on the 128^3 FP64 one 8.  Smaller grids take shorter pencils, see choose_pencils.
 template <typename T>
 __host__ __device__ constexpr int pencil_len() { return sizeof(T) == 4 ? 6 : 8; }
 
@@ -104,9 +107,9 @@ struct Line {
 // fastest as the cells do.  D is a run-time value, the same for the whole block: one body serves the
 // three sweeps (three instances in one kernel spilled 364 bytes of registers in FP32, against 72).
 template <typename T>
-__device__ __forceinline__ Line line_of_pencil(const Box<T>& B, int D, idx_t p) {
+__device__ __forceinline__ Line line_of_pencil(const Box<T>& B, const Pencils& P, int D, idx_t p) {
   const Geom& g = B.g;
-  const int S = B.seg[D], nx = g.n[0], ny = g.n[1];
+  const int S = P.seg[D], nx = g.n[0], ny = g.n[1];
   int seg, i = 0, j = 0, k = 0;
   if (D == 0) {
     if (sizeof(T) == 8) {
@@ -138,8 +141,8 @@ __device__ __forceinline__ Line line_of_pencil(const Box<T>& B, int D, idx_t p) 
   L.stride = D == 0 ? 1 : D == 1 ? nx : nx * ny;
   L.fbase = (k * (ny + 1) + j) * (nx + 1) + i;
   L.fstride = D == 0 ? 1 : D == 1 ? nx + 1 : (nx + 1) * (ny + 1);
-  L.f0 = seg * B.plen;
-  L.nfp = min(B.plen, L.n + 1 - L.f0);
+  L.f0 = seg * P.len[D];
+  L.nfp = min(P.len[D], L.n + 1 - L.f0);
   return L;
 }
 
@@ -225,43 +228,106 @@ __global__ void __launch_bounds__(512) kb_prim(const Box<T>* __restrict__ boxes,
 }
 
 // ------------------------------------------------------------------------------------------------
-// Eulerian pencils that stream their parabolas (the FP64 path: its bound is FP64 instructions)
-template <typename T>
-__host__ __device__ constexpr bool euler_streams() { return sizeof(T) == 8; }
+// Dynamic shared memory of the FP64 pencils: slots of this thread (slot k at [k blockDim.x +
+// threadIdx.x], so a warp's accesses are consecutive), then a Step 4 ring per warp.
+extern __shared__ __align__(16) unsigned char pencil_smem_raw[];
+__device__ __forceinline__ double& pencil_slot(int k) {
+  return reinterpret_cast<double*>(pencil_smem_raw)[k * blockDim.x + threadIdx.x];
+}
 
-// The FP64 Eulerian pencils keep each primitive's DevStream in this thread's slots of dynamic shared
-// memory between faces (9 values x 6 primitives; value k of primitive v at [(9 v + k) blockDim.x +
-// threadIdx.x], so a warp's accesses are consecutive).
-template <typename T>
-__device__ __forceinline__ T& stream_slot(int v, int k) {
-  extern __shared__ __align__(16) unsigned char stream_smem_raw[];
-  T* sm = reinterpret_cast<T*>(stream_smem_raw);
-  return sm[(9 * v + k) * blockDim.x + threadIdx.x];
+// Step 4 of the FP64 parabolas, gathered over the warp.  Step 4 acts on one parabola in ten or less, but
+// nearly every warp has a lane where it does, so as a branch its 10 FP64 instructions cost almost every
+// parabola as much as its other 7.  The lanes put what it needs in a ring of the warp in shared memory
+// instead, and when 32 have come together (or the results are wanted) the warp does them at once, one
+// per lane.  The deviations wait in slots of the owner's column; a result does not depend on how the ring
+// groups it.  All 32 lanes call push and flush together.  128^3 FP64 step at the developed flow: 20.0 ->
+// 17.2 ms (Eulerian faces 11.9 -> 10.8, Lagrangian 5.9 -> 4.1 ms, there with the FP64 pipe 92 % busy).
+struct Step4Ring {
+  static constexpr int N = 64;  // at most 31 left over and 32 new
+  static constexpr size_t BYTES = N * (4 * sizeof(double) + sizeof(int));
+  double* num;   // num, s0, h0, mn of the items, N each
+  int* who;      // the owner's slot of A; that of B lies `off` further
+  int off;
+  int head = 0, count = 0;
+  __device__ __forceinline__ Step4Ring(int slots, int slots_to_B) : off(slots_to_B * (int)blockDim.x) {
+    unsigned char* base = pencil_smem_raw + (size_t)slots * blockDim.x * sizeof(double) + (threadIdx.x >> 5) * BYTES;
+    num = reinterpret_cast<double*>(base);
+    who = reinterpret_cast<int*>(base + 4 * N * sizeof(double));
+  }
+  __device__ __forceinline__ void process(int n) {
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    if (lane < n) {
+      const int i = (head + lane) & (N - 1);
+      double* ab = reinterpret_cast<double*>(pencil_smem_raw) + who[i];
+      const Dev<double> P = step4(Dev<double>{ab[0], ab[off]}, num[2 * N + i], num[i], num[N + i], num[3 * N + i]);
+      ab[0] = P.A;
+      ab[off] = P.B;
+    }
+    head = (head + n) & (N - 1);
+    count -= n;
+    __syncwarp();
+  }
+  // slot: the slot of A (B is at slot + slots_to_B)
+  __device__ __forceinline__ void push(bool cand, int slot, double num_, double s0, double h0, double mn) {
+    const unsigned m = __ballot_sync(0xffffffffu, cand);
+    if (cand) {
+      const int i = (head + count + __popc(m & ((1u << (threadIdx.x & 31)) - 1))) & (N - 1);
+      num[i] = num_;
+      num[N + i] = s0;
+      num[2 * N + i] = h0;
+      num[3 * N + i] = mn;
+      who[i] = slot * blockDim.x + threadIdx.x;
+    }
+    count += __popc(m);
+    if (count >= 32) process(32);
+  }
+  __device__ __forceinline__ void flush() {
+    if (count > 0) process(count);
+  }
+};
+// shared memory of a block with the given slots per thread and a ring per warp
+constexpr size_t pencil_smem_bytes(int slots, int block) {
+  return (size_t)slots * block * sizeof(double) + (size_t)(block / 32) * Step4Ring::BYTES;
 }
-template <typename T>
-__device__ __forceinline__ void stream_save(const DevStream<T>& S, int v) {
-  stream_slot<T>(v, 0) = S.qm;
-  stream_slot<T>(v, 1) = S.q0;
-  stream_slot<T>(v, 2) = S.qp;
-  stream_slot<T>(v, 3) = S.dp;
-  stream_slot<T>(v, 4) = S.h0;
-  stream_slot<T>(v, 5) = S.A;
-  stream_slot<T>(v, 6) = S.Cm;
-  stream_slot<T>(v, 7) = S.C0;
-  stream_slot<T>(v, 8) = S.s0;
+// limits of the next cell of a stream (live: this lane has one): Step 2 at once, the deviations into the
+// slots, Step 4 into the ring
+__device__ __forceinline__ void stream_limits(DevStream<double>& S, double qn, bool live, Step4Ring& ring, int slotA,
+                                              int slotB) {
+  S.next(qn, [&](double A, double B, double h0, double Dp, double Dm, double s0, double qp1, double qm1) {
+    const Dev<double> P = dev_monotone(A, B);
+    pencil_slot(slotA) = P.A;
+    pencil_slot(slotB) = P.B;
+    const double num = sub_t(Dm, Dp), mn = min_nn(abs_b(qp1), abs_b(qm1));
+    ring.push(live && step4_candidate(Dp, Dm, num, s0, mn), slotA, num, s0, h0, mn);
+  });
 }
-template <typename T>
-__device__ __forceinline__ DevStream<T> stream_load(int v) {
-  DevStream<T> S;
-  S.qm = stream_slot<T>(v, 0);
-  S.q0 = stream_slot<T>(v, 1);
-  S.qp = stream_slot<T>(v, 2);
-  S.dp = stream_slot<T>(v, 3);
-  S.h0 = stream_slot<T>(v, 4);
-  S.A = stream_slot<T>(v, 5);
-  S.Cm = stream_slot<T>(v, 6);
-  S.C0 = stream_slot<T>(v, 7);
-  S.s0 = stream_slot<T>(v, 8);
+
+// The FP64 Eulerian pencils keep each primitive's DevStream (9 values) in the slots 9 v .. 9 v + 8, and
+// the new cell's deviations in the slots 54 + v (A) and 60 + v (B).
+constexpr int EULER_SLOTS = 9 * 6 + 12;
+__device__ __forceinline__ void stream_save(const DevStream<double>& S, int v) {
+  pencil_slot(9 * v) = S.qm;
+  pencil_slot(9 * v + 1) = S.q0;
+  pencil_slot(9 * v + 2) = S.qp;
+  pencil_slot(9 * v + 3) = S.dp;
+  pencil_slot(9 * v + 4) = S.h0;
+  pencil_slot(9 * v + 5) = S.A;
+  pencil_slot(9 * v + 6) = S.Cm;
+  pencil_slot(9 * v + 7) = S.C0;
+  pencil_slot(9 * v + 8) = S.s0;
+}
+__device__ __forceinline__ DevStream<double> stream_load(int v) {
+  DevStream<double> S;
+  S.qm = pencil_slot(9 * v);
+  S.q0 = pencil_slot(9 * v + 1);
+  S.qp = pencil_slot(9 * v + 2);
+  S.dp = pencil_slot(9 * v + 3);
+  S.h0 = pencil_slot(9 * v + 4);
+  S.A = pencil_slot(9 * v + 5);
+  S.Cm = pencil_slot(9 * v + 6);
+  S.C0 = pencil_slot(9 * v + 7);
+  S.s0 = pencil_slot(9 * v + 8);
   return S;
 }
 
@@ -297,7 +363,7 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, int D, idx_
                                                     int fs = 0) {
   const int D1 = D == 2 ? 0 : D + 1, D2 = D == 0 ? 2 : D - 1;
   const Geom& g = B.g;
-  const Line L = line_of_pencil(B, D, p);
+  const Line L = line_of_pencil(B, B.pe, D, p);
   const int f0 = L.f0, nfp = L.nfp;
   const T tau_h = (T)B.sc->tau_h;
   const bool inside = f0 >= 3 && f0 + nfp + 2 <= L.n;
@@ -385,63 +451,72 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, int D, idx_
 }
 
 // Eulerian faces of direction D (Sec. 2.4): the face i_D - 1/2 lies between cells i_D - 1 and i_D.
-// One thread takes the faces i_D in [s P, min((s+1) P, n_D + 1)), P = plen, of one pencil s (the
+// One thread takes the faces i_D in [s P, min((s+1) P, n_D + 1)), P = pe.len[D], of one pencil s (the
 // other two indices in [0, n)); each cell's parabolas are built once and serve both its faces.
 // Per face: the PPM parabolas of (v_n, v_t1, v_t2, B_t1, B_t2, p) of the two cells, the Riemann
-// solve, and the non-advective fluxes with the two EMF contributions E = B x U (Sec. 2.5).  The
-// FP64 form keeps the streams in shared memory, the FP32 form in registers.
-template <typename T>
-__device__ __forceinline__ void euler_pencil(const Box<T>& B, int D, idx_t p) {
-  if constexpr (!euler_streams<T>()) {
-    euler_pencil_window<T>(B, D, p);
-    return;
-  }
+// solve, and the non-advective fluxes with the two EMF contributions E = B x U (Sec. 2.5).  This is
+// the FP64 form; the FP32 form is euler_pencil_window.  The lanes of a warp go through the pencil
+// together (Step4Ring); live: this lane has a pencil.
+__device__ __forceinline__ void euler_pencil(const Box<double>& B, int D, idx_t p, bool live) {
   const int D1 = D == 2 ? 0 : D + 1, D2 = D == 0 ? 2 : D - 1;
   const Geom& g = B.g;
-  const Line L = line_of_pencil(B, D, p);
-  const int f0 = L.f0, f1 = L.f0 + L.nfp;
-  const T tau_h = (T)B.sc->tau_h;
-  const T* qv[6] = {B.w.v[D], B.w.v[D1], B.w.v[D2], B.w.B[D1], B.w.B[D2], B.w.p};
+  const Line L = line_of_pencil(B, B.pe, D, p);
+  const int f0 = L.f0, nfp = live ? L.nfp : 0;
+  const double tau_h = B.sc->tau_h;
+  const double* qv[6] = {B.w.v[D], B.w.v[D1], B.w.v[D2], B.w.B[D1], B.w.B[D2], B.w.p};
   auto cell_at = [&](int i) { return L.cell(g, i); };
-  FaceSide<T> l, r;  // the face's two cells; l.P carries the previous face's right cell
+  Step4Ring ring(EULER_SLOTS, 6);
   {
-    idx_t cell[5];
+    idx_t cell[4];
 #pragma unroll
-    for (int o = 0; o < 5; ++o) cell[o] = cell_at(f0 - 3 + o);
+    for (int o = 0; o < 4; ++o) cell[o] = cell_at(f0 - 3 + o);
 #pragma unroll
     for (int v = 0; v < 6; ++v) {
-      DevStream<T> S;
+      DevStream<double> S;
       S.prime(qv[v][cell[0]], qv[v][cell[1]], qv[v][cell[2]], qv[v][cell[3]]);
-      l.P[v] = S.next(qv[v][cell[4]]);  // cell f0 - 1
       stream_save(S, v);
     }
   }
-  for (int i = f0; i < f1; ++i) {
-    const idx_t cl = cell_at(i - 1), cr = cell_at(i), cn = cell_at(i + 2);
+  FaceSide<double> l, r;  // the face's two cells; l.P carries the previous face's right cell
+#pragma unroll 1
+  for (int k = -1; k < pencil_len<double>(); ++k) {  // cell f0 + k, then (from k = 0 on) the face on its left
+    const int i = f0 + k;
+    const bool on = k < nfp;
+    if (!__any_sync(0xffffffffu, on)) break;
+    const idx_t cn = cell_at(on ? i + 2 : f0);
 #pragma unroll
     for (int v = 0; v < 6; ++v) {
-      DevStream<T> S = stream_load<T>(v);
-      l.q[v] = S.qm;               // cell i - 1
-      r.P[v] = S.next(qv[v][cn]);  // cell i
-      r.q[v] = S.qm;
+      DevStream<double> S = stream_load(v);
+      l.q[v] = S.qm;  // cell i - 1
+      stream_limits(S, qv[v][cn], on, ring, 54 + v, 60 + v);
+      r.q[v] = S.qm;  // cell i
       stream_save(S, v);
     }
-    l.w[0] = B.s.rho[cl];
-    l.w[1] = l.q[5];
-    l.w[2] = B.w.g[cl];
-    l.w[3] = l.q[3];
-    l.w[4] = l.q[4];
-    l.w[5] = B.w.sr[cl];
-    r.w[0] = B.s.rho[cr];
-    r.w[1] = r.q[5];
-    r.w[2] = B.w.g[cr];
-    r.w[3] = r.q[3];
-    r.w[4] = r.q[4];
-    r.w[5] = B.w.sr[cr];
-    const T Bn = B.s.b[D][cr];
-    T qs[6];
-    riemann(l, r, Bn, tau_h, qs);
-    store_face_fluxes(B.fo[D], L.face(g, i), Bn, qs);
+    ring.flush();
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      r.P[v].A = pencil_slot(54 + v);
+      r.P[v].B = pencil_slot(60 + v);
+    }
+    if (k >= 0 && on) {
+      const idx_t cl = cell_at(i - 1), cr = cell_at(i);
+      l.w[0] = B.s.rho[cl];
+      l.w[1] = l.q[5];
+      l.w[2] = B.w.g[cl];
+      l.w[3] = l.q[3];
+      l.w[4] = l.q[4];
+      l.w[5] = B.w.sr[cl];
+      r.w[0] = B.s.rho[cr];
+      r.w[1] = r.q[5];
+      r.w[2] = B.w.g[cr];
+      r.w[3] = r.q[3];
+      r.w[4] = r.q[4];
+      r.w[5] = B.w.sr[cr];
+      const double Bn = B.s.b[D][cr];
+      double qs[6];
+      riemann(l, r, Bn, tau_h, qs);
+      store_face_fluxes(B.fo[D], L.face(g, i), Bn, qs);
+    }
 #pragma unroll
     for (int v = 0; v < 6; ++v) l.P[v] = r.P[v];
   }
@@ -463,16 +538,15 @@ __device__ __forceinline__ void euler_pencil(const Box<T>& B, int D, idx_t p) {
 // off the SMs.
 template <typename T>
 __global__ void __launch_bounds__(256, 2) kb_euler_x_staged(const Box<T>* __restrict__ boxes, Tiles tl) {
-  extern __shared__ __align__(16) unsigned char stream_smem_raw[];
-  T* rows = reinterpret_cast<T*>(stream_smem_raw + 16);
-  const unsigned bar = smem_u32(stream_smem_raw), rows_s = smem_u32(rows);
+  T* rows = reinterpret_cast<T*>(pencil_smem_raw + 16);
+  const unsigned bar = smem_u32(pencil_smem_raw), rows_s = smem_u32(rows);
   const unsigned cap = dynamic_smem_bytes();
   if (threadIdx.x == 0 && cap >= 16) mbar_init(bar);
   __syncthreads();
   unsigned parity = 0;
   MHD_TILE_LOOP(tl) {
     const Box<T>& B = boxes[tl.box[t_] & ((1 << TILE_DIR_SHIFT) - 1)];
-    const int nx = B.g.n[0], S = B.seg[0];
+    const int nx = B.g.n[0], S = B.pe.seg[0];
     const idx_t total = (idx_t)S * B.g.n[1] * B.g.n[2];
     const idx_t p0 = tl.start[t_], p = p0 + (idx_t)threadIdx.x;
     const idx_t pe = p0 + (idx_t)blockDim.x < total ? p0 + (idx_t)blockDim.x : total;
@@ -517,8 +591,8 @@ __device__ __forceinline__ const Box<T>& box_of_tile(const Box<T>* boxes, int co
   return boxes[code & ((1 << TILE_DIR_SHIFT) - 1)];
 }
 template <typename T>
-__device__ __forceinline__ idx_t pencil_count(const Box<T>& B, int dir) {
-  return (idx_t)(dir == 0 ? B.seg[0] : B.g.n[0]) * (dir == 1 ? B.seg[1] : B.g.n[1]) * (dir == 2 ? B.seg[2] : B.g.n[2]);
+__device__ __forceinline__ idx_t pencil_count(const Box<T>& B, const Pencils& P, int dir) {
+  return (idx_t)(dir == 0 ? P.seg[0] : B.g.n[0]) * (dir == 1 ? P.seg[1] : B.g.n[1]) * (dir == 2 ? P.seg[2] : B.g.n[2]);
 }
 
 template <typename T>
@@ -526,8 +600,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) kb_euler_pencil(c
   MHD_TILE_LOOP(tl) {
     int dir;
     const Box<T>& B = box_of_tile(boxes, tl.box[t_], dir);
-    const idx_t p = tl.start[t_] + (idx_t)threadIdx.x;
-    if (p < pencil_count(B, dir)) euler_pencil<T>(B, dir, p);
+    const idx_t p = tl.start[t_] + (idx_t)threadIdx.x, total = pencil_count(B, B.pe, dir);
+    if constexpr (sizeof(T) == 8)
+      euler_pencil(B, dir, p < total ? p : total - 1, p < total);
+    else if (p < total)
+      euler_pencil_window<T>(B, dir, p);
   }
 }
 
@@ -764,75 +841,86 @@ __global__ void __launch_bounds__(256) kb_lag_face(const Box<T>* __restrict__ bo
   }
 }
 
-// The same fluxes for the faces i_D - 1/2, i_D in [s P, min((s+1) P, n_D + 1)), of one
-// pencil s: the face velocities first, then field by field the parabolas of the pencil's cells in
-// one PPMStream along D, each face taking the average of its upwind cell.
-template <typename T, bool IONS>
-__device__ __forceinline__ void lag_pencil(const Box<T>& B, int D, idx_t p) {
+// The same fluxes in FP64 for the faces i_D - 1/2, i_D in [s P, min((s+1) P, n_D + 1)), P = pl.len[D],
+// of one pencil s: the face velocities first, then field by field the deviations of the pencil's cells in one
+// DevStream along D, Step 4 gathered over the warp (Step4Ring), then each face's average of its upwind
+// cell.  Slots: v_n and the two average coefficients of each face, then A, B and the value of each cell.
+constexpr int LAG_FACES = pencil_len<double>(), LAG_CELLS = LAG_FACES + 1;
+constexpr int LAG_SLOTS = 3 * LAG_FACES + 3 * LAG_CELLS;
+template <bool IONS>
+__device__ __forceinline__ void lag_pencil(const Box<double>& B, int D, idx_t p, bool live) {
   const Geom& g = B.g;
-  const Line L = line_of_pencil(B, D, p);
-  const int f0 = L.f0, nfp = L.nfp;
-  const T tau_h = (T)B.sc->tau_h;
+  const Line L = line_of_pencil(B, B.pl, D, p);
+  const int f0 = L.f0, nfp = live ? L.nfp : 0;
+  const double tau_h = B.sc->tau_h;
   auto cell_at = [&](int i) { return L.cell(g, i); };
+  constexpr int VN = 0, KP = LAG_FACES, KR = 2 * LAG_FACES, CA = 3 * LAG_FACES, CB = CA + LAG_CELLS, CQ = CB + LAG_CELLS;
+  Step4Ring ring(LAG_SLOTS, LAG_CELLS);
   // per face: v_n and the coefficients of the average over the upwind fraction y = |v_n| tau / h,
   // q + p A + r B of the left cell (v_n >= 0) or q - r A - p B of the right cell: with (X, Z) = (A, B)
-  // or (-B, -A) both are q + p X + r Z
-  T vn[pencil_len<T>()];
-  AvgCoef<T> kc[pencil_len<T>()];
-  // v_n = (v_l sqrt(rho_l) + v_r sqrt(rho_r)) / (sqrt(rho_l) + sqrt(rho_r)) from the per-cell
-  // m / sqrt(rho) and rho / sqrt(rho) = sqrt(rho), each formed once and carried to the next face
-  T al, bl;
+  // or (-B, -A) both are q + p X + r Z.  v_n = (v_l sqrt(rho_l) + v_r sqrt(rho_r)) / (sqrt(rho_l) +
+  // sqrt(rho_r)) from the per-cell m / sqrt(rho) and rho / sqrt(rho) = sqrt(rho), each formed once and
+  // carried to the next face
+  double al, bl;
   {
     const idx_t c0 = cell_at(f0 - 1);
-    const T r0 = B.s.rho[c0], is0 = rsqrt_n(r0);
+    const double r0 = B.s.rho[c0], is0 = rsqrt_n(r0);
     al = mul_t(B.s.m[D][c0], is0);
     bl = mul_t(r0, is0);
   }
-#pragma unroll
-  for (int k = 0; k < pencil_len<T>(); ++k) {
-    vn[k] = T(0);
-    kc[k].p = kc[k].r = T(0);
-    if (k < nfp) {
-      const idx_t cr = cell_at(f0 + k);
-      const T rr = B.s.rho[cr], isr = rsqrt_n(rr);
-      const T ar = mul_t(B.s.m[D][cr], isr), br = mul_t(rr, isr);
-      vn[k] = mul_t(add_t(al, ar), rcp_t(add_t(bl, br)));
-      al = ar;
-      bl = br;
-      kc[k] = avg_coef(mul_t(abs_b(vn[k]), tau_h));
-    }
+#pragma unroll 2
+  for (int k = 0; k < nfp; ++k) {
+    const idx_t cr = cell_at(f0 + k);
+    const double rr = B.s.rho[cr], isr = rsqrt_n(rr);
+    const double ar = mul_t(B.s.m[D][cr], isr), br = mul_t(rr, isr);
+    const double vn = mul_t(add_t(al, ar), rcp_t(add_t(bl, br)));
+    al = ar;
+    bl = br;
+    const AvgCoef<double> kc = avg_coef(mul_t(abs_b(vn), tau_h));
+    pencil_slot(VN + k) = vn;
+    pencil_slot(KP + k) = kc.p;
+    pencil_slot(KR + k) = kc.r;
   }
+  __syncwarp();
   const int nv = B.nv;
 #pragma unroll 1
   for (int v = 0; v < nv; ++v) {
-    const T* a = v == 0 ? B.s.rho : v < 4 ? B.s.m[v - 1] : v == 4 ? B.s.E : v == 5 ? B.s.eint
-                 : (IONS && v == 7) ? B.s.rhp : B.s.rh2;
-    T* out = B.fo[D].f[v];
-    DevStream<T> S;
+    const double* a = v == 0 ? B.s.rho : v < 4 ? B.s.m[v - 1] : v == 4 ? B.s.E : v == 5 ? B.s.eint
+                      : (IONS && v == 7) ? B.s.rhp : B.s.rh2;
+    DevStream<double> S;
     S.prime(a[cell_at(f0 - 3)], a[cell_at(f0 - 2)], a[cell_at(f0 - 1)], a[cell_at(f0)]);
-    Dev<T> Pl = S.next(a[cell_at(f0 + 1)]);  // cell f0 - 1
-#pragma unroll
-    for (int k = 0; k < pencil_len<T>(); ++k) {
-      if (k < nfp) {
-        const T ql = S.qm;
-        const Dev<T> Pr = S.next(a[cell_at(f0 + k + 2)]);  // cell f0 + k
-        const bool left = !sign_bit_b(vn[k]);  // v_n = -0: a zero flux either way
-        const T q = left ? ql : S.qm;
-        const T X = left ? Pl.A : neg_b(Pr.B), Z = left ? Pl.B : neg_b(Pr.A);
-        out[L.face(g, f0 + k)] = mul_t(vn[k], fma(kc[k].r, Z, fma(kc[k].p, X, q)));
-        Pl = Pr;
-      }
+    double q1 = a[cell_at(f0 + 1)];  // one cell ahead, so that its latency overlaps the cell before
+#pragma unroll 1
+    for (int c = 0; c < LAG_CELLS; ++c) {  // cell f0 - 1 + c
+      const bool on = c <= nfp && live;
+      if (!__any_sync(0xffffffffu, on)) break;
+      const double qn = q1;
+      q1 = a[cell_at(c < nfp ? f0 + 2 + c : f0)];
+      pencil_slot(CQ + c) = S.q0;
+      stream_limits(S, qn, on, ring, CA + c, CB + c);
     }
+    ring.flush();
+    double* out = B.fo[D].f[v];
+#pragma unroll 2
+    for (int k = 0; k < nfp; ++k) {
+      const double vn = pencil_slot(VN + k);
+      const bool left = !sign_bit_b(vn);  // v_n = -0: a zero flux either way
+      const int c = left ? k : k + 1;
+      const double A = pencil_slot(CA + c), Bv = pencil_slot(CB + c);
+      const double X = left ? A : neg_b(Bv), Z = left ? Bv : neg_b(A);
+      out[L.face(g, f0 + k)] = mul_t(vn, fma(pencil_slot(KR + k), Z, fma(pencil_slot(KP + k), X, pencil_slot(CQ + c))));
+    }
+    __syncwarp();
   }
 }
 
-template <typename T, bool IONS>
-__global__ void __launch_bounds__(256, 1) kb_lag_pencil(const Box<T>* __restrict__ boxes, Tiles tl) {
+template <bool IONS>
+__global__ void __launch_bounds__(256, 1) kb_lag_pencil(const Box<double>* __restrict__ boxes, Tiles tl) {
   MHD_TILE_LOOP(tl) {
     int dir;
-    const Box<T>& B = box_of_tile(boxes, tl.box[t_], dir);
-    const idx_t p = tl.start[t_] + (idx_t)threadIdx.x;
-    if (p < pencil_count(B, dir)) lag_pencil<T, IONS>(B, dir, p);
+    const Box<double>& B = box_of_tile(boxes, tl.box[t_], dir);
+    const idx_t p = tl.start[t_] + (idx_t)threadIdx.x, total = pencil_count(B, B.pl, dir);
+    lag_pencil<IONS>(B, dir, p < total ? p : total - 1, p < total);
   }
 }
 

@@ -63,13 +63,9 @@ inline int report_class(int tag) { return tag >= PROF_KC_BASE ? profile_class(ta
 template <typename T>
 constexpr bool lag_in_pencils() { return sizeof(T) == 8; }
 
-// shared memory per thread of the FP64 Eulerian pencils: six DevStreams
-template <typename T>
-constexpr size_t euler_pencil_smem() { return euler_streams<T>() ? 6 * 9 * sizeof(T) : 0; }
-
 template <typename T>
 inline int class_domain(int kc) {
-  const int lag = lag_in_pencils<T>() ? DOM_PENCILS : DOM_FACES;
+  const int lag = lag_in_pencils<T>() ? DOM_LAG_PENCILS : DOM_FACES;
   const int m[NKC] = {DOM_CELLS, DOM_PENCILS, DOM_LATTICE, DOM_CELLS, lag, DOM_CELLS, DOM_CELLS};
   return m[kc];
 }
@@ -138,7 +134,8 @@ long long domain_size(const Box<T>& B, int dom, int dir) {
   switch (dom) {
     case DOM_CELLS: return g.N;
     case DOM_FACES: e[dir] += 1; break;
-    case DOM_PENCILS: e[dir] = B.seg[dir]; break;
+    case DOM_PENCILS: e[dir] = B.pe.seg[dir]; break;
+    case DOM_LAG_PENCILS: e[dir] = B.pl.seg[dir]; break;
     default: return g.NF;
   }
   return e[0] * e[1] * e[2];
@@ -148,7 +145,7 @@ template <typename T>
 cudaError_t ensure_table(Exec<T>& X, int dom, int block) {
   TileTable& t = X.tab[dom][tile_slot(block)];
   if (t.d) return cudaSuccess;
-  const int ndir = dom == DOM_FACES || dom == DOM_PENCILS ? 3 : 1;
+  const int ndir = dom == DOM_CELLS || dom == DOM_LATTICE ? 1 : 3;
   std::vector<int> bx, st;
   for (int q = 0; q < ndir; ++q) {
     t.first[q] = (int)bx.size();
@@ -234,7 +231,7 @@ size_t euler_x_stage_bytes(const Exec<T>& X, int block) {
   for (int b = 0; b < X.nb; ++b) {
     const int nx = X.h[b].g.n[0];
     if (nx % 4 != 0) return 0;
-    const size_t rows = (size_t)((block - 1) / X.h[b].seg[0] + 2);
+    const size_t rows = (size_t)((block - 1) / X.h[b].pe.seg[0] + 2);
     const size_t need = 16 + rows * 6 * (size_t)nx * sizeof(T);
     m = need > m ? need : m;
   }
@@ -247,36 +244,73 @@ size_t euler_x_stage_bytes(const Exec<T>& X, int block) {
 // of T are (the float launchers live in their own translation unit).
 template <typename T>
 cudaError_t prepare_kernels() {
-  if constexpr (euler_pencil_smem<T>() == 0)
+  if constexpr (sizeof(T) == 4) {
     return cudaFuncSetAttribute(kb_euler_x_staged<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXStageMax);
-  if constexpr (euler_pencil_smem<T>() > 0) {
-    const int bytes = (int)(256 * euler_pencil_smem<T>());
-    return cudaFuncSetAttribute(kb_euler_pencil<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  } else {
+    const int eb = (int)pencil_smem_bytes(EULER_SLOTS, 256), lb = (int)pencil_smem_bytes(LAG_SLOTS, 256);
+    cudaError_t e = cudaFuncSetAttribute(kb_euler_pencil<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, eb);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kb_lag_pencil<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lb);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kb_lag_pencil<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lb);
+    return e;
   }
-  return cudaSuccess;
 }
 
-// The length of the pencils: the longest of 1, 2, 4, ... faces (up to pencil_len<T>()) at which the
-// three sweeps of the boxes still have kPencilWarps warps per SM.  A pencil's own cost (one more cell
-// and the priming of its streams) falls with its length; a grid with fewer warps leaves the pipes idle
-// while each thread walks its pencil alone.  The faces' results do not depend on the length.  Measured
-// with 1 / 2 / 4 / 8 faces, ms per FP64 step: 128x4x4 0.24 / 0.31 / 0.43 / 0.69, 32^3 0.65 / 0.61 / 0.60 / 0.72,
-// 64^3 4.0 / 3.3 / 3.1 / 2.9; with 1 / 2 / 6 / 12 in FP32: 32^3 0.117 / 0.111 / 0.120 / 0.142, 256^3 19.0 / 16.4 /
-// 14.6 / 14.8.  (One launch per direction and pencils of 8 and 12 faces took 0.72 ms for 128x4x4 and
-// 0.154 ms for the FP32 32^3.)
-constexpr int kPencilWarps = 4;
+// The pencils of a face kernel.  A pencil has a cost of its own (one more cell and the priming of its
+// streams, as much as `own` faces), so long ones suit large grids; on a small grid they leave SMs idle
+// while each thread walks its pencil alone, and in between the last round of blocks decides.  The model:
+// of the blocks on the busiest SM every `resident` make a round, a round takes (len + own), and a part
+// of a round with k blocks the share part[k] of it.  Fitted to FP64 steps of 16^3 to 80^3, 128x4x4 and
+// 128x128x4 cells with 1 to 8 faces, it comes within 0.5 % (Eulerian, at worst 4 %) and 0.3 % (Lagrangian, 2 %)
+// of the best length's time on average: 8 faces against the chosen 1 is 0.36 against 0.09 ms of Eulerian faces
+// at 128x4x4, against the chosen 6 0.50 / 0.44 ms at 40^3; 1 against the chosen 7 is 3.8 / 2.8 ms at 80^3.  The
+// faces' results do not depend on it.
+struct PencilModel {
+  int resident;
+  double own, part[4];
+};
+constexpr PencilModel kEulerPencils64 = {2, 0.8, {0.0, 0.9}}, kLagPencils64 = {3, 2.0, {0.0, 0.6, 0.8}},
+                      kEulerPencils32 = {4, 1.5, {0.0, 0.55, 0.7, 0.85}};
+template <typename T>
+Pencils pencils_of(const Box<T>& b, int len) {
+  Pencils P;
+  for (int q = 0; q < 3; ++q) {
+    P.seg[q] = (b.g.n[q] + len) / len;            // of the n + 1 faces of a line
+    P.len[q] = (b.g.n[q] + P.seg[q]) / P.seg[q];  // shared out evenly
+  }
+  return P;
+}
+template <typename T>
+int pencil_length(const Exec<T>& X, int block, const PencilModel& m) {
+  int best = 1;
+  double least = 0.0;
+  for (int len = 1; len <= pencil_len<T>(); ++len) {
+    long long blocks = 0;
+    int longest = 1;
+    for (const Box<T>& b : X.h) {
+      const Pencils P = pencils_of(b, len);
+      for (int q = 0; q < 3; ++q) {
+        blocks += (b.g.N / b.g.n[q] * P.seg[q] + block - 1) / block;
+        longest = longest > P.len[q] ? longest : P.len[q];
+      }
+    }
+    const long long per_sm = (blocks + X.nsm - 1) / X.nsm;
+    const double cost = ((double)(per_sm / m.resident) + m.part[per_sm % m.resident]) * (longest + m.own);
+    if (len == 1 || cost < least) {
+      best = len;
+      least = cost;
+    }
+  }
+  return best;
+}
 template <typename T>
 void choose_pencils(Exec<T>& X) {
-  int plen = pencil_len<T>();
-  for (; plen > 1; plen /= 2) {
-    long long pencils = 0;
-    for (const Box<T>& b : X.h)
-      for (int q = 0; q < 3; ++q) pencils += b.g.N / b.g.n[q] * ((b.g.n[q] + plen) / plen);
-    if (pencils >= 32ll * kPencilWarps * X.nsm) break;
-  }
+  const int le = pencil_length(X, X.cfg[KC_EFACE].block, sizeof(T) == 8 ? kEulerPencils64 : kEulerPencils32);
+  const int ll = sizeof(T) == 8 ? pencil_length(X, X.cfg[KC_LFACE].block, kLagPencils64) : 1;
   for (Box<T>& b : X.h) {
-    b.plen = plen;
-    for (int q = 0; q < 3; ++q) b.seg[q] = (b.g.n[q] + plen) / plen;
+    b.pe = pencils_of(b, le);
+    b.pl = pencils_of(b, ll);
   }
 }
 
@@ -289,10 +323,10 @@ cudaError_t exec_init(Exec<T>& X, const std::vector<Box<T>>& boxes) {
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&X.nsm, cudaDevAttrMultiProcessorCount, dev);
-  choose_pencils(X);
   cudaError_t e = prepare_kernels<T>();
   if (e != cudaSuccess) return e;
   default_cfgs(X);
+  choose_pencils(X);
   e = cudaMalloc(&X.d, sizeof(Box<T>) * (size_t)X.nb);
   if (e != cudaSuccess) return e;
   e = cudaMemcpy(X.d, X.h.data(), sizeof(Box<T>) * (size_t)X.nb, cudaMemcpyHostToDevice);
@@ -315,13 +349,13 @@ void exec_free(Exec<T>& X) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// launchers
+// launchers (slots: those of the FP64 pencils' shared memory)
 template <typename T, typename K, typename... A>
-void launch_ks(Exec<T>& X, cudaStream_t st, int kc, int dom, size_t smem_per_thread, K kernel, A... args) {
+void launch_ks(Exec<T>& X, cudaStream_t st, int kc, int dom, int slots, K kernel, A... args) {
   const LaunchCfg& c = X.cfg[kc];
   Tiles t = tiles_of(X, dom, c.block);
   PScope p(X.prof, st, PROF_KC_BASE + kc);  // the profiler records the kernel class
-  kernel<<<grid_of(t, c, X.nsm), c.block, smem_per_thread * c.block, st>>>(X.d, t, args...);
+  kernel<<<grid_of(t, c, X.nsm), c.block, slots ? pencil_smem_bytes(slots, c.block) : 0, st>>>(X.d, t, args...);
 }
 // the directions q0 .. q1 - 1 of a face table, with the block's dynamic shared memory in bytes
 template <typename T, typename K>
@@ -358,15 +392,13 @@ void launch_euler_stage(Exec<T>& X, cudaStream_t st) {
       launch_k(X, st, KC_PRIM, DOM_CELLS, kb_prim<T, true>);
     else
       launch_k(X, st, KC_PRIM, DOM_CELLS, kb_prim<T, false>);
-    size_t xs = 0;
-    if constexpr (!euler_streams<T>()) xs = X.x_stage ? euler_x_stage_bytes(X, X.cfg[KC_EFACE].block) : 0;
-    if (xs > 0) {
-      if constexpr (!euler_streams<T>()) {
-        launch_dirs(X, st, KC_EFACE, DOM_PENCILS, 0, 1, xs, kb_euler_x_staged<T>);
-        launch_dirs(X, st, KC_EFACE, DOM_PENCILS, 1, 3, 0, kb_euler_pencil<T>);
-      }
+    if constexpr (sizeof(T) == 8) {
+      launch_ks(X, st, KC_EFACE, DOM_PENCILS, EULER_SLOTS, kb_euler_pencil<T>);
+    } else if (const size_t xs = X.x_stage ? euler_x_stage_bytes(X, X.cfg[KC_EFACE].block) : 0) {
+      launch_dirs(X, st, KC_EFACE, DOM_PENCILS, 0, 1, xs, kb_euler_x_staged<T>);
+      launch_dirs(X, st, KC_EFACE, DOM_PENCILS, 1, 3, 0, kb_euler_pencil<T>);
     } else {
-      launch_ks(X, st, KC_EFACE, DOM_PENCILS, euler_pencil_smem<T>(), kb_euler_pencil<T>);
+      launch_k(X, st, KC_EFACE, DOM_PENCILS, kb_euler_pencil<T>);
     }
     launch_k(X, st, KC_EDGES, DOM_LATTICE, kb_edges<T>);
     if (grav)
@@ -383,8 +415,8 @@ void launch_lag_stage(Exec<T>& X, cudaStream_t st, bool fuse_last) {
   NvtxRange range("Lagrangian stage (Sec. 2.6)");
   for (int r = 0; r < 3; ++r) {
     if constexpr (lag_in_pencils<T>()) {
-      if (X.ions) launch_k(X, st, KC_LFACE, DOM_PENCILS, kb_lag_pencil<T, true>);
-      else launch_k(X, st, KC_LFACE, DOM_PENCILS, kb_lag_pencil<T, false>);
+      if (X.ions) launch_ks(X, st, KC_LFACE, DOM_LAG_PENCILS, LAG_SLOTS, kb_lag_pencil<true>);
+      else launch_ks(X, st, KC_LFACE, DOM_LAG_PENCILS, LAG_SLOTS, kb_lag_pencil<false>);
     } else {
       if (X.ions) launch_k(X, st, KC_LFACE, DOM_FACES, kb_lag_face<T, true>);
       else launch_k(X, st, KC_LFACE, DOM_FACES, kb_lag_face<T, false>);
