@@ -374,6 +374,7 @@ int mhd_set_option(mhd_sim* S, int key, double v) {
       if (!(v > 0.0)) return fail(MHD_EINVAL, "Doppler parameter must be > 0");
       S->ph.bdop = v;
       S->ph.ibdop = 1.0 / v;
+      mhd::set_shielding(S->ph);
       break;
     case MHD_OPT_CHEM_XNORM:
       if (!(v > 0.0)) return fail(MHD_EINVAL, "x normaliser must be > 0");

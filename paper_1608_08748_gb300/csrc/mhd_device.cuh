@@ -61,6 +61,7 @@ struct Phys {
   double bdop, xnorm, taud;
   double ibdop, ixnorm;  // 1 / bdop, 1 / xnorm
   double taud_ls, ls_ixnorm;  // taud L_s and L_s / xnorm, L_s the shielding length in cm (set_shielding)
+  float taud_ls_f[2], ls_ixnorm_f[2], ibdop_f[2];  // taud_ls, ls_ixnorm, ibdop as float pairs (set_shielding)
   int heatcool;          // Sec. 2.8 heating/cooling stage on (needs chem)
   double grav_g;         // gravitational constant in code units (0: no self-gravity)
   int ions;              // reactions 5-8 with H+ and electrons on (needs chem)
@@ -70,6 +71,7 @@ struct Phys {
 struct Scalars {
   double cfl, t_end;       // set by the host with a kernel launch (graph-safe)
   double tau, tau_h;       // this step's tau and tau / dx
+  float ts[2];             // tau in seconds as a float pair (the FP32 path's chemistry)
   double t;                // simulated time
   unsigned long long dmax; // bits of max CFL denominator of the current state (positive double)
   unsigned long long vel_branch;
@@ -890,6 +892,13 @@ inline void set_shielding(Phys& ph) {
   const double Ls = (ph.lshield > 0.0 ? ph.lshield : ph.dx) * ChemConst::PC;
   ph.taud_ls = ph.taud * Ls;
   ph.ls_ixnorm = Ls * ph.ixnorm;
+  auto pair = [](double x, float* f) {
+    f[0] = (float)x;
+    f[1] = (float)(x - (double)f[0]);
+  };
+  pair(ph.taud_ls, ph.taud_ls_f);
+  pair(ph.ls_ixnorm, ph.ls_ixnorm_f);
+  pair(ph.ibdop, ph.ibdop_f);
 }
 
 // The App. D formulas in FP64 with few FP64 instructions (the rates agree with a term-by-term
@@ -1007,6 +1016,159 @@ __device__ __forceinline__ ChemOut chem_cell(const Phys& ph, double rho, double 
     out.rhp = nHpn;
   }
   return out;
+}
+
+// ------------------------------------------------------------------------------------------------
+// The H/H2 network in pairs of floats, for the FP32-bulk path (without the ions).  That path stores
+// rho_H2 in 24 bits; evaluated in FP64, its 79 instructions per cell were the bound of the post kernel
+// (an FP64 instruction takes the SM as long as 64 FP32 ones).  A pair h + l with |l| <= ulp(h)/2 carries
+// about 48 bits: products and sums lose under 2^-44, far below the 2^-25 of the final rounding, so the stored
+// rho_H2 is the FP64 evaluation's but for cells within 2^-40 of a rounding boundary
+// (tests/test_chem_pairs_host.py).  256^3 FP32 step: the last Lagrangian update with the post stage 2.81 ->
+// 1.11 ms, now near the HBM bound of its 45 arrays.  The elementary steps are the error-free sums and products of Dekker
+// (Numer. Math. 18, 1971) and Knuth with the FMA for a product's error; they use the rounded operations
+// that the compiler does not contract.
+struct FF {
+  float h, l;
+};
+__device__ __forceinline__ float fadd_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fadd_rn(a, b);
+#else
+  return a + b;
+#endif
+}
+__device__ __forceinline__ FF ff_fast_sum(float a, float b) {  // |a| >= |b| or a = 0
+  const float s = fadd_rn(a, b);
+  return FF{s, fadd_rn(b, -fadd_rn(s, -a))};
+}
+__device__ __forceinline__ FF ff_sum(float a, float b) {
+  const float s = fadd_rn(a, b), t = fadd_rn(s, -a);
+  return FF{s, fadd_rn(fadd_rn(a, -fadd_rn(s, -t)), fadd_rn(b, -t))};
+}
+__device__ __forceinline__ FF ff_add(FF a, FF b) {
+  const FF s = ff_sum(a.h, b.h);
+  return ff_fast_sum(s.h, fadd_rn(s.l, fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ FF ff_add(FF a, float b) {
+  const FF s = ff_sum(a.h, b);
+  return ff_fast_sum(s.h, fadd_rn(s.l, a.l));
+}
+__device__ __forceinline__ FF ff_mul(FF a, FF b) {
+  const float p = fmul_rn(a.h, b.h);
+  return ff_fast_sum(p, fma(a.h, b.l, fma(a.l, b.h, fma(a.h, b.h, -p))));
+}
+__device__ __forceinline__ FF ff_mul(FF a, float b) {
+  const float p = fmul_rn(a.h, b);
+  return ff_fast_sum(p, fma(a.l, b, fma(a.h, b, -p)));
+}
+__device__ __forceinline__ FF ff_neg(FF a) { return FF{-a.h, -a.l}; }
+// 1/x and 1/sqrt(x) by the series of rcp_nr and rsqrt_nr from the float approximations (a few 2^-23)
+__device__ __forceinline__ FF ff_rcp(FF x) {
+  const float r = rcp_t(x.h);
+  const float e = fma(-x.l, r, fma(-x.h, r, 1.0f));
+  return ff_fast_sum(r, fmul_rn(r, fma(e, e, e)));
+}
+__device__ __forceinline__ FF ff_rsqrt(FF x) {
+  const float y = rsqrt_t(x.h), y2 = fmul_rn(y, y), dy2 = fma(y, y, -y2);
+  const float e = fma(-x.l, y2, fma(-x.h, dy2, fma(-x.h, y2, 1.0f)));
+  return ff_fast_sum(y, fmul_rn(y, fmul_rn(e, fma(0.375f, e, 0.5f))));
+}
+// 2^(j/32) in pairs
+struct FFPair {
+  float h, l;
+};
+__device__ const FFPair kExp2Frac32Pairs[32] = {
+    {0x1.000000p+0f, 0x0.0p+0f}, {0x1.059b0ep+0f, -0x1.9d4f52p-25f}, {0x1.0b5586p+0f, 0x1.9f3122p-25f},
+    {0x1.11301ep+0f, -0x1.fdb496p-25f}, {0x1.172b84p+0f, -0x1.c15742p-27f}, {0x1.1d4874p+0f, -0x1.d2e8cap-25f},
+    {0x1.2387a6p+0f, 0x1.ceac48p-25f}, {0x1.29e9e0p+0f, -0x1.5c0424p-25f}, {0x1.306fe0p+0f, 0x1.4636e2p-25f},
+    {0x1.371a74p+0f, -0x1.18aac6p-25f}, {0x1.3dea64p+0f, 0x1.824684p-25f}, {0x1.44e086p+0f, 0x1.8624b4p-30f},
+    {0x1.4bfdaep+0f, -0x1.593abcp-25f}, {0x1.5342b6p+0f, -0x1.2c5610p-25f}, {0x1.5ab07ep+0f, -0x1.5bd5ecp-27f},
+    {0x1.6247ecp+0f, -0x1.f8b550p-25f}, {0x1.6a09e6p+0f, 0x1.9fcef4p-26f}, {0x1.71f75ep+0f, 0x1.1d8beep-25f},
+    {0x1.7a1148p+0f, -0x1.829fd0p-25f}, {0x1.82589ap+0f, -0x1.accc7cp-26f}, {0x1.8ace54p+0f, 0x1.15506ep-27f},
+    {0x1.93737cp+0f, -0x1.e64744p-25f}, {0x1.9c4918p+0f, 0x1.51f848p-27f}, {0x1.a5503cp+0f, -0x1.b83b54p-25f},
+    {0x1.ae89fap+0f, -0x1.a94b14p-26f}, {0x1.b7f770p+0f, -0x1.a09438p-25f}, {0x1.c199bep+0f, -0x1.3d56b2p-27f},
+    {0x1.cb720ep+0f, -0x1.8837ccp-27f}, {0x1.d5818ep+0f, -0x1.822dbcp-27f}, {0x1.dfc974p+0f, -0x1.908c94p-25f},
+    {0x1.ea4afap+0f, 0x1.52486cp-27f}, {0x1.f50766p+0f, -0x1.246eb0p-26f}};
+// e^x for -87 <= x <= 0 (0 below: e^-87 is 1.6e-38), exp_tang's method: k = 32 m + j the integer nearest
+// to 32 x / ln 2, r = x - k ln2/32 with ln2/32 in three parts whose products with |k| < 2^12 are exact in
+// the first two, e^r - 1 = r + r^2/2 + r^3 (1/6 + r/24 + r^2/120) with the first two terms in pairs (the
+// neglected r^6/720 is below 2^-48).
+__device__ __forceinline__ FF ff_exp(FF x) {
+  if (!(x.h >= -87.0f)) return FF{0.0f, 0.0f};
+  const float t = fadd_rn(fmul_rn(x.h, 0x1.715476p+5f), 12582912.0f);
+  const float kf = fadd_rn(t, -12582912.0f);
+  const int k = (int)kf;
+  const float r1 = fma(-kf, 0x1.62ep-6f, x.h);
+  FF r = ff_sum(r1, -fmul_rn(kf, 0x1.0cp-20f));
+  r = ff_fast_sum(r.h, fadd_rn(r.l, fma(-kf, -0x1.05c61p-34f, x.l)));
+  const float hr = fmul_rn(0.5f, r.h), q = fmul_rn(hr, r.h), dq = fma(hr, r.h, -q);
+  const float c = fmul_rn(fmul_rn(fmul_rn(r.h, r.h), r.h), fma(r.h, fma(r.h, 1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f));
+  const FF p0 = ff_fast_sum(r.h, q);
+  const FF p = ff_fast_sum(p0.h, fadd_rn(p0.l, fadd_rn(fma(r.h, r.l, r.l), fadd_rn(dq, c))));
+#ifdef __CUDA_ARCH__
+  const float2 tj = __ldg(reinterpret_cast<const float2*>(kExp2Frac32Pairs) + (k & 31));
+  const FF T = {tj.x, tj.y};
+  const float sc = __int_as_float((127 + (k >> 5)) << 23);  // m >= -126
+#else
+  const FF T = {kExp2Frac32Pairs[k & 31].h, kExp2Frac32Pairs[k & 31].l};
+  const float sc = std::ldexp(1.0f, k >> 5);
+#endif
+  const FF y = ff_mul(T, p);
+  const FF z = ff_add(FF{T.h, 0.0f}, FF{y.h, fadd_rn(y.l, T.l)});
+  return FF{fmul_rn(z.h, sc), fmul_rn(z.l, sc)};
+}
+// the product of a constant's pair with a float or a pair
+#define MHD_FF(c) (FF{(float)(c), (float)((c) - (double)(float)(c))})
+
+// chem_cell<false> in pairs: the same formulas with the rates multiplied by the step's seconds ts, so that
+// the numbers stay within the floats' range (a rate that flushes to zero moves nothing).  false where an
+// input lies outside the range that this holds for (also NaN): the caller takes the FP64 form.
+__device__ __forceinline__ bool chem_cell_pairs(const Phys& ph, const float ts_pair[2], float rho, float eint,
+                                                float rh2, float& rh2_new) {
+  const double P0 = ChemConst::MH * ChemConst::KMS * ChemConst::KMS;
+  const FF ts = {ts_pair[0], ts_pair[1]};
+  const float nH2 = 0.5f * rh2, n = rho;
+  const FF nH = ff_sum(rho, -rh2);
+  const bool ok = rho > 1e-8f && rho < 1e8f && eint > 1e-10f && eint < 1e10f && rh2 >= 0.0f && rh2 <= 2.0f * rho &&
+                  ts.h > 1e-10f && ts.h < 1e20f;
+  if (!ok) return false;
+  const FF num = ff_mul(MHD_FF(2.0 * P0 / ChemConst::KB), eint);
+  const FF den3 = ff_add(ff_mul(nH, 3.0f), ff_mul(FF{nH2, 0.0f}, 5.0f));
+  if (!(den3.h > 1e-8f)) return false;
+  const FF q = ff_rsqrt(ff_mul(num, den3));
+  const FF sT = ff_mul(num, q), dq = ff_mul(den3, q);
+  const FF T = ff_mul(sT, sT), iT = ff_mul(dq, dq);
+  const FF x = ff_mul(FF{ph.ls_ixnorm_f[0], ph.ls_ixnorm_f[1]}, nH2);
+  const FF dust = ff_mul(FF{ph.taud_ls_f[0], ph.taud_ls_f[1]}, ff_add(nH, nH2));
+  if (!(T.h < 1e9f && x.h < 1e15f && iT.h < 1e15f)) return false;
+  // reactions 2 and 3 (their exponentials flush to zero in gas below about 720 K and 830 K)
+  const bool hot2 = T.h > 7390.0f || (T.h == 7390.0f && T.l > 0.0f), hot3 = T.h > 7291.0f || (T.h == 7291.0f && T.l > 0.0f);
+  FF D = {0.0f, 0.0f};
+  if (T.h > 700.0f) {
+    const FF w2 = ff_mul(iT, 6750.0f), w3 = ff_mul(iT, 7500.0f);
+    const FF a2 = hot2 ? ff_mul(iT, -2.93e4f) : ff_neg(ff_mul(w2, w2));
+    const FF a3 = hot3 ? ff_mul(iT, -3.22e4f) : ff_neg(ff_add(ff_mul(iT, 4060.0f), ff_mul(w3, w3)));
+    const FF k2 = ff_mul(ff_mul(hot2 ? MHD_FF(6.11e-14) : MHD_FF(2.67e-15), ts), ff_exp(a2));
+    const FF k3 = ff_mul(ff_mul(hot3 ? MHD_FF(5.22e-14) : MHD_FF(3.17e-15), ts), ff_exp(a3));
+    D = ff_add(ff_mul(k2, nH), ff_mul(k3, nH2));
+  }
+  // reaction 4
+  const FF u = ff_add(ff_mul(x, FF{ph.ibdop_f[0], ph.ibdop_f[1]}), 1.0f);
+  const FF x1 = ff_add(x, 1.0f), isx = ff_rsqrt(x1), sx = ff_mul(x1, isx);
+  const FF f1 = ff_mul(MHD_FF(3.3 * 1.7e-11 * 0.965), ff_rcp(ff_mul(u, u)));
+  const FF f2 = ff_mul(ff_mul(MHD_FF(3.3 * 1.7e-11 * 0.035), isx), ff_exp(ff_mul(sx, MHD_FF(-8.5e-4))));
+  const FF k4 = ff_mul(ff_mul(ff_add(f1, f2), ts), ff_exp(ff_neg(dust)));
+  D = ff_add(D, k4);
+  // reaction 1: 3e-17 s / (1 + 0.4 s + 0.2 t + 0.08 t^2), t = T / 100, s = sqrt(t) = sqrt(T) / 10
+  const FF d1 = ff_add(ff_add(ff_mul(ff_add(ff_mul(T, MHD_FF(0.08 * 1e-4)), MHD_FF(0.2 * 1e-2)), T), ff_mul(sT, MHD_FF(0.4 * 0.1))), 1.0f);
+  const FF k1 = ff_mul(ff_mul(ff_mul(MHD_FF(3e-17 * 0.1), ts), sT), ff_rcp(d1));
+  const FF C = ff_mul(ff_mul(k1, n), nH);
+  const FF dn = ff_mul(ff_add(C, ff_neg(ff_mul(D, nH2))), ff_rcp(ff_add(D, 1.0f)));
+  float r = 2.0f * ff_add(dn, nH2).h;
+  r = r < 0.0f ? 0.0f : r;
+  rh2_new = r > n ? n : r;
+  return true;
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -1031,7 +1031,17 @@ __device__ __forceinline__ void post_cell(const Box<T>& B, idx_t c, bool valid, 
     int q[3];
     decode_cell(g, c, q);
     const double tau = B.sc->tau;
-    if ((cell_stages & 1) && ph.chem) {
+    bool fp64_chem = (cell_stages & 1) && ph.chem;
+    if constexpr (sizeof(T) == 4) {
+      if (fp64_chem && !ions) {
+        float r;
+        if (chem_cell_pairs(ph, B.sc->ts, s.rho[c], s.eint[c], s.rh2[c], r)) {
+          s.rh2[c] = r;
+          fp64_chem = false;
+        }
+      }
+    }
+    if (fp64_chem) {
       const ChemOut co = chem_cell<IONS>(ph, (double)s.rho[c], (double)s.eint[c], (double)s.rh2[c],
                                          ions ? (double)s.rhp[c] : 0.0, tau);
       s.rh2[c] = (T)co.rh2;
@@ -1169,6 +1179,9 @@ __global__ void kb_begin_step(const Box<T>* __restrict__ boxes, int nb) {
     sc->tau = tau;
   }
   sc->tau_h = sc->tau / dx;
+  const double ts = sc->tau * (ChemConst::PC / ChemConst::KMS);
+  sc->ts[0] = (float)ts;
+  sc->ts[1] = (float)(ts - (double)sc->ts[0]);
   if (!(sc->tau > 0.0)) sc->flags |= 2;
   sc->dmax = 0ull;  // the post kernel of this step accumulates the next state's denominator
 }

@@ -204,9 +204,9 @@ inline unsigned grid_of(const Tiles& t, const LaunchCfg& c, int nsm) {
 
 // default launch shapes: the face kernels are register heavy (150-230 registers), so 128-thread
 // blocks let two or three blocks share an SM; the rest 256, one block per tile.  The FP32 path's
-// HBM-bound cell kernels (primitives, edge EMFs, the two updates) run grid-stride over their tiles
-// with a few blocks per SM: on the 256^3 box that takes 0.04, 0.11, 0.15 and 0.24 ms per step off
-// one block per tile (measured over 128-512 threads and 2-8 blocks per SM).
+// HBM-bound cell kernels (primitives, edge EMFs, the two updates, the post stage) run grid-stride over
+// their tiles with a few blocks per SM: on the 256^3 box that takes 0.04, 0.11, 0.15, 0.24 and 0.09 ms per
+// step off one block per tile (measured over 64-512 threads and 2-16 blocks per SM).
 template <typename T>
 void default_cfgs(Exec<T>& X) {
   for (int kc = 0; kc < NKC; ++kc) X.cfg[kc] = LaunchCfg{256, 0};
@@ -217,6 +217,7 @@ void default_cfgs(Exec<T>& X) {
     X.cfg[KC_EDGES] = LaunchCfg{512, 4};
     X.cfg[KC_EUPD] = LaunchCfg{128, 8};
     X.cfg[KC_LUPD] = LaunchCfg{128, 8};
+    X.cfg[KC_POST] = LaunchCfg{128, 8};
   }
 }
 
