@@ -447,6 +447,8 @@ int mhd_set_state(mhd_sim* S, const mhd_fields* in) {
     }
   }
   int rc;
+  if ((rc = ensure_exec(S)) != MHD_OK) return rc;
+  if ((rc = reset_scalars(S)) != MHD_OK) return rc;  // before the load, which forms the first CFL maximum
   if (in->dtype == MHD_F64) {
     const double* p[9];
     for (int q = 0; q < 9; ++q) p[q] = (const double*)dev[q];
@@ -456,8 +458,6 @@ int mhd_set_state(mhd_sim* S, const mhd_fields* in) {
     for (int q = 0; q < 9; ++q) p[q] = (const float*)dev[q];
     CK(S->precision ? load_state(S, S->b32, p) : load_state(S, S->b64, p));
   }
-  if ((rc = reset_scalars(S)) != MHD_OK) return rc;
-  if ((rc = refresh_cfl(S)) != MHD_OK) return rc;
   CK(cudaStreamSynchronize(S->stream));
   *(volatile int*)S->hflags_host = 0;  // the steps before this load are finished
   S->has_state = true;

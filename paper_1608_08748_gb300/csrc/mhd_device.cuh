@@ -74,6 +74,7 @@ struct Scalars {
   float ts[2];             // tau in seconds as a float pair (the FP32 path's chemistry)
   double t;                // simulated time
   unsigned long long dmax; // bits of max CFL denominator of the current state (positive double)
+  int dlow;                // bits of a lower bound of that maximum (non-negative float), see post_cell
   unsigned long long vel_branch;
   long long steps;
   int flags;               // bit 0: non-physical state, bit 1: tau <= 0
@@ -1131,7 +1132,7 @@ __device__ __forceinline__ bool chem_cell_pairs(const Phys& ph, const float ts_p
   const float nH2 = 0.5f * rh2, n = rho;
   const FF nH = ff_sum(rho, -rh2);
   const bool ok = rho > 1e-8f && rho < 1e8f && eint > 1e-10f && eint < 1e10f && rh2 >= 0.0f && rh2 <= 2.0f * rho &&
-                  ts.h > 1e-10f && ts.h < 1e20f;
+                  (ts.h == 0.0f || ts.h > 1e-10f) && ts.h < 1e20f;
   if (!ok) return false;
   const FF num = ff_mul(MHD_FF(2.0 * P0 / ChemConst::KB), eint);
   const FF den3 = ff_add(ff_mul(nH, 3.0f), ff_mul(FF{nH2, 0.0f}, 5.0f));

@@ -1009,15 +1009,54 @@ __device__ __forceinline__ float warp_max_f(float v) {
   return v;
 }
 
+// The CFL denominator of the new state of one cell for the next tau (Sec. 2.3).  All lanes of the warp
+// call it (candidate marks those with a physical cell): the FP64 denominator is evaluated only where the
+// FP32 screen (cfl_estimate_f32) cannot exclude the cell from the box's maximum; D stays 0 elsewhere.
+//
+// The screen: a finite estimate raised by 2^-12 below a lower bound of the maximum excludes the cell: any
+// finite estimate lowered by 2^-12 (whose cell is evaluated unless it is excluded too), or the FP64
+// maximum reached so far.  The warp's largest goes into the box's dlow before the test, and what the
+// other warps have put there by then comes back, so that the first wave's warps need not each
+// evaluate their own largest cell.
+template <typename T>
+__device__ __forceinline__ void cfl_of_cell(const Phys& ph, Scalars* sc, bool candidate, bool ions, T rho, const T m[3],
+                                            const T Bc[3], T eint, T rh2, T rhp, double& D) {
+  float D32 = 0.0f;  // 0: no candidate
+  if (candidate)
+    D32 = cfl_estimate_f32((float)rho, (float)m[0], (float)m[1], (float)m[2], (float)Bc[0], (float)Bc[1],
+                           (float)Bc[2], (float)eint,
+                           gamma_minus_one_f32(ph.chem, ph.gamma, (float)rho, (float)rh2, (float)rhp));
+  float bound = warp_max_f(D32 <= 3.0e38f ? D32 : 0.0f) * (1.0f - 0x1p-12f);
+  if ((threadIdx.x & 31) == 0) {
+    const int mine = __float_as_int(bound);
+    int low = *(volatile int*)&sc->dlow;
+    if (mine > low) low = max(mine, atomicMax(&sc->dlow, mine));
+    bound = __int_as_float(low);
+  }
+  bound = __shfl_sync(0xffffffffu, bound, 0);
+  bound = fmaxf(bound, __double2float_rd(__longlong_as_double(*(volatile long long*)&sc->dmax)));
+  if (candidate && !(D32 * (1.0f + 0x1p-12f) < bound)) {
+    // FP64 CFL of the new state (FP32 fields widened)
+    double gm = ph.chem ? gamma_eff((double)rho, (double)rh2) : ph.gamma;
+    if (ions) gm = gamma_eff((double)rho, (double)rh2, (double)rhp);
+    D = cfl_denominator((double)rho, (double)m[0], (double)m[1], (double)m[2], (double)Bc[0],
+                        (double)Bc[1], (double)Bc[2], gm * ((gm - 1.0) * (double)eint));
+  }
+}
+// the warp's share of the largest FP64 CFL denominator
+__device__ __forceinline__ void cfl_warp_reduce(Scalars* sc, double D) {
+  if (__any_sync(0xffffffffu, D > 0.0)) {
+    D = warp_max(D);
+    if ((threadIdx.x & 31) == 0) atomicMax(&sc->dmax, (unsigned long long)__double_as_longlong(D));
+  }
+}
+
 // Per cell, after the Lagrangian stage: chemistry (Sec. 2.7, FP64), heating/cooling (Sec. 2.8,
 // FP64, when on), regularisation (Sec. 2.9), the non-physical check, and the CFL denominator of the
 // new state for the next tau (Sec. 2.3).  cell_stages selects the per-cell stages (bit 0
 // chemistry, bit 1 heating/cooling; the full step runs both), do_reg the regularisation;
 // cell_stages = do_reg = 0 computes only the CFL denominator.  All lanes of the warp call it (valid
-// marks those with a cell): the FP64 denominator is evaluated only where the FP32 screen
-// (cfl_estimate_f32) cannot exclude the cell from the maximum, against the largest estimate of the
-// warp and the FP64 maximum the box has reached so far; D stays 0 elsewhere.  Returns the flags via
-// the warp-aggregated atomics of the caller.
+// marks those with a cell).  Returns the flags via the warp-aggregated atomics of the caller.
 template <typename T, bool IONS>
 __device__ __forceinline__ void post_cell(const Box<T>& B, idx_t c, bool valid, int cell_stages,
                                           int do_reg, double& D, int& bad, unsigned& vb) {
@@ -1026,7 +1065,6 @@ __device__ __forceinline__ void post_cell(const Box<T>& B, idx_t c, bool valid, 
   const bool ions = IONS && ph.ions;
   const State<T>& s = B.s;
   T rho = T(0), m[3] = {T(0), T(0), T(0)}, Bc[3] = {T(0), T(0), T(0)}, eint = T(0), rh2 = T(0), rhp = T(0);
-  float D32 = 0.0f;  // 0: no candidate
   if (valid) {
     int q[3];
     decode_cell(g, c, q);
@@ -1095,24 +1133,8 @@ __device__ __forceinline__ void post_cell(const Box<T>& B, idx_t c, bool valid, 
     for (int k = 0; k < 11; ++k)
       if (!isfinite(vals[k])) bad = 1;
     if (!(rho > T(0)) || !(eint > T(0))) bad = 1;
-    if (!bad)
-      D32 = cfl_estimate_f32((float)rho, (float)m[0], (float)m[1], (float)m[2], (float)Bc[0], (float)Bc[1],
-                             (float)Bc[2], (float)eint,
-                             gamma_minus_one_f32(ph.chem, ph.gamma, (float)rho, (float)rh2, (float)rhp));
   }
-  // the screen: a finite estimate raised by 2^-12 below the largest finite estimate of the warp
-  // lowered by 2^-12 (whose cell is evaluated unless it is excluded too), or below the FP64 maximum
-  // reached so far, excludes the cell
-  const float wmax = warp_max_f(D32 <= 3.0e38f ? D32 : 0.0f);
-  const double reached = __longlong_as_double(*(volatile long long*)&B.sc->dmax);
-  const float bound = fmaxf(__double2float_rd(reached), wmax * (1.0f - 0x1p-12f));
-  if (valid && !bad && !(D32 * (1.0f + 0x1p-12f) < bound)) {
-    // FP64 CFL of the new state (FP32 fields widened)
-    double gm = ph.chem ? gamma_eff((double)rho, (double)rh2) : ph.gamma;
-    if (ions) gm = gamma_eff((double)rho, (double)rh2, (double)rhp);
-    D = cfl_denominator((double)rho, (double)m[0], (double)m[1], (double)m[2], (double)Bc[0],
-                        (double)Bc[1], (double)Bc[2], gm * ((gm - 1.0) * (double)eint));
-  }
+  cfl_of_cell(ph, B.sc, valid && !bad, ions, rho, m, Bc, eint, rh2, rhp, D);
 }
 
 // the warp's share of the post stage's box scalars: the largest FP64 CFL denominator, the
@@ -1120,11 +1142,10 @@ __device__ __forceinline__ void post_cell(const Box<T>& B, idx_t c, bool valid, 
 template <typename T>
 __device__ __forceinline__ void post_warp_reduce(const Box<T>& B, double D, int bad, unsigned vb, int check) {
   if (!check) bad = 0;
-  if (__any_sync(0xffffffffu, D > 0.0)) D = warp_max(D);
+  cfl_warp_reduce(B.sc, D);
   int anybad = __any_sync(0xffffffffu, bad);
   unsigned nvb = __popc(__ballot_sync(0xffffffffu, vb));
   if ((threadIdx.x & 31) == 0) {
-    if (D > 0.0) atomicMax(&B.sc->dmax, (unsigned long long)__double_as_longlong(D));
     if (anybad) atomicOr(&B.sc->flags, 1);
     if (nvb) atomicAdd(&B.sc->vel_branch, (unsigned long long)nvb);
   }
@@ -1184,6 +1205,7 @@ __global__ void kb_begin_step(const Box<T>* __restrict__ boxes, int nb) {
   sc->ts[1] = (float)(ts - (double)sc->ts[0]);
   if (!(sc->tau > 0.0)) sc->flags |= 2;
   sc->dmax = 0ull;  // the post kernel of this step accumulates the next state's denominator
+  sc->dlow = 0;
 }
 
 template <typename T>
@@ -1212,38 +1234,79 @@ __global__ void kb_set_params(const Box<T>* __restrict__ boxes, int nb, double c
 template <typename T>
 __global__ void kb_zero_dmax(const Box<T>* __restrict__ boxes, int nb) {
   int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < nb) boxes[b].sc->dmax = 0ull;
+  if (b >= nb) return;
+  boxes[b].sc->dmax = 0ull;
+  boxes[b].sc->dlow = 0;
 }
 
 // ------------------------------------------------------------------------------------------------
 // set_state helpers
+// (a + b) / 2 of two inputs in FP64, rounded to T; of two floats to a float the FP32 sum and halving give
+// the same value
 template <typename T, typename In>
-__global__ void k_load_cells(Geom g, State<T> s, const In* rho, const In* mx, const In* my,
-                             const In* mz, const In* E, const In* rh2) {
-  long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= g.N) return;
-  s.rho[c] = (T)rho[c];
-  s.m[0][c] = (T)mx[c];
-  s.m[1][c] = (T)my[c];
-  s.m[2][c] = (T)mz[c];
-  s.E[c] = (T)E[c];
-  if (s.rh2) s.rh2[c] = rh2 ? (T)rh2[c] : T(0);
-  if (s.rhp) s.rhp[c] = T(0);
+__device__ __forceinline__ T half_sum(In a, In b) {
+  if constexpr (sizeof(T) == 4 && sizeof(In) == 4) return 0.5f * (a + b);
+  else return (T)(0.5 * ((double)a + (double)b));
 }
-
-// A17: face b_d(i_d - 1/2) = (B_d(i_d - 1) + B_d(i_d)) / 2 from cell-centred input (in FP64)
+// The state from cell-centred input in one pass: the cell fields, the faces b_d(i_d - 1/2) = (B_d(i_d - 1) +
+// B_d(i_d)) / 2 (A17), rho eps = rho E - |m|^2 / (2 rho) - |B_cell|^2 / 2 with B_cell from the stored
+// faces, whose upper one is formed again from the input (with an open boundary the upper face of
+// the last cell is its lower one), and the first tau's CFL denominator (the box's scalars are zero).  As
+// five launches (cells, faces, rho eps, the scalars' reset, the CFL pass) mhd_set_state from device memory
+// took 1.27 ms for 256^3 cells of FP32 and 0.068 ms for 32^3, as one 0.41 and 0.044 ms.  (The half sums of
+// floats in FP64 alone cost 0.6 ms: each conversion takes the FP64 pipe as long as an FMA.)
 template <typename T, typename In>
-__global__ void k_faces_from_cells(Geom g, State<T> s, const In* Bx, const In* By, const In* Bz) {
-  long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= g.N) return;
-  int i = (int)(c % g.n[0]);
-  long long r = c / g.n[0];
-  int j = (int)(r % g.n[1]);
-  int k = (int)(r / g.n[1]);
-  const In* B[3] = {Bx, By, Bz};
-  long long lo[3] = {cmap(g, i - 1, j, k), cmap(g, i, j - 1, k), cmap(g, i, j, k - 1)};
+__global__ void __launch_bounds__(256) k_load_state(Geom g, Phys ph, Scalars* sc, State<T> s, const In* rho_,
+                                                    const In* mx, const In* my, const In* mz, const In* E_,
+                                                    const In* Bx, const In* By, const In* Bz, const In* rh2) {
+  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const bool valid = c < g.N;
+  T rho = T(0), m[3] = {T(0), T(0), T(0)}, B[3] = {T(0), T(0), T(0)}, eint = T(0), h2 = T(0);
+  bool bad = false;
+  if (valid) {
+    int q[3];
+    decode_cell(g, (idx_t)c, q);
+    const In* Bi[3] = {Bx, By, Bz};
+    T b[3];
+    m[0] = (T)mx[c];
+    m[1] = (T)my[c];
+    m[2] = (T)mz[c];
+    rho = (T)rho_[c];
+    const T E = (T)E_[c];
+    if (rh2) h2 = (T)rh2[c];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) s.b[d][c] = (T)(0.5 * ((double)B[d][lo[d]] + (double)B[d][c]));
+    for (int d = 0; d < 3; ++d) {
+      int lo[3] = {q[0], q[1], q[2]}, hi[3] = {q[0], q[1], q[2]};
+      lo[d] -= 1;
+      hi[d] += 1;
+      const In Bc = Bi[d][c];
+      b[d] = half_sum<T>(Bi[d][cmap(g, lo[0], lo[1], lo[2])], Bc);
+      const bool last = g.bc[d] != 0 && hi[d] == g.n[d];
+      const T up = last ? b[d] : half_sum<T>(Bc, Bi[d][cmap(g, hi[0], hi[1], hi[2])]);
+      B[d] = T(0.5) * (b[d] + up);
+    }
+    const T kin = T(0.5) * (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) / rho;
+    const T mag = T(0.5) * (B[0] * B[0] + B[1] * B[1] + B[2] * B[2]);
+    eint = E - kin - mag;
+    s.rho[c] = rho;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      s.m[d][c] = m[d];
+      s.b[d][c] = b[d];
+    }
+    s.E[c] = E;
+    s.eint[c] = eint;
+    if (s.rh2) s.rh2[c] = h2;
+    if (s.rhp) s.rhp[c] = T(0);
+    const T vals[10] = {rho, m[0], m[1], m[2], E, eint, ph.chem ? h2 : T(0), b[0], b[1], b[2]};
+#pragma unroll
+    for (int k = 0; k < 10; ++k)
+      if (!isfinite(vals[k])) bad = true;
+    if (!(rho > T(0)) || !(eint > T(0))) bad = true;
+  }
+  double D = 0.0;
+  cfl_of_cell(ph, sc, valid && !bad, ph.chem && ph.ions, rho, m, B, eint, ph.chem ? h2 : T(0), T(0), D);
+  cfl_warp_reduce(sc, D);
 }
 
 template <typename T>

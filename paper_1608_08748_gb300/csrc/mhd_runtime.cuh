@@ -533,9 +533,8 @@ void grav_free(mhd_sim* S);
 template <typename T, typename In>
 cudaError_t load_state(mhd_sim* S, Box<T>& B, const In* const* p) {
   const Geom& g = S->g;
-  k_load_cells<T, In><<<nblk(g.N, 256), 256, 0, S->stream>>>(g, B.s, p[0], p[1], p[2], p[3], p[4], p[8]);
-  k_faces_from_cells<T, In><<<nblk(g.N, 256), 256, 0, S->stream>>>(g, B.s, p[5], p[6], p[7]);
-  k_derive_eint<T><<<nblk(g.N, 256), 256, 0, S->stream>>>(g, B.s);
+  k_load_state<T, In><<<nblk(g.N, 256), 256, 0, S->stream>>>(g, S->ph, S->sc, B.s, p[0], p[1], p[2], p[3], p[4],
+                                                             p[5], p[6], p[7], p[8]);
   return cudaGetLastError();
 }
 
