@@ -146,6 +146,14 @@ __device__ __forceinline__ Line line_of_pencil(const Box<T>& B, const Pencils& P
   return L;
 }
 
+// Programmatic dependent launch: the step's kernels are launched so that a kernel's blocks may take their
+// places while the one before it drains (launch_dep).  Every such kernel first lets the next one come
+// and then waits until the one before it has finished and its writes are visible; as each kernel does so
+// before it reads or writes anything, the order of the memory accesses is that of plain launches.
+__device__ __forceinline__ void dependent_launch_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 #define MHD_TILE_LOOP(tl) for (int t_ = blockIdx.x; t_ < (tl).n; t_ += gridDim.x)
 
 // Bulk asynchronous copies from global into shared memory (the copy engine moves the bytes; the
@@ -220,6 +228,7 @@ __device__ __forceinline__ void prim_cell(const Box<T>& B, idx_t c) {
 
 template <typename T, bool IONS>
 __global__ void __launch_bounds__(512) kb_prim(const Box<T>* __restrict__ boxes, Tiles tl) {
+  dependent_launch_begin();
   MHD_TILE_LOOP(tl) {
     const Box<T>& B = boxes[tl.box[t_]];
     idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
@@ -538,6 +547,7 @@ __device__ __forceinline__ void euler_pencil(const Box<double>& B, int D, idx_t 
 // off the SMs.
 template <typename T>
 __global__ void __launch_bounds__(256, 2) kb_euler_x_staged(const Box<T>* __restrict__ boxes, Tiles tl) {
+  dependent_launch_begin();
   T* rows = reinterpret_cast<T*>(pencil_smem_raw + 16);
   const unsigned bar = smem_u32(pencil_smem_raw), rows_s = smem_u32(rows);
   const unsigned cap = dynamic_smem_bytes();
@@ -597,6 +607,7 @@ __device__ __forceinline__ idx_t pencil_count(const Box<T>& B, const Pencils& P,
 
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) kb_euler_pencil(const Box<T>* __restrict__ boxes, Tiles tl) {
+  dependent_launch_begin();
   MHD_TILE_LOOP(tl) {
     int dir;
     const Box<T>& B = box_of_tile(boxes, tl.box[t_], dir);
@@ -641,6 +652,7 @@ __device__ __forceinline__ void edges_point(const Box<T>& B, idx_t t) {
 
 template <typename T>
 __global__ void __launch_bounds__(512) kb_edges(const Box<T>* __restrict__ boxes, Tiles tl) {
+  dependent_launch_begin();
   MHD_TILE_LOOP(tl) {
     const Box<T>& B = boxes[tl.box[t_]];
     idx_t t = tl.start[t_] + (idx_t)threadIdx.x;
@@ -767,6 +779,7 @@ __device__ __forceinline__ void euler_update_cell(const Box<T>& B, idx_t c, int 
 
 template <typename T, bool GRAV>
 __global__ void __launch_bounds__(512) kb_euler_update(const Box<T>* __restrict__ boxes, Tiles tl, int r) {
+  dependent_launch_begin();
   MHD_TILE_LOOP(tl) {
     const Box<T>& B = boxes[tl.box[t_]];
     idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
@@ -832,6 +845,7 @@ __device__ __forceinline__ void lag_face(const Box<T>& B, int D, idx_t t) {
 
 template <typename T, bool IONS>
 __global__ void __launch_bounds__(256) kb_lag_face(const Box<T>* __restrict__ boxes, Tiles tl) {
+  dependent_launch_begin();
   MHD_TILE_LOOP(tl) {
     int dir;
     const Box<T>& B = box_of_tile(boxes, tl.box[t_], dir);
@@ -916,6 +930,7 @@ __device__ __forceinline__ void lag_pencil(const Box<double>& B, int D, idx_t p,
 
 template <bool IONS>
 __global__ void __launch_bounds__(256, 1) kb_lag_pencil(const Box<double>* __restrict__ boxes, Tiles tl) {
+  dependent_launch_begin();
   MHD_TILE_LOOP(tl) {
     int dir;
     const Box<double>& B = box_of_tile(boxes, tl.box[t_], dir);
@@ -988,6 +1003,7 @@ __device__ __forceinline__ void lag_update_cell(const Box<T>& B, idx_t c, int r)
 
 template <typename T, bool IONS>
 __global__ void __launch_bounds__(512) kb_lag_update(const Box<T>* __restrict__ boxes, Tiles tl, int r) {
+  dependent_launch_begin();
   MHD_TILE_LOOP(tl) {
     const Box<T>& B = boxes[tl.box[t_]];
     idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
@@ -1154,6 +1170,7 @@ __device__ __forceinline__ void post_warp_reduce(const Box<T>& B, double D, int 
 template <typename T, bool IONS>
 __global__ void __launch_bounds__(512) kb_post(const Box<T>* __restrict__ boxes, Tiles tl, int cell_stages,
                                                int do_reg, int check) {
+  dependent_launch_begin();
   MHD_TILE_LOOP(tl) {
     const Box<T>& B = boxes[tl.box[t_]];
     idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
@@ -1172,6 +1189,7 @@ __global__ void __launch_bounds__(512) kb_post(const Box<T>* __restrict__ boxes,
 template <typename T, bool IONS>
 __global__ void __launch_bounds__(512) kb_lag_update_post(const Box<T>* __restrict__ boxes, Tiles tl,
                                                           int cell_stages, int do_reg, int check) {
+  dependent_launch_begin();
   MHD_TILE_LOOP(tl) {
     const Box<T>& B = boxes[tl.box[t_]];
     idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
@@ -1189,6 +1207,7 @@ __global__ void __launch_bounds__(512) kb_lag_update_post(const Box<T>* __restri
 // CFL h / D equals CFL h / max D since rounding is monotone), truncated at t_end (A18).
 template <typename T>
 __global__ void kb_begin_step(const Box<T>* __restrict__ boxes, int nb) {
+  dependent_launch_begin();
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nb) return;
   Scalars* sc = boxes[b].sc;
@@ -1210,6 +1229,7 @@ __global__ void kb_begin_step(const Box<T>* __restrict__ boxes, int nb) {
 
 template <typename T>
 __global__ void kb_end_step(const Box<T>* __restrict__ boxes, int nb) {
+  dependent_launch_begin();
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nb) return;
   Scalars* sc = boxes[b].sc;

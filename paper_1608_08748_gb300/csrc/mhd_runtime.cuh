@@ -350,13 +350,30 @@ void exec_free(Exec<T>& X) {
 }
 
 // ------------------------------------------------------------------------------------------------
+// a launch whose blocks may start while the kernel before it in the stream drains
+// (dependent_launch_begin); in a captured step a programmatic edge.  The small grids' steps are chains of
+// 20 short kernels: 128x4x4 FP64 PDL0 -> PDL1, 32^3 FP32 PDL2 -> PDL3 us per step.
+template <typename... P, typename... A>
+void launch_dep(cudaStream_t st, unsigned grid, unsigned block, size_t smem, void (*kernel)(P...), A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+}
 // launchers (slots: those of the FP64 pencils' shared memory)
 template <typename T, typename K, typename... A>
 void launch_ks(Exec<T>& X, cudaStream_t st, int kc, int dom, int slots, K kernel, A... args) {
   const LaunchCfg& c = X.cfg[kc];
   Tiles t = tiles_of(X, dom, c.block);
   PScope p(X.prof, st, PROF_KC_BASE + kc);  // the profiler records the kernel class
-  kernel<<<grid_of(t, c, X.nsm), c.block, slots ? pencil_smem_bytes(slots, c.block) : 0, st>>>(X.d, t, args...);
+  launch_dep(st, grid_of(t, c, X.nsm), c.block, slots ? pencil_smem_bytes(slots, c.block) : 0, kernel, X.d, t, args...);
 }
 // the directions q0 .. q1 - 1 of a face table, with the block's dynamic shared memory in bytes
 template <typename T, typename K>
@@ -364,7 +381,7 @@ void launch_dirs(Exec<T>& X, cudaStream_t st, int kc, int dom, int q0, int q1, s
   const LaunchCfg& c = X.cfg[kc];
   Tiles t = tiles_of_dirs(X, dom, c.block, q0, q1);
   PScope p(X.prof, st, PROF_KC_BASE + kc);
-  kernel<<<grid_of(t, c, X.nsm), c.block, bytes, st>>>(X.d, t);
+  launch_dep(st, grid_of(t, c, X.nsm), c.block, bytes, kernel, X.d, t);
 }
 template <typename T, typename K, typename... A>
 void launch_k(Exec<T>& X, cudaStream_t st, int kc, int dom, K kernel, A... args) {
@@ -377,8 +394,8 @@ void launch_small(Exec<T>& X, cudaStream_t st, int which, double cfl = 0, double
                   int fixed = 0, double tau = 0) {
   PScope p_(X.prof, st, MHD_K_SMALL);
   unsigned g = nblk(X.nb, 128);
-  if (which == 0) kb_begin_step<T><<<g, 128, 0, st>>>(X.d, X.nb);
-  if (which == 1) kb_end_step<T><<<g, 128, 0, st>>>(X.d, X.nb);
+  if (which == 0) launch_dep(st, g, 128, 0, kb_begin_step<T>, X.d, X.nb);
+  if (which == 1) launch_dep(st, g, 128, 0, kb_end_step<T>, X.d, X.nb);
   if (which == 2) kb_set_params<T><<<g, 128, 0, st>>>(X.d, X.nb, cfl, t_end, fixed, tau);
   if (which == 3) kb_zero_dmax<T><<<g, 128, 0, st>>>(X.d, X.nb);
 }
