@@ -15,6 +15,13 @@
 #include <math.h>
 #include <stdint.h>
 
+// one body per translation unit, whatever the kernel that calls it
+#ifdef __CUDACC__
+#define MHD_NOINLINE __noinline__
+#else
+#define MHD_NOINLINE
+#endif
+
 namespace mhd {
 
 // ------------------------------------------------------------------------------------------------
@@ -323,12 +330,20 @@ __device__ __forceinline__ double in_register(double c) {
 }
 __device__ __forceinline__ float in_register(float c) { return c; }
 
-// Sums and products of the bulk type where no FMA takes both (the face kernels write their FMAs out).
+// Sums and products of the bulk type where no FMA takes both (the kernels write their FMAs out).  The FP32
+// ones are the rounded operations that the compiler does not contract: a kernel has an instance for one
+// box and one for many, and a box's results must not depend on which of them contracts what.
 // In FP64 they are FMAs with 1 or -0 in a register, exact and by the figures above 16 % faster: 128^3
 // FP64 step 19.4 -> 17.9 ms (Eulerian faces 12.8 -> 11.9, Lagrangian 5.6 -> 5.1 ms).
-__device__ __forceinline__ float add_t(float a, float b) { return a + b; }
-__device__ __forceinline__ float sub_t(float a, float b) { return a - b; }
-__device__ __forceinline__ float mul_t(float a, float b) { return a * b; }
+__device__ __forceinline__ float add_t(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fadd_rn(a, b);
+#else
+  return a + b;
+#endif
+}
+__device__ __forceinline__ float sub_t(float a, float b) { return add_t(a, -b); }
+__device__ __forceinline__ float mul_t(float a, float b) { return fmul_rn(a, b); }
 __device__ __forceinline__ double add_t(double a, double b) { return fma(a, in_register(1.0), b); }
 __device__ __forceinline__ double sub_t(double a, double b) { return fma(-b, in_register(1.0), a); }
 __device__ __forceinline__ double mul_t(double a, double b) { return fma(a, b, in_register(-0.0)); }
@@ -810,7 +825,8 @@ __device__ __forceinline__ void riemann(const T wl[6], const T wr[6], T Bn, cons
 // sqrt(rho), so the largest one is that of the axis of the largest |B_d|.  Takes the momenta and
 // gamma p; 1/sqrt(rho) is the one reciprocal: |v| = |m| / rho, b = |B| / sqrt(rho),
 // c = sqrt(gamma p) / sqrt(rho) and c_f + c_s = sqrt(gamma p + B^2 + 2 sqrt(gamma p) |B_d|) / sqrt(rho).
-__device__ __forceinline__ double cfl_denominator(double rho, double mx, double my, double mz,
+// Compiled once (as the chemistry and the heating/cooling are), so that every kernel gets the same bits.
+__device__ MHD_NOINLINE inline double cfl_denominator(double rho, double mx, double my, double mz,
                                                   double Bx, double By, double Bz, double gp) {
   const double irs = rsqrt(rho);
   const double irho = irs * irs;
@@ -866,15 +882,15 @@ __device__ __forceinline__ float gamma_minus_one_f32(bool chem, double gamma, fl
 template <typename T>
 __device__ __forceinline__ T gamma_eff(T rho, T rh2) {
   T nH = rho - rh2, nH2 = T(0.5) * rh2;
-  return (T(5) * nH + T(7) * nH2) * rcp_t(T(3) * nH + T(5) * nH2);
+  return mul_t(fma(T(7), nH2, mul_t(T(5), nH)), rcp_t(fma(T(5), nH2, mul_t(T(3), nH))));
 }
 
 // ... and with H+ and electrons: the monatomic particles n_1 = n_H + n_H+ + n_e replace n_H, with
 // the neutral atoms n_H = rho - rho_H2 - rho_H+ and n_H+ = n_e = rho_H+ (rho_H+ = 0: the form above)
 template <typename T>
 __device__ __forceinline__ T gamma_eff(T rho, T rh2, T rhp) {
-  T n1 = (rho - rh2 - rhp) + T(2) * rhp, nH2 = T(0.5) * rh2;
-  return (T(5) * n1 + T(7) * nH2) * rcp_t(T(3) * n1 + T(5) * nH2);
+  T n1 = fma(T(2), rhp, rho - rh2 - rhp), nH2 = T(0.5) * rh2;
+  return mul_t(fma(T(7), nH2, mul_t(T(5), n1)), rcp_t(fma(T(5), nH2, mul_t(T(3), n1))));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -950,7 +966,7 @@ __device__ __forceinline__ IonRates ion_rates(double lnT) {
 // IONS: the kernel may see boxes with the ions on (ph.ions decides per box); without it the ion
 // code is compiled out and rhp must be 0.
 template <bool IONS>
-__device__ __forceinline__ ChemOut chem_cell(const Phys& ph, double rho, double eint, double rh2,
+__device__ MHD_NOINLINE ChemOut chem_cell(const Phys& ph, double rho, double eint, double rh2,
                                              double rhp, double tau) {
   const double P0 = ChemConst::MH * ChemConst::KMS * ChemConst::KMS;  // code pressure, erg cm^-3
   const double T0 = ChemConst::PC / ChemConst::KMS;                  // code time, s
@@ -1032,13 +1048,7 @@ __device__ __forceinline__ ChemOut chem_cell(const Phys& ph, double rho, double 
 struct FF {
   float h, l;
 };
-__device__ __forceinline__ float fadd_rn(float a, float b) {
-#ifdef __CUDA_ARCH__
-  return __fadd_rn(a, b);
-#else
-  return a + b;
-#endif
-}
+__device__ __forceinline__ float fadd_rn(float a, float b) { return add_t(a, b); }
 __device__ __forceinline__ FF ff_fast_sum(float a, float b) {  // |a| >= |b| or a = 0
   const float s = fadd_rn(a, b);
   return FF{s, fadd_rn(b, -fadd_rn(s, -a))};
@@ -1187,7 +1197,7 @@ __device__ __forceinline__ bool chem_cell_pairs(const Phys& ph, const float ts_p
 //   the change is limited to at most half of rho eps (the explicit step of a cooling time shorter
 //   than tau would drive rho eps negative).
 template <bool IONS>
-__device__ __forceinline__ double heatcool_delta(const Phys& ph, double rho, double eint, double rh2,
+__device__ MHD_NOINLINE double heatcool_delta(const Phys& ph, double rho, double eint, double rh2,
                                                  double rhp, double tau) {
   const double P0 = ChemConst::MH * ChemConst::KMS * ChemConst::KMS;  // erg cm^-3
   const double T0 = ChemConst::PC / ChemConst::KMS;                  // s

@@ -60,6 +60,36 @@ struct Tiles {
 };
 constexpr int TILE_DIR_SHIFT = 28;
 
+// Where a kernel takes its boxes from: a table of boxes and of their tiles, or one box.  A simulation on its
+// own passes its box by value: the descriptor then lies in the kernel's parameter bank, so its 60-odd
+// pointers cost neither loads nor registers, and a tile's place is arithmetic.  Against a table of one
+// box: 256^3 FP32 step 13.0 -> 12.1 ms (Eulerian faces 4.43 -> 4.09, every other kernel but the primitives
+// 3 to 12 % less), 128^3 FP64 16.7 -> 16.5, 32^3 FP32 99 -> 85 us, 128x4x4 FP64 224 -> 214 us.
+template <typename T>
+struct ManyBoxes {
+  const Box<T>* boxes;
+  Tiles tl;
+  __device__ __forceinline__ int count() const { return tl.n; }
+  // the box of tile t, its direction and the tile's first element
+  __device__ __forceinline__ const Box<T>& tile(int t, int& dir, idx_t& start) const {
+    const int code = tl.box[t];
+    dir = code >> TILE_DIR_SHIFT;
+    start = tl.start[t];
+    return boxes[code & ((1 << TILE_DIR_SHIFT) - 1)];
+  }
+};
+template <typename T>
+struct OneBox {
+  Box<T> box;
+  int n, first1, first2;  // tiles, and the first ones of the directions 1 and 2
+  __device__ __forceinline__ int count() const { return n; }
+  __device__ __forceinline__ const Box<T>& tile(int t, int& dir, idx_t& start) const {
+    dir = (t >= first1) + (t >= first2);
+    start = (t - (dir == 0 ? 0 : dir == 1 ? first1 : first2)) * (int)blockDim.x;
+    return box;
+  }
+};
+
 // domains of the tile tables; those of faces and pencils hold the three directions one after another,
 // so one launch covers the three sweeps of a stage
 enum { DOM_CELLS = 0, DOM_FACES = 1, DOM_LATTICE = 2, DOM_PENCILS = 3, DOM_LAG_PENCILS = 4, NDOM = 5 };
@@ -154,7 +184,7 @@ __device__ __forceinline__ void dependent_launch_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-#define MHD_TILE_LOOP(tl) for (int t_ = blockIdx.x; t_ < (tl).n; t_ += gridDim.x)
+#define MHD_TILE_LOOP(src) for (int t_ = blockIdx.x; t_ < (src).count(); t_ += gridDim.x)
 
 // Bulk asynchronous copies from global into shared memory (the copy engine moves the bytes; the
 // issuing thread spends one instruction per copy) completed on an mbarrier.  Both addresses are
@@ -226,12 +256,14 @@ __device__ __forceinline__ void prim_cell(const Box<T>& B, idx_t c) {
   B.w.sr[c] = sqrt_t(rho);
 }
 
-template <typename T, bool IONS>
-__global__ void __launch_bounds__(512) kb_prim(const Box<T>* __restrict__ boxes, Tiles tl) {
+template <typename T, typename SRC, bool IONS>
+__global__ void __launch_bounds__(512) kb_prim(const __grid_constant__ SRC src) {
   dependent_launch_begin();
-  MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
+  MHD_TILE_LOOP(src) {
+    int dir;
+    idx_t c;
+    const Box<T>& B = src.tile(t_, dir, c);
+    c += (idx_t)threadIdx.x;
     if (c < B.g.N) prim_cell<T, IONS>(B, c);
   }
 }
@@ -554,7 +586,7 @@ __global__ void __launch_bounds__(256, 2) kb_euler_x_staged(const Box<T>* __rest
   if (threadIdx.x == 0 && cap >= 16) mbar_init(bar);
   __syncthreads();
   unsigned parity = 0;
-  MHD_TILE_LOOP(tl) {
+  for (int t_ = blockIdx.x; t_ < tl.n; t_ += gridDim.x) {
     const Box<T>& B = boxes[tl.box[t_] & ((1 << TILE_DIR_SHIFT) - 1)];
     const int nx = B.g.n[0], S = B.pe.seg[0];
     const idx_t total = (idx_t)S * B.g.n[1] * B.g.n[2];
@@ -596,22 +628,19 @@ __global__ void __launch_bounds__(256, 2) kb_euler_x_staged(const Box<T>* __rest
 // The three sweeps in one launch: they read the same cells and write separate arrays, so a sweep's
 // last wave overlaps the next sweep's first, and the small grids pay one launch instead of three.
 template <typename T>
-__device__ __forceinline__ const Box<T>& box_of_tile(const Box<T>* boxes, int code, int& dir) {
-  dir = code >> TILE_DIR_SHIFT;
-  return boxes[code & ((1 << TILE_DIR_SHIFT) - 1)];
-}
-template <typename T>
 __device__ __forceinline__ idx_t pencil_count(const Box<T>& B, const Pencils& P, int dir) {
   return (idx_t)(dir == 0 ? P.seg[0] : B.g.n[0]) * (dir == 1 ? P.seg[1] : B.g.n[1]) * (dir == 2 ? P.seg[2] : B.g.n[2]);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) kb_euler_pencil(const Box<T>* __restrict__ boxes, Tiles tl) {
+template <typename T, typename SRC>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) kb_euler_pencil(const __grid_constant__ SRC src) {
   dependent_launch_begin();
-  MHD_TILE_LOOP(tl) {
+  MHD_TILE_LOOP(src) {
     int dir;
-    const Box<T>& B = box_of_tile(boxes, tl.box[t_], dir);
-    const idx_t p = tl.start[t_] + (idx_t)threadIdx.x, total = pencil_count(B, B.pe, dir);
+    idx_t p;
+    const Box<T>& B = src.tile(t_, dir, p);
+    p += (idx_t)threadIdx.x;
+    const idx_t total = pencil_count(B, B.pe, dir);
     if constexpr (sizeof(T) == 8)
       euler_pencil(B, dir, p < total ? p : total - 1, p < total);
     else if (p < total)
@@ -650,12 +679,14 @@ __device__ __forceinline__ void edges_point(const Box<T>& B, idx_t t) {
     if (c[d] < g.n[d]) B.e[d][t] = e[d];
 }
 
-template <typename T>
-__global__ void __launch_bounds__(512) kb_edges(const Box<T>* __restrict__ boxes, Tiles tl) {
+template <typename T, typename SRC>
+__global__ void __launch_bounds__(512) kb_edges(const __grid_constant__ SRC src) {
   dependent_launch_begin();
-  MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    idx_t t = tl.start[t_] + (idx_t)threadIdx.x;
+  MHD_TILE_LOOP(src) {
+    int dir;
+    idx_t t;
+    const Box<T>& B = src.tile(t_, dir, t);
+    t += (idx_t)threadIdx.x;
     if (t < B.g.NF) edges_point(B, t);
   }
 }
@@ -663,14 +694,12 @@ __global__ void __launch_bounds__(512) kb_edges(const Box<T>* __restrict__ boxes
 // SSP-RK3 combination of Sec. 2.2 for one value: a Q^n + b Q + g tau R, with g tau R = gth S for a
 // flux-difference sum S (R = S / h, gth = g tau / h once per thread).  The first substage has
 // a = 0, b = g = 1 and returns Q + gth S; its caller stores Q^n (the stage's start value, the Q it
-// read) in the RK register, which later substages read as q0.  (The FP64 update kernels are bound
-// by the FP64 pipe, so the constants are folded.)
+// read) in the RK register, which later substages read as q0.  (FP64 rounds a Q^n, FP32 b Q: against
+// 64-bit arithmetic as written the other FP64 order is 20 % further off after one step.)
 template <typename T>
-__device__ __forceinline__ T rk_value(T q, T q0, T a, T b, T gthS, int r) {
-  if constexpr (sizeof(T) == 8)
-    return r == 0 ? add_t(q, gthS) : fma(a, q0, fma(b, q, gthS));
-  else
-    return r == 0 ? q + gthS : (a * q0 + b * q) + gthS;
+__device__ __forceinline__ T rk_value(T q, T q0, T a, T b, T gth, T S, int r) {
+  if constexpr (sizeof(T) == 8) return fma(gth, S, r == 0 ? q : fma(b, q, mul_t(a, q0)));
+  else return fma(gth, S, r == 0 ? q : fma(a, q0, mul_t(b, q)));
 }
 
 // The cell kernels (primitives, edge EMFs, and the two updates in FP32) issue every load of a cell
@@ -725,9 +754,9 @@ __device__ __forceinline__ void euler_update_cell(const Box<T>& B, idx_t c, int 
     const T rho = B.s.rho[c];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const T gd = -(B.phi[upc[d]] - B.phi[dn[d]]) * T(0.5);  // h (-d Phi / dx_d)
-      Rv[d] = Rv[d] + rho * gd;
-      Rv[3] = Rv[3] + B.s.m[d][c] * gd;
+      const T gd = mul_t(sub_t(B.phi[dn[d]], B.phi[upc[d]]), T(0.5));  // h (-d Phi / dx_d)
+      Rv[d] = fma(rho, gd, Rv[d]);
+      Rv[3] = fma(B.s.m[d][c], gd, Rv[3]);
     }
   }
   T* qq[5] = {B.s.m[0], B.s.m[1], B.s.m[2], B.s.E, B.s.eint};
@@ -753,36 +782,38 @@ __device__ __forceinline__ void euler_update_cell(const Box<T>& B, idx_t c, int 
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       if (r == 0) q0[v][c] = qv[v];
-      qq[v][c] = rk_value(qv[v], q0v[v], a, bb, mul_t(gth, Rv[v]), r);
+      qq[v][c] = rk_value(qv[v], q0v[v], a, bb, gth, Rv[v], r);
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       if (r == 0) B.s0.b[d][c] = bv[d];
-      B.s.b[d][c] = rk_value(bv[d], b0v[d], a, bb, mul_t(gth, curl[d]), r);
+      B.s.b[d][c] = rk_value(bv[d], b0v[d], a, bb, gth, curl[d], r);
     }
   } else {
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const T qv = qq[v][c], q0v = r ? q0[v][c] : T(0);
       if (r == 0) q0[v][c] = qv;
-      qq[v][c] = rk_value(qv, q0v, a, bb, mul_t(gth, Rv[v]), r);
+      qq[v][c] = rk_value(qv, q0v, a, bb, gth, Rv[v], r);
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const T curl = curl_of(d);
       const T bv = B.s.b[d][c], b0v = r ? B.s0.b[d][c] : T(0);
       if (r == 0) B.s0.b[d][c] = bv;
-      B.s.b[d][c] = rk_value(bv, b0v, a, bb, mul_t(gth, curl), r);
+      B.s.b[d][c] = rk_value(bv, b0v, a, bb, gth, curl, r);
     }
   }
 }
 
-template <typename T, bool GRAV>
-__global__ void __launch_bounds__(512) kb_euler_update(const Box<T>* __restrict__ boxes, Tiles tl, int r) {
+template <typename T, typename SRC, bool GRAV>
+__global__ void __launch_bounds__(512) kb_euler_update(const __grid_constant__ SRC src, int r) {
   dependent_launch_begin();
-  MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
+  MHD_TILE_LOOP(src) {
+    int dir;
+    idx_t c;
+    const Box<T>& B = src.tile(t_, dir, c);
+    c += (idx_t)threadIdx.x;
     if (c < B.g.N) euler_update_cell<T, GRAV>(B, c, r);
   }
 }
@@ -816,8 +847,8 @@ __device__ __forceinline__ void lag_face(const Box<T>& B, int D, idx_t t) {
   // v_l sqrt(rho_l) = m_l / sqrt(rho_l) and sqrt(rho) = rho / sqrt(rho): two 1/sqrt and a division
   T rl = B.s.rho[cl], rr = B.s.rho[cr];
   T isl = rsqrt_t(rl), isr = rsqrt_t(rr);
-  T vn = (B.s.m[D][cl] * isl + B.s.m[D][cr] * isr) * rcp_t(rl * isl + rr * isr);
-  const AvgCoef<T> kc = avg_coef(T(fabs(vn) * tau_h));
+  const T vn = mul_t(fma(B.s.m[D][cr], isr, mul_t(B.s.m[D][cl], isl)), rcp_t(fma(rr, isr, mul_t(rl, isl))));
+  const AvgCoef<T> kc = avg_coef(mul_t(abs_b(vn), tau_h));
   const T* q[7] = {B.s.rho, B.s.m[0], B.s.m[1], B.s.m[2], B.s.E, B.s.eint, B.s.rh2};
   const idx_t f = fidx(g, i, j, k);
   const int o0 = vn >= T(0) ? 0 : 1;  // upwind cell: stencil cells o0 .. o0 + 4
@@ -843,13 +874,14 @@ __device__ __forceinline__ void lag_face(const Box<T>& B, int D, idx_t t) {
   }
 }
 
-template <typename T, bool IONS>
-__global__ void __launch_bounds__(256) kb_lag_face(const Box<T>* __restrict__ boxes, Tiles tl) {
+template <typename T, typename SRC, bool IONS>
+__global__ void __launch_bounds__(256) kb_lag_face(const __grid_constant__ SRC src) {
   dependent_launch_begin();
-  MHD_TILE_LOOP(tl) {
+  MHD_TILE_LOOP(src) {
     int dir;
-    const Box<T>& B = box_of_tile(boxes, tl.box[t_], dir);
-    const idx_t t = tl.start[t_] + (idx_t)threadIdx.x;
+    idx_t t;
+    const Box<T>& B = src.tile(t_, dir, t);
+    t += (idx_t)threadIdx.x;
     if (t < (idx_t)(B.g.n[0] + (dir == 0)) * (B.g.n[1] + (dir == 1)) * (B.g.n[2] + (dir == 2)))
       lag_face<T, IONS>(B, dir, t);
   }
@@ -928,13 +960,15 @@ __device__ __forceinline__ void lag_pencil(const Box<double>& B, int D, idx_t p,
   }
 }
 
-template <bool IONS>
-__global__ void __launch_bounds__(256, 1) kb_lag_pencil(const Box<double>* __restrict__ boxes, Tiles tl) {
+template <typename T, typename SRC, bool IONS>
+__global__ void __launch_bounds__(256, 1) kb_lag_pencil(const __grid_constant__ SRC src) {
   dependent_launch_begin();
-  MHD_TILE_LOOP(tl) {
+  MHD_TILE_LOOP(src) {
     int dir;
-    const Box<double>& B = box_of_tile(boxes, tl.box[t_], dir);
-    const idx_t p = tl.start[t_] + (idx_t)threadIdx.x, total = pencil_count(B, B.pl, dir);
+    idx_t p;
+    const Box<double>& B = src.tile(t_, dir, p);
+    p += (idx_t)threadIdx.x;
+    const idx_t total = pencil_count(B, B.pl, dir);
     lag_pencil<IONS>(B, dir, p < total ? p : total - 1, p < total);
   }
 }
@@ -984,7 +1018,7 @@ __device__ __forceinline__ void lag_update_cell(const Box<T>& B, idx_t c, int r)
         const int v = h * H + i;
         if (v < NV && v < nv) {
           if (r == 0) q0[v][c] = qv[i];
-          qq[v][c] = rk_value(qv[i], q0v[i], a, bb, mul_t(gth, acc[i]), r);
+          qq[v][c] = rk_value(qv[i], q0v[i], a, bb, gth, acc[i], r);
         }
       }
     }
@@ -996,17 +1030,19 @@ __device__ __forceinline__ void lag_update_cell(const Box<T>& B, idx_t c, int r)
       const T acc = sum_of(v);
       const T qv = qq[v][c], q0v = r ? q0[v][c] : T(0);
       if (r == 0) q0[v][c] = qv;
-      qq[v][c] = rk_value(qv, q0v, a, bb, mul_t(gth, acc), r);
+      qq[v][c] = rk_value(qv, q0v, a, bb, gth, acc, r);
     }
   }
 }
 
-template <typename T, bool IONS>
-__global__ void __launch_bounds__(512) kb_lag_update(const Box<T>* __restrict__ boxes, Tiles tl, int r) {
+template <typename T, typename SRC, bool IONS>
+__global__ void __launch_bounds__(512) kb_lag_update(const __grid_constant__ SRC src, int r) {
   dependent_launch_begin();
-  MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
+  MHD_TILE_LOOP(src) {
+    int dir;
+    idx_t c;
+    const Box<T>& B = src.tile(t_, dir, c);
+    c += (idx_t)threadIdx.x;
     if (c < B.g.N) lag_update_cell<T, IONS>(B, c, r);
   }
 }
@@ -1110,24 +1146,24 @@ __device__ __forceinline__ void post_cell(const Box<T>& B, idx_t c, bool valid, 
     idx_t up[3] = {cmap(g, q[0] + 1, q[1], q[2]), cmap(g, q[0], q[1] + 1, q[2]),
                    cmap(g, q[0], q[1], q[2] + 1)};
 #pragma unroll
-    for (int d = 0; d < 3; ++d) Bc[d] = T(0.5) * (s.b[d][c] + s.b[d][up[d]]);
+    for (int d = 0; d < 3; ++d) Bc[d] = mul_t(T(0.5), add_t(s.b[d][c], s.b[d][up[d]]));
     rho = s.rho[c];
 #pragma unroll
     for (int d = 0; d < 3; ++d) m[d] = s.m[d][c];
     T E = s.E[c];
     eint = s.eint[c];
     if (do_reg) {
-      T m2 = m[0] * m[0] + m[1] * m[1] + m[2] * m[2];
-      T kin = T(0.5) * m2 / rho;
-      T mag = T(0.5) * (Bc[0] * Bc[0] + Bc[1] * Bc[1] + Bc[2] * Bc[2]);
-      T e = E - kin - mag;
+      const T m2 = fma(m[2], m[2], fma(m[1], m[1], mul_t(m[0], m[0])));
+      const T kin = mul_t(T(0.5), m2) / rho;
+      const T mag = mul_t(T(0.5), fma(Bc[2], Bc[2], fma(Bc[1], Bc[1], mul_t(Bc[0], Bc[0]))));
+      const T e = sub_t(sub_t(E, kin), mag);
       T f = e / E;
       bool entropy_branch = f >= T(1e-3);
       if (ph.regul_mode == 2) entropy_branch = !entropy_branch;
       if (entropy_branch) {
         if (ph.regul_mode != 0 || e > eint) eint = e;
       } else {
-        T v2 = T(2) * (E - eint - mag) / rho;
+        T v2 = mul_t(T(2), sub_t(sub_t(E, eint), mag)) / rho;
         if (v2 < T(0)) v2 = T(0);
         T vnew = sqrt(v2);
         T vold = sqrt(m2) / rho;
@@ -1167,13 +1203,15 @@ __device__ __forceinline__ void post_warp_reduce(const Box<T>& B, double D, int 
   }
 }
 
-template <typename T, bool IONS>
-__global__ void __launch_bounds__(512) kb_post(const Box<T>* __restrict__ boxes, Tiles tl, int cell_stages,
+template <typename T, typename SRC, bool IONS>
+__global__ void __launch_bounds__(512) kb_post(const __grid_constant__ SRC src, int cell_stages,
                                                int do_reg, int check) {
   dependent_launch_begin();
-  MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
+  MHD_TILE_LOOP(src) {
+    int dir;
+    idx_t c;
+    const Box<T>& B = src.tile(t_, dir, c);
+    c += (idx_t)threadIdx.x;
     double D = 0.0;
     int bad = 0;
     unsigned vb = 0;
@@ -1186,13 +1224,15 @@ __global__ void __launch_bounds__(512) kb_post(const Box<T>* __restrict__ boxes,
 // reads the face fluxes and the cell's own fields, and its post stage reads only the cell's own
 // fields and the face field b, which neither changes; so one thread takes both, in program order,
 // and the update's HBM traffic overlaps the post stage's FP64 work.
-template <typename T, bool IONS>
-__global__ void __launch_bounds__(512) kb_lag_update_post(const Box<T>* __restrict__ boxes, Tiles tl,
+template <typename T, typename SRC, bool IONS>
+__global__ void __launch_bounds__(512) kb_lag_update_post(const __grid_constant__ SRC src,
                                                           int cell_stages, int do_reg, int check) {
   dependent_launch_begin();
-  MHD_TILE_LOOP(tl) {
-    const Box<T>& B = boxes[tl.box[t_]];
-    idx_t c = tl.start[t_] + (idx_t)threadIdx.x;
+  MHD_TILE_LOOP(src) {
+    int dir;
+    idx_t c;
+    const Box<T>& B = src.tile(t_, dir, c);
+    c += (idx_t)threadIdx.x;
     const bool valid = c < B.g.N;
     if (valid) lag_update_cell<T, IONS>(B, c, 2);
     double D = 0.0;

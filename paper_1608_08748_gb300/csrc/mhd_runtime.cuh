@@ -157,7 +157,7 @@ cudaError_t ensure_table(Exec<T>& X, int dom, int block) {
       }
     }
   }
-  for (int q = ndir; q < 4; ++q) t.first[q] = (int)bx.size();
+  for (int q = ndir; q < 4; ++q) t.first[q] = (int)bx.size();  // one direction: the others are empty
   t.n = (int)bx.size();
   if (t.n == 0) return cudaSuccess;
   cudaError_t e = cudaMalloc(&t.d, sizeof(int) * 2 * (size_t)t.n);
@@ -176,15 +176,6 @@ cudaError_t ensure_tables(Exec<T>& X) {
   return cudaSuccess;
 }
 
-template <typename T>
-Tiles tiles_of(const Exec<T>& X, int dom, int block) {
-  const TileTable& t = X.tab[dom][tile_slot(block)];
-  Tiles r;
-  r.box = t.d;
-  r.start = t.d + t.n;
-  r.n = t.n;
-  return r;
-}
 // the tiles of the directions q0 .. q1 - 1 of a face table
 template <typename T>
 Tiles tiles_of_dirs(const Exec<T>& X, int dom, int block, int q0, int q1) {
@@ -249,11 +240,14 @@ cudaError_t prepare_kernels() {
     return cudaFuncSetAttribute(kb_euler_x_staged<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXStageMax);
   } else {
     const int eb = (int)pencil_smem_bytes(EULER_SLOTS, 256), lb = (int)pencil_smem_bytes(LAG_SLOTS, 256);
-    cudaError_t e = cudaFuncSetAttribute(kb_euler_pencil<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, eb);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kb_lag_pencil<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lb);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kb_lag_pencil<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lb);
+    const void* euler[2] = {(const void*)kb_euler_pencil<T, OneBox<T>>, (const void*)kb_euler_pencil<T, ManyBoxes<T>>};
+    const void* lag[4] = {(const void*)kb_lag_pencil<T, OneBox<T>, false>, (const void*)kb_lag_pencil<T, OneBox<T>, true>,
+                          (const void*)kb_lag_pencil<T, ManyBoxes<T>, false>, (const void*)kb_lag_pencil<T, ManyBoxes<T>, true>};
+    cudaError_t e = cudaSuccess;
+    for (const void* k : euler)
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, eb);
+    for (const void* k : lag)
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lb);
     return e;
   }
 }
@@ -367,28 +361,28 @@ void launch_dep(cudaStream_t st, unsigned grid, unsigned block, size_t smem, voi
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, (P)args...);
 }
-// launchers (slots: those of the FP64 pencils' shared memory)
-template <typename T, typename K, typename... A>
-void launch_ks(Exec<T>& X, cudaStream_t st, int kc, int dom, int slots, K kernel, A... args) {
+// a kernel's two instances, for one box and for many
+#define MHD_BOTH(kernel, ...) kernel<T, OneBox<T>, ##__VA_ARGS__>, kernel<T, ManyBoxes<T>, ##__VA_ARGS__>
+// launch of the tiles of a domain (directions q0 .. q1 - 1 of the face tables; bytes: dynamic shared memory)
+template <typename T, typename K1, typename KN, typename... A>
+void launch_dirs(Exec<T>& X, cudaStream_t st, int kc, int dom, int q0, int q1, size_t bytes, K1 one, KN many, A... args) {
   const LaunchCfg& c = X.cfg[kc];
-  Tiles t = tiles_of(X, dom, c.block);
+  const TileTable& t = X.tab[dom][tile_slot(c.block)];
+  const Tiles tl = tiles_of_dirs(X, dom, c.block, q0, q1);
+  const unsigned grid = grid_of(tl, c, X.nsm);
   PScope p(X.prof, st, PROF_KC_BASE + kc);  // the profiler records the kernel class
-  launch_dep(st, grid_of(t, c, X.nsm), c.block, slots ? pencil_smem_bytes(slots, c.block) : 0, kernel, X.d, t, args...);
+  if (X.nb == 1 && q0 == 0) {
+    OneBox<T> src{X.h[0], tl.n, t.first[1], t.first[2]};
+    launch_dep(st, grid, c.block, bytes, one, src, args...);
+  } else {
+    ManyBoxes<T> src{X.d, tl};
+    launch_dep(st, grid, c.block, bytes, many, src, args...);
+  }
 }
-// the directions q0 .. q1 - 1 of a face table, with the block's dynamic shared memory in bytes
-template <typename T, typename K>
-void launch_dirs(Exec<T>& X, cudaStream_t st, int kc, int dom, int q0, int q1, size_t bytes, K kernel) {
-  const LaunchCfg& c = X.cfg[kc];
-  Tiles t = tiles_of_dirs(X, dom, c.block, q0, q1);
-  PScope p(X.prof, st, PROF_KC_BASE + kc);
-  launch_dep(st, grid_of(t, c, X.nsm), c.block, bytes, kernel, X.d, t);
+template <typename T, typename K1, typename KN, typename... A>
+void launch_k(Exec<T>& X, cudaStream_t st, int kc, int dom, size_t bytes, K1 one, KN many, A... args) {
+  launch_dirs(X, st, kc, dom, 0, 3, bytes, one, many, args...);
 }
-template <typename T, typename K, typename... A>
-void launch_k(Exec<T>& X, cudaStream_t st, int kc, int dom, K kernel, A... args) {
-  launch_ks(X, st, kc, dom, 0, kernel, args...);
-}
-
-
 template <typename T>
 void launch_small(Exec<T>& X, cudaStream_t st, int which, double cfl = 0, double t_end = 0,
                   int fixed = 0, double tau = 0) {
@@ -407,22 +401,27 @@ void launch_euler_stage(Exec<T>& X, cudaStream_t st) {
   const bool grav = X.nb == 1 && X.h[0].phi != nullptr;
   for (int r = 0; r < 3; ++r) {
     if (X.ions)
-      launch_k(X, st, KC_PRIM, DOM_CELLS, kb_prim<T, true>);
+      launch_k(X, st, KC_PRIM, DOM_CELLS, 0, MHD_BOTH(kb_prim, true));
     else
-      launch_k(X, st, KC_PRIM, DOM_CELLS, kb_prim<T, false>);
+      launch_k(X, st, KC_PRIM, DOM_CELLS, 0, MHD_BOTH(kb_prim, false));
     if constexpr (sizeof(T) == 8) {
-      launch_ks(X, st, KC_EFACE, DOM_PENCILS, EULER_SLOTS, kb_euler_pencil<T>);
+      launch_k(X, st, KC_EFACE, DOM_PENCILS, pencil_smem_bytes(EULER_SLOTS, X.cfg[KC_EFACE].block), MHD_BOTH(kb_euler_pencil));
     } else if (const size_t xs = X.x_stage ? euler_x_stage_bytes(X, X.cfg[KC_EFACE].block) : 0) {
-      launch_dirs(X, st, KC_EFACE, DOM_PENCILS, 0, 1, xs, kb_euler_x_staged<T>);
-      launch_dirs(X, st, KC_EFACE, DOM_PENCILS, 1, 3, 0, kb_euler_pencil<T>);
+      {
+        const LaunchCfg& c = X.cfg[KC_EFACE];
+        const Tiles tl = tiles_of_dirs(X, DOM_PENCILS, c.block, 0, 1);
+        PScope p(X.prof, st, PROF_KC_BASE + KC_EFACE);
+        launch_dep(st, grid_of(tl, c, X.nsm), c.block, xs, kb_euler_x_staged<T>, X.d, tl);
+      }
+      launch_dirs(X, st, KC_EFACE, DOM_PENCILS, 1, 3, 0, MHD_BOTH(kb_euler_pencil));
     } else {
-      launch_k(X, st, KC_EFACE, DOM_PENCILS, kb_euler_pencil<T>);
+      launch_k(X, st, KC_EFACE, DOM_PENCILS, 0, MHD_BOTH(kb_euler_pencil));
     }
-    launch_k(X, st, KC_EDGES, DOM_LATTICE, kb_edges<T>);
+    launch_k(X, st, KC_EDGES, DOM_LATTICE, 0, MHD_BOTH(kb_edges));
     if (grav)
-      launch_k(X, st, KC_EUPD, DOM_CELLS, kb_euler_update<T, true>, r);
+      launch_k(X, st, KC_EUPD, DOM_CELLS, 0, MHD_BOTH(kb_euler_update, true), r);
     else
-      launch_k(X, st, KC_EUPD, DOM_CELLS, kb_euler_update<T, false>, r);
+      launch_k(X, st, KC_EUPD, DOM_CELLS, 0, MHD_BOTH(kb_euler_update, false), r);
   }
 }
 
@@ -433,17 +432,18 @@ void launch_lag_stage(Exec<T>& X, cudaStream_t st, bool fuse_last) {
   NvtxRange range("Lagrangian stage (Sec. 2.6)");
   for (int r = 0; r < 3; ++r) {
     if constexpr (lag_in_pencils<T>()) {
-      if (X.ions) launch_ks(X, st, KC_LFACE, DOM_LAG_PENCILS, LAG_SLOTS, kb_lag_pencil<true>);
-      else launch_ks(X, st, KC_LFACE, DOM_LAG_PENCILS, LAG_SLOTS, kb_lag_pencil<false>);
+      const size_t lag_bytes = pencil_smem_bytes(LAG_SLOTS, X.cfg[KC_LFACE].block);
+      if (X.ions) launch_k(X, st, KC_LFACE, DOM_LAG_PENCILS, lag_bytes, MHD_BOTH(kb_lag_pencil, true));
+      else launch_k(X, st, KC_LFACE, DOM_LAG_PENCILS, lag_bytes, MHD_BOTH(kb_lag_pencil, false));
     } else {
-      if (X.ions) launch_k(X, st, KC_LFACE, DOM_FACES, kb_lag_face<T, true>);
-      else launch_k(X, st, KC_LFACE, DOM_FACES, kb_lag_face<T, false>);
+      if (X.ions) launch_k(X, st, KC_LFACE, DOM_FACES, 0, MHD_BOTH(kb_lag_face, true));
+      else launch_k(X, st, KC_LFACE, DOM_FACES, 0, MHD_BOTH(kb_lag_face, false));
     }
     if (r == 2 && fuse_last) break;
     if (X.ions)
-      launch_k(X, st, KC_LUPD, DOM_CELLS, kb_lag_update<T, true>, r);
+      launch_k(X, st, KC_LUPD, DOM_CELLS, 0, MHD_BOTH(kb_lag_update, true), r);
     else
-      launch_k(X, st, KC_LUPD, DOM_CELLS, kb_lag_update<T, false>, r);
+      launch_k(X, st, KC_LUPD, DOM_CELLS, 0, MHD_BOTH(kb_lag_update, false), r);
   }
 }
 
@@ -453,9 +453,9 @@ template <typename T>
 void launch_post(Exec<T>& X, cudaStream_t st, int cell_stages, int do_reg, int check) {
   NvtxRange range("chemistry, heating/cooling, regularisation, CFL (Sec. 2.7-2.9, 2.3)");
   if (X.ions)
-    launch_k(X, st, KC_POST, DOM_CELLS, kb_post<T, true>, cell_stages, do_reg, check);
+    launch_k(X, st, KC_POST, DOM_CELLS, 0, MHD_BOTH(kb_post, true), cell_stages, do_reg, check);
   else
-    launch_k(X, st, KC_POST, DOM_CELLS, kb_post<T, false>, cell_stages, do_reg, check);
+    launch_k(X, st, KC_POST, DOM_CELLS, 0, MHD_BOTH(kb_post, false), cell_stages, do_reg, check);
 }
 
 // the last Lagrangian update with the post stage (kb_lag_update_post; the post stage's launch
@@ -464,9 +464,9 @@ template <typename T>
 void launch_lag_post(Exec<T>& X, cudaStream_t st, int cell_stages, int do_reg, int check) {
   NvtxRange range("last Lagrangian update + chemistry, heating/cooling, regularisation, CFL");
   if (X.ions)
-    launch_k(X, st, KC_POST, DOM_CELLS, kb_lag_update_post<T, true>, cell_stages, do_reg, check);
+    launch_k(X, st, KC_POST, DOM_CELLS, 0, MHD_BOTH(kb_lag_update_post, true), cell_stages, do_reg, check);
   else
-    launch_k(X, st, KC_POST, DOM_CELLS, kb_lag_update_post<T, false>, cell_stages, do_reg, check);
+    launch_k(X, st, KC_POST, DOM_CELLS, 0, MHD_BOTH(kb_lag_update_post, false), cell_stages, do_reg, check);
 }
 
 template <typename T>
