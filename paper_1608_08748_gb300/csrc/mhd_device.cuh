@@ -78,6 +78,8 @@ struct Phys {
 struct Scalars {
   double cfl, t_end;       // set by the host with a kernel launch (graph-safe)
   double tau, tau_h;       // this step's tau and tau / dx
+  double gth[3];           // g tau / dx of the three substages (Sec. 2.2)
+  float tau_h32;           // tau / dx in float (a conversion takes the FP64 pipe as long as an FMA)
   float ts[2];             // tau in seconds as a float pair (the FP32 path's chemistry)
   double t;                // simulated time
   unsigned long long dmax; // bits of max CFL denominator of the current state (positive double)

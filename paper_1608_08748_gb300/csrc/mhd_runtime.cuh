@@ -193,21 +193,22 @@ inline unsigned grid_of(const Tiles& t, const LaunchCfg& c, int nsm) {
   return (unsigned)(g > 0 ? g : 1);
 }
 
-// default launch shapes: the face kernels are register heavy (150-230 registers), so 128-thread
-// blocks let two or three blocks share an SM; the rest 256, one block per tile.  The FP32 path's
-// HBM-bound cell kernels (primitives, edge EMFs, the two updates, the post stage) run grid-stride over
-// their tiles with a few blocks per SM: on the 256^3 box that takes 0.04, 0.11, 0.15, 0.24 and 0.09 ms per
-// step off one block per tile (measured over 64-512 threads and 2-16 blocks per SM).
+// default launch shapes: the face kernels are register heavy (up to 242 registers), so 128-thread
+// blocks let two or more blocks share an SM; the rest 256, one block per tile.  The FP32 path's
+// HBM-bound cell kernels run grid-stride over their tiles with a few blocks per SM where that is faster
+// (256^3 step, measured over 64-512 threads and 2-16 blocks per SM: Lagrangian update 0.98 ms with 12 blocks
+// of 128 per SM, 1.20 with 8; Eulerian update 1.46 with 8, 1.52 one block per tile; edges 0.49 / 0.51;
+// post stage 0.93 / 0.95; primitives 0.53 ms one block per tile, 0.60 with 4 blocks of 512).
 template <typename T>
 void default_cfgs(Exec<T>& X) {
   for (int kc = 0; kc < NKC; ++kc) X.cfg[kc] = LaunchCfg{256, 0};
   X.cfg[KC_EFACE].block = 128;
   X.cfg[KC_LFACE].block = 128;
   if constexpr (sizeof(T) == 4) {
-    X.cfg[KC_PRIM] = LaunchCfg{512, 4};
+    X.cfg[KC_PRIM] = LaunchCfg{256, 0};
     X.cfg[KC_EDGES] = LaunchCfg{512, 4};
     X.cfg[KC_EUPD] = LaunchCfg{128, 8};
-    X.cfg[KC_LUPD] = LaunchCfg{128, 8};
+    X.cfg[KC_LUPD] = LaunchCfg{128, 12};
     X.cfg[KC_POST] = LaunchCfg{128, 8};
   }
 }
