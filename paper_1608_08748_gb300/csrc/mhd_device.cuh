@@ -445,6 +445,14 @@ __device__ __forceinline__ double quarter_nn(double x) {
   return with_hi(x, h > 0 ? h : 0);
 }
 __device__ __forceinline__ float quarter_nn(float x) { return 0.25f * x; }
+// x / 2 for x >= 0, likewise, and 4 x for a normal x
+__device__ __forceinline__ double half_nn(double x) {
+  const int h = hi_of(x) - (1 << 20);
+  return with_hi(x, h > 0 ? h : 0);
+}
+__device__ __forceinline__ float half_nn(float x) { return 0.5f * x; }
+__device__ __forceinline__ double four_b(double x) { return with_hi(x, hi_of(x) + (2 << 20)); }
+__device__ __forceinline__ float four_b(float x) { return 4.0f * x; }
 
 // A sufficient test of x > 2^-K s for x >= 0 and s > 0 on the high words (K exponents below s or more
 // fails, and so does a value under 2^-1022); FP32 takes the comparison it guards.
@@ -652,7 +660,7 @@ struct AvgCoef {
 };
 template <typename T>
 __device__ __forceinline__ AvgCoef<T> avg_coef(T y) {
-  const T h = in_register(T(0.5)), u = sub_t(in_register(T(1)), y), hu = fma(-h, y, h);
+  const T u = sub_t(in_register(T(1)), y), hu = scale_down_b<1>(u);
   return AvgCoef<T>{mul_t(y, hu), mul_t(u, hu)};
 }
 // the average next to the right edge of a cell less the cell's value, and the average next to the left
@@ -675,10 +683,8 @@ struct FaceSide {
 
 // The speeds, alpha factors and eigenvector entries are those of App. A in few FP64 instructions:
 //   one reciprocal of the weight sum; 1/sqrt(rho) gives 1/rho, sqrt(rho) and c_a = |B_n| / sqrt(rho);
-//   c_f^2 = (c^2 + c_a^2 + b_perp^2 + sq)/2 with sq = c_f^2 - c_s^2 =
-//     sqrt((c^2 - c_a^2)^2 + b_perp^2 (2 c^2 + 2 c_a^2 + b_perp^2)), sums of non-negative terms, and
-//     c_s = c c_a / c_f;
-//   with Z = c^2 - c_a^2 - b_perp^2: alpha_f^2 = (c^2 - c_s^2)/sq = (1 + Z/sq)/2 and alpha_s^2 =
+//   with Z = c^2 - c_a^2 - b_perp^2: c_f^2 = (c^2 + c_a^2 + b_perp^2 + sq)/2 with sq = c_f^2 - c_s^2 =
+//     sqrt(Z^2 + 4 c^2 b_perp^2), sums of non-negative terms, and c_s = c c_a / c_f; alpha_f^2 = (c^2 - c_s^2)/sq = (1 + Z/sq)/2 and alpha_s^2 =
 //     (c_f^2 - c^2)/sq = (1 - Z/sq)/2.  The larger of the two is formed from |Z|, without
 //     cancellation, and the other from alpha_f alpha_s = c b_perp / sq, with the one reciprocal square
 //     root of the larger: exactly 0 where B_perp = 0;
@@ -711,8 +717,8 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
   const T ca2 = mul_t(mul_t(Bn, Bn), irho);
   const T bp2 = fma(Bt1, Bt1, mul_t(Bt2, Bt2));
   const T b2 = mul_t(bp2, irho);  // b_perp^2
-  const T X = sub_t(c2, ca2), s2 = add_t(c2, ca2), s = add_t(s2, b2);
-  const T sq2 = fma(X, X, mul_t(b2, fma(T(2), s2, b2)));
+  const T s = add_t(add_t(c2, ca2), b2), Z = sub_t(sub_t(c2, ca2), b2);
+  const T sq2 = fma(Z, Z, mul_t(b2, four_b(c2)));
   // the directions of B_perp; the degenerate case keeps |B_perp| itself
   T by = INV_SQRT2, bz = INV_SQRT2, bper;
   if (surely_above<78>(b2, s) || gt_nn(bp2, T(1e-24) * rho * s)) {  // 1e-24 < 2^-79
@@ -729,8 +735,7 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
     const T isq = rsqrt_n(sq2), sqn = mul_t(sq2, isq);
     if (surely_above<38>(sqn, s) || gt_nn(sqn, T(1e-12) * s)) {  // 1e-12 < 2^-39
       sq = sqn;
-      const T Z = sub_t(X, b2);
-      const T big2 = fma(mul_t(HALF, abs_b(Z)), isq, HALF);  // in [1/2, 1]
+      const T big2 = fma(half_nn(abs_b(Z)), isq, HALF);  // in [1/2, 1]
       const T rb = rsqrt_n(big2), big = mul_t(big2, rb);
       const T small = mul_t(mul_t(mul_t(c, bper), mul_t(rs, isq)), rb);
       const bool fast = !sign_bit_b(Z);
@@ -738,7 +743,7 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
       as = fast ? small : big;
     }
   }
-  const T cf2 = mul_t(HALF, add_t(s, sq));
+  const T cf2 = half_nn(add_t(s, sq));
   const T rcf = rsqrt_n(cf2);
   const T cf = mul_t(cf2, rcf), ca = mul_t(abs_b(Bn), rs);
   const T cs = mul_t(mul_t(c, ca), rcf);
@@ -765,8 +770,8 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
     const T vl = fma(bys, ql[2], -mul_t(bzs, ql[1])), vr = fma(bys, qr[2], -mul_t(bzs, qr[1]));
     const T bl = fma(bz, ql[3], -mul_t(by, ql[4])), br = fma(bz, qr[3], -mul_t(by, qr[4]));
     const T sp = fma(rs, bl, vl), sm = fma(-rs, br, vr);
-    hv = mul_t(HALF, add_t(sp, sm));
-    hb = mul_t(mul_t(HALF, sqr), sub_t(sp, sm));
+    hv = scale_down_b<1>(add_t(sp, sm));
+    hb = mul_t(half_nn(sqr), sub_t(sp, sm));
   }
   // the magnetosonic waves on (v_n, v_par sgn(B_n), B_par, p): the +c_f wave has
   // L = (lf, -ls, as i2sc, af i2r), R = (af cf, -as cs, as sc, af gp), the +c_s wave
@@ -779,7 +784,7 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
   const Dev<T> rb = {along(r.P[3].A, r.P[4].A), along(r.P[3].B, r.P[4].B)};
   const T dv = along_s(d[1], d[2]), db = along(d[3], d[4]);
   const T af_cf = mul_t(af, cf), as_cs = mul_t(as, cs);
-  const T i2c2 = mul_t(mul_t(HALF, rc), rc), i2sc = mul_t(mul_t(HALF, rs), rc), i2r = mul_t(i2c2, irho);
+  const T hrc = half_nn(rc), i2c2 = mul_t(hrc, rc), i2sc = mul_t(rs, hrc), i2r = mul_t(i2c2, irho);
   const T lf = mul_t(af_cf, i2c2), ls = mul_t(as_cs, i2c2);
   auto pair = [&](AvgCoef<T> k, T l0, T l1, T l2, T l3, T& dif, T& sum) {
     const T sp = fma(l0, inc_right(l.P[0], k),

@@ -387,10 +387,11 @@ __device__ __forceinline__ void store_face_fluxes(const FaceOut<T>& fo, idx_t f,
   const T Vn = qs[0], Vt1 = qs[1], Vt2 = qs[2], Bt1 = qs[3], Bt2 = qs[4], P = qs[5];
   const T Bn2 = mul_t(Bn, Bn);
   const T pstar = fma(T(0.5), fma(Bt1, Bt1, fma(Bt2, Bt2, Bn2)), P);
-  fo.f[0][f] = sub_t(pstar, Bn2);
-  fo.f[1][f] = -mul_t(Bn, Bt1);
-  fo.f[2][f] = -mul_t(Bn, Bt2);
-  fo.f[3][f] = fma(pstar, Vn, -mul_t(Bn, fma(Bn, Vn, fma(Bt1, Vt1, mul_t(Bt2, Vt2)))));
+  const T Fn = sub_t(pstar, Bn2), F1 = -mul_t(Bn, Bt1), F2 = -mul_t(Bn, Bt2);
+  fo.f[0][f] = Fn;
+  fo.f[1][f] = F1;
+  fo.f[2][f] = F2;
+  fo.f[3][f] = fma(Fn, Vn, fma(F1, Vt1, mul_t(F2, Vt2)));  // p* V_n - B_n (B . V)
   fo.f[4][f] = Vn;
   fo.f[5][f] = fma(Bn, Vt1, -mul_t(Bt1, Vn));
   fo.f[6][f] = fma(Bt2, Vn, -mul_t(Bn, Vt2));
