@@ -487,12 +487,12 @@ __device__ __forceinline__ T half_slope(T s, T dn, T dp) {
 //   Step 5: Delta q = (A + B)/2 and q6 = 3 (A - B)/2 are not formed: the averages of Sec. 2.4 over
 //           the fraction y next to the right or the left edge are
 //             q + y u A/2 + u^2 B/2   and   q - u^2 A/2 - y u B/2   with u = 1 - y.
-// On the FP64 pipe, the bound of the FP64 faces, a streamed parabola takes 7 instructions besides
-// Step 4's blend (with edge values, Delta q and q6 it took 17), and an average the same two FMAs; on
-// the FP32 path it takes about half the instructions.  The deviations also round less: no edge value
-// is formed from which q is subtracted again.  With the Riemann solve below, one step of the turbulence
-// box went from 25.6 to 19.4 ms at 128^3 in FP64 (Eulerian faces 16.2 -> 12.8, Lagrangian 8.7 -> 5.6 ms)
-// and from 15.9 to 14.5 ms at 256^3 in FP32 (5.2 -> 4.5, 4.1 -> 3.4 ms).
+// A streamed parabola takes 7 floating-point instructions besides Step 4's blend (with edge values, Delta q
+// and q6 it took 17), and an average the same two FMAs; the FP64 faces form the same deviations in fixed
+// point (fix_dev below).  The deviations also round less: no edge value is formed from which q is subtracted
+// again.  With the Riemann solve below, one step of the turbulence box went from 25.6 to 19.4 ms at 128^3
+// in FP64 (then still with FP64 parabolas) and from 15.9 to 14.5 ms at 256^3 in FP32 (Eulerian faces
+// 5.2 -> 4.5, Lagrangian 4.1 -> 3.4 ms).
 template <typename T>
 struct Dev {
   T A, B;
@@ -502,35 +502,22 @@ struct Dev {
 // D-, s0 = q_{+1} - q_{-1} and the two neighbours' values.  Step 4's eta = -(D+ - D-)/(3 s0) acts where
 // |s0| > min(|q_{+1}|, |q_{-1}|)/100 (the smaller of the paper's three values is one of the two) and
 // D+ D- <= 0; hbar = 20 (eta - 1/20) = (20/3)(D- - D+)/s0 - 1, clamped to [0, 1].
-// In FP64: Step 2 by comparisons of magnitudes on the integer pipe (where the signs agree neither is 0).
-__device__ __forceinline__ Dev<double> dev_monotone(double A, double B) {
-  const bool mono = same_sign(A, B);
-  const double aA = abs_b(A), aB = abs_b(B), A2 = twice_b(A), B2 = twice_b(B);
-  const bool up = gt_nn(aA, abs_b(B2)), dn = gt_nn(aB, abs_b(A2));
-  return Dev<double>{mono ? (up ? B2 : A) : 0.0, mono ? (dn ? A2 : B) : 0.0};
-}
-// Whether Step 4 may act (num = D- - D+, mn = min(|q_{+1}|, |q_{-1}|)): D+ D- <= 0 exactly, and hbar > 0,
-// |s0| > mn / 100 on the high words, which are e + f for 2^e (1 + f) and lie at most 0.0861 below the
-// base-2 logarithm: hbar > 0 is log2 |num| > log2 |s0| - 2.7370 with the sign of s0, |s0| > mn / 100 is
-// log2 |s0| > log2 mn - 6.6439.  It never misses a cell where Step 4 acts; step4 makes the exact test.
-__device__ __forceinline__ bool step4_candidate(double Dp, double Dm, double num, double s0, double mn) {
-  const int hn = hi_of(abs_b(num)), hs = hi_of(abs_b(s0));
-  return same_sign(num, s0) && !same_sign(Dp, Dm) && hn > hs - (int)(2.83 * (1 << 20)) &&
-         hs > hi_of(mn) - (int)(6.74 * (1 << 20));
-}
-// Step 4's blend.  hbar = 20 eta - 1 is continuous where it crosses 0 and 1, so the clamps' rounding
-// cannot move the result.
-__device__ __forceinline__ Dev<double> step4(Dev<double> P, double h0, double num, double s0, double mn) {
-  double hb = fma(mul_t(in_register(20.0 / 3.0), num), rcp_nr(s0), -in_register(1.0));
-  hb = min_nn(hb, 1.0);
-  if (sign_bit_b(hb) || !gt_nn(abs_b(s0), mul_t(in_register(0.01), mn))) hb = 0.0;
-  return Dev<double>{fma(hb, sub_t(h0, P.A), P.A), fma(hb, sub_t(h0, P.B), P.B)};
-}
+// In FP64 (only the wide stencils of the fixed-point form below come here): hbar is continuous where it
+// crosses 0 and 1, so the clamps' rounding cannot move the result.
 __device__ __forceinline__ Dev<double> dev_limit(double A, double B, double h0, double Dp, double Dm, double s0,
                                                  double qp1, double qm1) {
-  const Dev<double> P = dev_monotone(A, B);
-  const double num = sub_t(Dm, Dp), mn = min_nn(abs_b(qp1), abs_b(qm1));
-  return step4_candidate(Dp, Dm, num, s0, mn) ? step4(P, h0, num, s0, mn) : P;
+  const bool mono = same_sign(A, B);
+  const double mA = min_nn(abs_b(A), abs_b(twice_b(B))), mB = min_nn(abs_b(B), abs_b(twice_b(A)));
+  A = mono ? with_sign_b(mA, A) : 0.0;
+  B = mono ? with_sign_b(mB, B) : 0.0;
+  if (!same_sign(Dp, Dm) && gt_nn(abs_b(s0), mul_t(0.01, min_nn(abs_b(qp1), abs_b(qm1))))) {
+    const double hb = min_nn(fma(mul_t(20.0 / 3.0, sub_t(Dm, Dp)), rcp_nr(s0), -1.0), 1.0);
+    if (!sign_bit_b(hb)) {
+      A = fma(hb, sub_t(h0, A), A);
+      B = fma(hb, sub_t(h0, B), B);
+    }
+  }
+  return Dev<double>{A, B};
 }
 // FP32: bound by instruction issue, so selects instead of branches, and the reciprocal is taken
 // everywhere and discarded where the detector is off (s0 may be 0 there); the clamp is the FMA's own
@@ -620,6 +607,145 @@ struct DevStream {
   }
 };
 
+// ------------------------------------------------------------------------------------------------
+// The FP64 parabolas in fixed point.  Steps 1 and 2 of Sec. 2.1 are differences, minima, small integer
+// multiples and comparisons, so within one stencil they need no floating point: the five values are
+// aligned to the largest exponent among them as 64-bit integers with 59 bits for the magnitude (the
+// largest value keeps all its 53 bits and 6 to spare; a smaller one is cut at 2^-59 of the largest), and the
+// work runs on the integer pipes, which issue 32 instructions in the time the FP64 pipe takes one.
+// A stencil's result depends on nothing else, so a pencil's length does not show.  Results are held as 3 A
+// and 3 B (no division by 3; the averages' coefficients carry the third), rounded once from the integers: against
+// 113-bit arithmetic the error of A is 0.4 to 1.3 times that of the FP64 form (r.m.s. over smooth, steep and rough
+// stencils) and that of a whole step the same (8.6e-17 of the density at 96^3).  A streamed parabola
+// took 7 FP64 instructions besides Step 4; here it takes none.  128^3 FP64 step at the developed flow, with the
+// pencils in blocks of 64 threads: 16.5 -> 14.2 ms (Eulerian faces 10.3 -> 9.3, Lagrangian 4.1 -> 2.8 ms).
+// Its callers keep their loops rolled: unrolled over cells the Lagrangian faces take 3.1 / 3.3 / 3.6 ms for 1, 2
+// and 3 cells (128-thread blocks).
+struct FixCell {
+  long long n;  // value 2^(1081 - e), |n| < 2^59
+  int e;        // biased exponent, at least 1
+};
+__device__ __forceinline__ long long bits_of(double q) {
+#ifdef __CUDA_ARCH__
+  return __double_as_longlong(q);
+#else
+  long long b;
+  __builtin_memcpy(&b, &q, 8);
+  return b;
+#endif
+}
+__device__ __forceinline__ double dbl_of(long long b) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double(b);
+#else
+  double q;
+  __builtin_memcpy(&q, &b, 8);
+  return q;
+#endif
+}
+__device__ __forceinline__ int min_i(int a, int b) { return a < b ? a : b; }
+__device__ __forceinline__ int max_i(int a, int b) { return a > b ? a : b; }
+__device__ __forceinline__ FixCell fix_cell(double q) {
+  const long long b = bits_of(q);
+  const int f = (int)((unsigned long long)b >> 52) & 0x7ff;
+  FixCell c;
+  c.e = f > 0 ? f : 1;
+  const long long m = ((b & 0xfffffffffffffll) | (f > 0 ? 1ll << 52 : 0)) << 6;
+  c.n = b < 0 ? -m : m;
+  return c;
+}
+__device__ __forceinline__ int leading_zeros(unsigned long long x) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)x);
+#else
+  return x ? __builtin_clzll(x) : 64;
+#endif
+}
+// sgn m 2^(E - 1081) as a double, m < 2^63, rounded to nearest (0 below 2^-1022); neg is 0 or -1
+__device__ __forceinline__ double fix_to_double(unsigned long long m, long long neg, int E) {
+  const int z = leading_zeros(m), e = E + 4 - z;  // the biased exponent less one
+  const unsigned long long f = ((m << (z - 1)) + 0x200) >> 10;
+  const unsigned long long b = f + ((unsigned long long)(unsigned)e << 52) + (neg & (1ull << 63));
+  return m != 0 && e >= 0 ? dbl_of((long long)b) : 0.0;
+}
+__device__ __forceinline__ unsigned long long uabs64(long long a) { return (unsigned long long)(a < 0 ? -a : a); }
+__device__ __forceinline__ double fix_value(FixCell c) { return fix_to_double(uabs64(c.n), c.n >> 63, c.e); }
+// min(a, b, (a + b)/4): the halved slope of a cell whose two differences a and b are not negative, negative where
+// one of them is
+__device__ __forceinline__ long long fix_half_slope(long long a, long long b) {
+  const long long m = a < b ? a : b, t = (a + b) >> 2;
+  return m < t ? m : t;
+}
+__device__ __forceinline__ long long not_negative(long long a) { return a & ~(a >> 63); }
+__device__ __forceinline__ int hi_word(long long a) { return (int)(a >> 32); }
+// What Step 4 takes of a cell: |num| = |D- - D+|, |s0|, three times the halved slope's magnitude and min(|q_{+1}|,
+// |q_{-1}|), all times 2^(1081 - E); the sign of the parabola is that of its deviations
+struct FixStep4 {
+  long long num, s0, h3, ql, qr;  // (ql, qr) = q_{-1}, q_{+1}
+  int E;
+};
+// Steps 1 and 2 of the cell in the middle of q_{-2} .. q_{+2}: 3 A and 3 B.  All is done with the sign of
+// q_0 - q_{-1} taken off: where q_{+1} - q_0 is then negative the cell is an extremum, and else the
+// cell's own slope and A and B are not negative, and a neighbour's slope counts only where it is not.  Returns
+// whether Step 4 may act (never false where it does): D- >= 0 >= D+, and by the high words |num| > 3 |s0| / 20
+// and |s0| > mn / 128.  A wide stencil, where the largest exponent is more than 5 above that of the cell and of one
+// of its neighbours (the results are at most a few times the smaller of the two differences, so the cut
+// would show), or with an infinity or a NaN, is done as a whole in FP64.
+__device__ __forceinline__ bool fix_dev(const FixCell c[5], Dev<double>& P, FixStep4& st) {
+  const int near = max_i(c[2].e, min_i(c[1].e, c[3].e));
+  const int E = max_i(max_i(max_i(c[0].e, c[1].e), max_i(c[3].e, c[4].e)), c[2].e);
+  const bool wide = E > near + 5 || E == 0x7ff;
+  long long q[5], d[4];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) q[k] = c[k].n >> min_i(E - c[k].e, 63);
+  const long long neg = (q[2] - q[1]) >> 63;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) d[k] = ((q[k + 1] - q[k]) ^ neg) - neg;
+  const long long h0 = fix_half_slope(d[1], d[2]), hm = not_negative(fix_half_slope(d[0], d[1])),
+                  hp = not_negative(fix_half_slope(d[2], d[3]));
+  const long long A = 3 * d[1] + 2 * (h0 - hm), B = 3 * d[2] - 2 * (hp - h0);  // below 5 2^60
+  const unsigned long long uA = (unsigned long long)A, uB = (unsigned long long)B;
+  const unsigned long long mA = uA < 2 * uB ? uA : 2 * uB, mB = uB < 2 * uA ? uB : 2 * uA;
+  const bool mono = d[2] >= 0;
+  P.A = fix_to_double(mono ? mA : 0, neg, E);
+  P.B = fix_to_double(mono ? mB : 0, neg, E);
+  const long long Dm = d[1] - d[0], Dp = d[2] - d[3];  // D- and -D+
+  st = FixStep4{Dm + Dp, d[1] + d[2], 3 * h0, q[1], q[3], E};
+  const int ml = hi_word(q[1]), mr = hi_word(q[3]);
+  const int mn = min_i(ml ^ (ml >> 31), mr ^ (mr >> 31));
+  const unsigned hn = (unsigned)hi_word(st.num) >> 2, hs = (unsigned)hi_word(st.s0) >> 2;
+  const bool cand = (hi_word(Dm) | hi_word(Dp) | hi_word(d[2])) >= 0 && st.num != 0 && 7u * (hn + 1) >= hs &&
+                    hs + 1 >= ((unsigned)mn >> 9);
+  if (wide) {
+    const Dev<double> W = dev_of(fix_value(c[0]), fix_value(c[1]), fix_value(c[2]), fix_value(c[3]), fix_value(c[4]));
+    P = Dev<double>{mul_t(3.0, W.A), mul_t(3.0, W.B)};
+    return false;
+  }
+  return cand;
+}
+__device__ __forceinline__ long long fix_min_abs(const FixStep4& st) {
+  const unsigned long long l = uabs64(st.ql), r = uabs64(st.qr);
+  return (long long)(l < r ? l : r);
+}
+// Step 4's blend from there (the integers convert on the FP64 pipe, once per 32 gathered cells): hbar =
+// (20/3) num / s0 - 1 clamped to [0, 1], 3 A += hbar (3 h - 3 A).
+__device__ __forceinline__ Dev<double> fix_step4(Dev<double> P, long long n, long long s, long long h3, long long mn,
+                                                 int E) {
+  const double num = (double)n, s0 = (double)s;
+  double hb = fma(mul_t(in_register(20.0 / 3.0), num), rcp_nr(s0), -in_register(1.0));
+  hb = min_nn(hb, 1.0);
+  if (sign_bit_b(hb) || !gt_nn(s0, mul_t(in_register(0.01), (double)mn))) hb = 0.0;
+  const double h = with_sign_b(fix_to_double((unsigned long long)h3, 0, E), P.A);  // A = 0: h = 0
+  return Dev<double>{fma(hb, sub_t(h, P.A), P.A), fma(hb, sub_t(h, P.B), P.B)};
+}
+// the deviations of the cell in the middle of five values, by the same steps
+__device__ __forceinline__ Dev<double> fix_dev_of(const FixCell c[5]) {
+  Dev<double> P;
+  FixStep4 st;
+  if (fix_dev(c, P, st)) P = fix_step4(P, st.num, st.s0, st.h3, fix_min_abs(st), st.E);
+  return Dev<double>{P.A * (1.0 / 3.0), P.B * (1.0 / 3.0)};
+}
+
 // The parabola by its edge values, Delta q = q^R - q^L and q6 (the paper's own form), from the value
 // and the deviations, and the forms that return it; the kernels take the deviations.
 template <typename T>
@@ -628,13 +754,33 @@ __device__ __forceinline__ Para<T> para_of(T q, Dev<T> P) {
 }
 template <typename T>
 __device__ __forceinline__ Para<T> ppm_lean(T qm2, T qm1, T qc, T qp1, T qp2) {
-  return para_of(qc, dev_of(qm2, qm1, qc, qp1, qp2));
+  if constexpr (sizeof(T) == 8) {
+    const FixCell c[5] = {fix_cell(qm2), fix_cell(qm1), fix_cell(qc), fix_cell(qp1), fix_cell(qp2)};
+    return para_of(qc, fix_dev_of(c));
+  } else {
+    return para_of(qc, dev_of(qm2, qm1, qc, qp1, qp2));
+  }
 }
+// consecutive cells along a line (FP64): prime with q_{J-2} .. q_{J+1}, then next(q_{j+2}) for j = J, J+1, ...
 template <typename T>
-struct PPMStream : DevStream<T> {
+struct PPMStream {
+  FixCell c[5];
+  T q[2];
+  __device__ __forceinline__ void prime(T qa, T qb, T qc, T qd) {
+    c[1] = fix_cell(qa);
+    c[2] = fix_cell(qb);
+    c[3] = fix_cell(qc);
+    c[4] = fix_cell(qd);
+    q[0] = qc;
+    q[1] = qd;
+  }
   __device__ __forceinline__ Para<T> next(T qn) {
-    const Dev<T> P = DevStream<T>::next(qn);
-    return para_of(this->qm, P);
+    for (int k = 0; k < 4; ++k) c[k] = c[k + 1];
+    c[4] = fix_cell(qn);
+    const T v = q[0];
+    q[0] = q[1];
+    q[1] = qn;
+    return para_of(v, fix_dev_of(c));
   }
 };
 // ... from the slopes of the cells i - 1, i, i + 1 and the second differences around them
@@ -653,14 +799,18 @@ __device__ __forceinline__ Para<T> ppm_direct(T qm2, T qm1, T qc, T qp1, T qp2) 
                      qp2 - T(2) * qp1 + qc, qc - T(2) * qm1 + qm2);
 }
 
-// the coefficients of A and B in the averages over the fraction y (Sec. 2.4): y u / 2 and u^2 / 2
+// the coefficients of A and B in the averages over the fraction y (Sec. 2.4): y u / 2 and u^2 / 2; in FP64 those
+// of 3 A and 3 B
 template <typename T>
 struct AvgCoef {
   T p, r;
 };
 template <typename T>
 __device__ __forceinline__ AvgCoef<T> avg_coef(T y) {
-  const T u = sub_t(in_register(T(1)), y), hu = scale_down_b<1>(u);
+  const T u = sub_t(in_register(T(1)), y);
+  T hu;
+  if constexpr (sizeof(T) == 8) hu = mul_t(u, in_register(1.0 / 6.0));
+  else hu = scale_down_b<1>(u);
   return AvgCoef<T>{mul_t(y, hu), mul_t(u, hu)};
 }
 // the average next to the right edge of a cell less the cell's value, and the average next to the left
@@ -815,9 +965,10 @@ __device__ __forceinline__ void riemann(const T wl[6], const T wr[6], T Bn, cons
     FaceSide<T> f;
     for (int m = 0; m < 6; ++m) {
       f.w[m] = w[m];
-      f.P[m].A = P[m].d + P[m].q6 * T(1.0 / 3.0);
-      f.P[m].B = P[m].d - P[m].q6 * T(1.0 / 3.0);
-      f.q[m] = P[m].L + T(0.5) * f.P[m].A;
+      const T A = P[m].d + P[m].q6 * T(1.0 / 3.0), B = P[m].d - P[m].q6 * T(1.0 / 3.0);
+      f.q[m] = P[m].L + T(0.5) * A;
+      f.P[m].A = sizeof(T) == 8 ? T(3) * A : A;
+      f.P[m].B = sizeof(T) == 8 ? T(3) * B : B;
     }
     return f;
   };

@@ -177,9 +177,10 @@ __device__ __forceinline__ Line line_of_pencil(const Box<T>& B, const Pencils& P
 }
 
 // Programmatic dependent launch: the step's kernels are launched so that a kernel's blocks may take their
-// places while the one before it drains (launch_dep).  Every such kernel first lets the next one come
-// and then waits until the one before it has finished and its writes are visible; as each kernel does so
-// before it reads or writes anything, the order of the memory accesses is that of plain launches.
+// places while the one before it drains (launch_dep).  Every such kernel first waits until the one before it has
+// finished and its writes are visible; as it does so before it reads or writes anything, the order of the
+// memory accesses is that of plain launches.  The next kernel may come when a block ends: let in at the start, its
+// waiting blocks crowd the places of the few running ones (128x4x4 FP64 step 262 against 224 us).
 __device__ __forceinline__ void dependent_launch_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -284,23 +285,23 @@ __device__ __forceinline__ double& pencil_slot(int k) {
 }
 
 // Step 4 of the FP64 parabolas, gathered over the warp.  Step 4 acts on one parabola in ten or less, but
-// nearly every warp has a lane where it does, so as a branch its 10 FP64 instructions cost almost every
-// parabola as much as its other 7.  The lanes put what it needs in a ring of the warp in shared memory
-// instead, and when 32 have come together (or the results are wanted) the warp does them at once, one
-// per lane.  The deviations wait in slots of the owner's column; a result does not depend on how the ring
-// groups it.  All 32 lanes call push and flush together.  128^3 FP64 step at the developed flow: 20.0 ->
-// 17.2 ms (Eulerian faces 11.9 -> 10.8, Lagrangian 5.9 -> 4.1 ms, there with the FP64 pipe 92 % busy).
+// nearly every warp has a lane where it does, so as a branch its FP64 instructions would cost every
+// parabola.  The lanes put what it needs in a ring of the warp in shared memory instead, and when 32 have
+// come together (or the results are wanted) the warp does them at once, one per lane.  The deviations wait
+// in slots of the owner's column; a result does not depend on how the ring groups it.  All 32 lanes call
+// push and flush together.  (With the parabolas in FP64, 128^3 FP64 step at the developed flow: as a branch
+// 20.0, gathered 17.2 ms.)
 struct Step4Ring {
   static constexpr int N = 64;  // at most 31 left over and 32 new
-  static constexpr size_t BYTES = N * (4 * sizeof(double) + sizeof(int));
-  double* num;   // num, s0, h0, mn of the items, N each
-  int* who;      // the owner's slot of A; that of B lies `off` further
+  static constexpr size_t BYTES = N * (4 * sizeof(long long) + 2 * sizeof(int));
+  long long* val;  // the four words of the items, N each
+  int* who;        // the owner's slot of A (that of B lies `off` further), and E
   int off;
   int head = 0, count = 0;
   __device__ __forceinline__ Step4Ring(int slots, int slots_to_B) : off(slots_to_B * (int)blockDim.x) {
     unsigned char* base = pencil_smem_raw + (size_t)slots * blockDim.x * sizeof(double) + (threadIdx.x >> 5) * BYTES;
-    num = reinterpret_cast<double*>(base);
-    who = reinterpret_cast<int*>(base + 4 * N * sizeof(double));
+    val = reinterpret_cast<long long*>(base);
+    who = reinterpret_cast<int*>(base + 4 * N * sizeof(long long));
   }
   __device__ __forceinline__ void process(int n) {
     __syncwarp();
@@ -308,7 +309,8 @@ struct Step4Ring {
     if (lane < n) {
       const int i = (head + lane) & (N - 1);
       double* ab = reinterpret_cast<double*>(pencil_smem_raw) + who[i];
-      const Dev<double> P = step4(Dev<double>{ab[0], ab[off]}, num[2 * N + i], num[i], num[N + i], num[3 * N + i]);
+      const Dev<double> P =
+          fix_step4(Dev<double>{ab[0], ab[off]}, val[i], val[N + i], val[2 * N + i], val[3 * N + i], who[N + i]);
       ab[0] = P.A;
       ab[off] = P.B;
     }
@@ -317,15 +319,16 @@ struct Step4Ring {
     __syncwarp();
   }
   // slot: the slot of A (B is at slot + slots_to_B)
-  __device__ __forceinline__ void push(bool cand, int slot, double num_, double s0, double h0, double mn) {
+  __device__ __forceinline__ void push(bool cand, int slot, const FixStep4& st) {
     const unsigned m = __ballot_sync(0xffffffffu, cand);
     if (cand) {
       const int i = (head + count + __popc(m & ((1u << (threadIdx.x & 31)) - 1))) & (N - 1);
-      num[i] = num_;
-      num[N + i] = s0;
-      num[2 * N + i] = h0;
-      num[3 * N + i] = mn;
+      val[i] = st.num;
+      val[N + i] = st.s0;
+      val[2 * N + i] = st.h3;
+      val[3 * N + i] = fix_min_abs(st);
       who[i] = slot * blockDim.x + threadIdx.x;
+      who[N + i] = st.E;
     }
     count += __popc(m);
     if (count >= 32) process(32);
@@ -338,45 +341,23 @@ struct Step4Ring {
 constexpr size_t pencil_smem_bytes(int slots, int block) {
   return (size_t)slots * block * sizeof(double) + (size_t)(block / 32) * Step4Ring::BYTES;
 }
-// limits of the next cell of a stream (live: this lane has one): Step 2 at once, the deviations into the
-// slots, Step 4 into the ring
-__device__ __forceinline__ void stream_limits(DevStream<double>& S, double qn, bool live, Step4Ring& ring, int slotA,
-                                              int slotB) {
-  S.next(qn, [&](double A, double B, double h0, double Dp, double Dm, double s0, double qp1, double qm1) {
-    const Dev<double> P = dev_monotone(A, B);
-    pencil_slot(slotA) = P.A;
-    pencil_slot(slotB) = P.B;
-    const double num = sub_t(Dm, Dp), mn = min_nn(abs_b(qp1), abs_b(qm1));
-    ring.push(live && step4_candidate(Dp, Dm, num, s0, mn), slotA, num, s0, h0, mn);
-  });
+// the deviations of the middle cell of c (live: this lane has one): Steps 1 and 2 at once, into the slots,
+// Step 4 into the ring
+__device__ __forceinline__ void ring_dev(const FixCell c[5], bool live, Step4Ring& ring, int slotA, int slotB) {
+  Dev<double> P;
+  FixStep4 st;
+  const bool cand = fix_dev(c, P, st);
+  pencil_slot(slotA) = P.A;
+  pencil_slot(slotB) = P.B;
+  ring.push(live && cand, slotA, st);
 }
 
-// The FP64 Eulerian pencils keep each primitive's DevStream (9 values) in the slots 9 v .. 9 v + 8, and
-// the new cell's deviations in the slots 54 + v (A) and 60 + v (B).
-constexpr int EULER_SLOTS = 9 * 6 + 12;
-__device__ __forceinline__ void stream_save(const DevStream<double>& S, int v) {
-  pencil_slot(9 * v) = S.qm;
-  pencil_slot(9 * v + 1) = S.q0;
-  pencil_slot(9 * v + 2) = S.qp;
-  pencil_slot(9 * v + 3) = S.dp;
-  pencil_slot(9 * v + 4) = S.h0;
-  pencil_slot(9 * v + 5) = S.A;
-  pencil_slot(9 * v + 6) = S.Cm;
-  pencil_slot(9 * v + 7) = S.C0;
-  pencil_slot(9 * v + 8) = S.s0;
-}
-__device__ __forceinline__ DevStream<double> stream_load(int v) {
-  DevStream<double> S;
-  S.qm = pencil_slot(9 * v);
-  S.q0 = pencil_slot(9 * v + 1);
-  S.qp = pencil_slot(9 * v + 2);
-  S.dp = pencil_slot(9 * v + 3);
-  S.h0 = pencil_slot(9 * v + 4);
-  S.A = pencil_slot(9 * v + 5);
-  S.Cm = pencil_slot(9 * v + 6);
-  S.C0 = pencil_slot(9 * v + 7);
-  S.s0 = pencil_slot(9 * v + 8);
-  return S;
+// The FP64 Eulerian pencils keep of each primitive v the last cells in rings of slots: the values of four
+// (10 v .. 10 v + 3), the integers of five (10 v + 4 .. 10 v + 8) and their exponents, 11 bits each, in one
+// word (10 v + 9); the new cell's deviations in the slots 60 + v (A) and 66 + v (B).
+constexpr int EULER_SLOTS = 10 * 6 + 12;
+__device__ __forceinline__ long long& pencil_word(int k) {
+  return reinterpret_cast<long long*>(pencil_smem_raw)[k * blockDim.x + threadIdx.x];
 }
 
 // The fluxes of one Eulerian face f of direction D from its Riemann solution q* = (V_n, V_t1, V_t2,
@@ -515,16 +496,19 @@ __device__ __forceinline__ void euler_pencil(const Box<double>& B, int D, idx_t 
   const double* qv[6] = {B.w.v[D], B.w.v[D1], B.w.v[D2], B.w.B[D1], B.w.B[D2], B.w.p};
   auto cell_at = [&](int i) { return L.cell(g, i); };
   Step4Ring ring(EULER_SLOTS, 6);
-  {
-    idx_t cell[4];
+  // cell j of the pencil (j = 0 is cell f0 - 3): its value in ring place j % 4, its integer in j % 5
 #pragma unroll
-    for (int o = 0; o < 4; ++o) cell[o] = cell_at(f0 - 3 + o);
+  for (int v = 0; v < 6; ++v) {
+    long long es = 0;
 #pragma unroll
-    for (int v = 0; v < 6; ++v) {
-      DevStream<double> S;
-      S.prime(qv[v][cell[0]], qv[v][cell[1]], qv[v][cell[2]], qv[v][cell[3]]);
-      stream_save(S, v);
+    for (int j = 0; j < 4; ++j) {
+      const double q = qv[v][cell_at(f0 - 3 + j)];
+      const FixCell c = fix_cell(q);
+      pencil_slot(10 * v + j) = q;
+      pencil_word(10 * v + 4 + j) = c.n;
+      es |= (long long)c.e << (11 * (j + 1));
     }
+    pencil_word(10 * v + 9) = es;
   }
   FaceSide<double> l, r;  // the face's two cells; l.P carries the previous face's right cell
 #pragma unroll 1
@@ -533,19 +517,34 @@ __device__ __forceinline__ void euler_pencil(const Box<double>& B, int D, idx_t 
     const bool on = k < nfp;
     if (!__any_sync(0xffffffffu, on)) break;
     const idx_t cn = cell_at(on ? i + 2 : f0);
+    const int w4 = (k + 1) & 3;  // the new cell's place in the value rings: cell f0 + k + 2 is j = k + 5
+    int w5[5];                   // the window's places in the integer rings: the cells j = k + 1 .. k + 5
+    w5[0] = (k + 1) % 5;
 #pragma unroll
+    for (int o = 1; o < 5; ++o) w5[o] = w5[o - 1] == 4 ? 0 : w5[o - 1] + 1;
+#pragma unroll 1
     for (int v = 0; v < 6; ++v) {
-      DevStream<double> S = stream_load(v);
-      l.q[v] = S.qm;  // cell i - 1
-      stream_limits(S, qv[v][cn], on, ring, 54 + v, 60 + v);
-      r.q[v] = S.qm;  // cell i
-      stream_save(S, v);
+      const double q = qv[v][cn];
+      FixCell c[5];
+      c[4] = fix_cell(q);
+      const long long es = ((unsigned long long)pencil_word(10 * v + 9) >> 11) | ((long long)c[4].e << 44);
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        c[o].n = pencil_word(10 * v + 4 + w5[o]);
+        c[o].e = (int)(es >> (11 * o)) & 0x7ff;
+      }
+      pencil_slot(10 * v + w4) = q;
+      pencil_word(10 * v + 4 + w5[4]) = c[4].n;
+      pencil_word(10 * v + 9) = es;
+      ring_dev(c, on, ring, 60 + v, 66 + v);
     }
     ring.flush();
 #pragma unroll
     for (int v = 0; v < 6; ++v) {
-      r.P[v].A = pencil_slot(54 + v);
-      r.P[v].B = pencil_slot(60 + v);
+      l.q[v] = pencil_slot(10 * v + ((k + 2) & 3));  // cell i - 1: j = k + 2
+      r.q[v] = pencil_slot(10 * v + ((k + 3) & 3));  // cell i
+      r.P[v].A = pencil_slot(60 + v);
+      r.P[v].B = pencil_slot(66 + v);
     }
     if (k >= 0 && on) {
       const idx_t cl = cell_at(i - 1), cr = cell_at(i);
@@ -890,9 +889,9 @@ __global__ void __launch_bounds__(256) kb_lag_face(const __grid_constant__ SRC s
 }
 
 // The same fluxes in FP64 for the faces i_D - 1/2, i_D in [s P, min((s+1) P, n_D + 1)), P = pl.len[D],
-// of one pencil s: the face velocities first, then field by field the deviations of the pencil's cells in one
-// DevStream along D, Step 4 gathered over the warp (Step4Ring), then each face's average of its upwind
-// cell.  Slots: v_n and the two average coefficients of each face, then A, B and the value of each cell.
+// of one pencil s: the face velocities first, then field by field the deviations of the pencil's cells from a
+// window of five integers that slides along D, Step 4 gathered over the warp (Step4Ring), then each face's
+// average of its upwind cell.  Slots: v_n and the two average coefficients of each face, then A, B and the value of each cell.
 constexpr int LAG_FACES = pencil_len<double>(), LAG_CELLS = LAG_FACES + 1;
 constexpr int LAG_SLOTS = 3 * LAG_FACES + 3 * LAG_CELLS;
 template <bool IONS>
@@ -935,8 +934,12 @@ __device__ __forceinline__ void lag_pencil(const Box<double>& B, int D, idx_t p,
   for (int v = 0; v < nv; ++v) {
     const double* a = v == 0 ? B.s.rho : v < 4 ? B.s.m[v - 1] : v == 4 ? B.s.E : v == 5 ? B.s.eint
                       : (IONS && v == 7) ? B.s.rhp : B.s.rh2;
-    DevStream<double> S;
-    S.prime(a[cell_at(f0 - 3)], a[cell_at(f0 - 2)], a[cell_at(f0 - 1)], a[cell_at(f0)]);
+    FixCell w[5];
+    double qa = a[cell_at(f0 - 1)], qb = a[cell_at(f0)];  // the values of the next two cells
+    w[1] = fix_cell(a[cell_at(f0 - 3)]);
+    w[2] = fix_cell(a[cell_at(f0 - 2)]);
+    w[3] = fix_cell(qa);
+    w[4] = fix_cell(qb);
     double q1 = a[cell_at(f0 + 1)];  // one cell ahead, so that its latency overlaps the cell before
 #pragma unroll 1
     for (int c = 0; c < LAG_CELLS; ++c) {  // cell f0 - 1 + c
@@ -944,8 +947,13 @@ __device__ __forceinline__ void lag_pencil(const Box<double>& B, int D, idx_t p,
       if (!__any_sync(0xffffffffu, on)) break;
       const double qn = q1;
       q1 = a[cell_at(c < nfp ? f0 + 2 + c : f0)];
-      pencil_slot(CQ + c) = S.q0;
-      stream_limits(S, qn, on, ring, CA + c, CB + c);
+      pencil_slot(CQ + c) = qa;
+      qa = qb;
+      qb = qn;
+#pragma unroll
+      for (int o = 0; o < 4; ++o) w[o] = w[o + 1];
+      w[4] = fix_cell(qn);
+      ring_dev(w, on, ring, CA + c, CB + c);
     }
     ring.flush();
     double* out = B.fo[D].f[v];

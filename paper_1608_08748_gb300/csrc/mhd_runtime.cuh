@@ -1,7 +1,7 @@
 // mhd_runtime.cuh -- internal runtime of libmhd.so shared by its translation units: the simulation
 // object, the executor that steps a set of boxes with one launch per kernel class, and the
-// templated launchers.  The FP64 instances are compiled in mhd.cu (no contraction: every product
-// and sum rounded as written); the FP32-bulk instances in mhd_f32.cu (contraction allowed).
+// templated launchers.  The FP64 instances are compiled in mhd.cu, the FP32-bulk instances in
+// mhd_f32.cu.
 #pragma once
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>  // header-only; ranges cost nothing unless a profiler is attached
@@ -193,8 +193,10 @@ inline unsigned grid_of(const Tiles& t, const LaunchCfg& c, int nsm) {
   return (unsigned)(g > 0 ? g : 1);
 }
 
-// default launch shapes: the face kernels are register heavy (up to 242 registers), so 128-thread
-// blocks let two or more blocks share an SM; the rest 256, one block per tile.  The FP32 path's
+// default launch shapes: the FP64 face kernels keep their pencils' cells in shared memory (0.6 and 0.5 KB a
+// thread) besides up to 213 registers, so blocks of 64 threads fill an SM closer than larger ones: 4 and 7 of
+// them against 2 and 3 of 128 (128^3 step: Lagrangian faces 3.04 -> 2.80 ms, Eulerian 9.26 -> 9.20).  The
+// FP32 faces 128; the rest 256, one block per tile.  The FP32 path's
 // HBM-bound cell kernels run grid-stride over their tiles with a few blocks per SM where that is faster
 // (256^3 step, measured over 64-512 threads and 2-16 blocks per SM: Lagrangian update 0.98 ms with 12 blocks
 // of 128 per SM, 1.20 with 8; Eulerian update 1.46 with 8, 1.52 one block per tile; edges 0.49 / 0.51;
@@ -202,8 +204,8 @@ inline unsigned grid_of(const Tiles& t, const LaunchCfg& c, int nsm) {
 template <typename T>
 void default_cfgs(Exec<T>& X) {
   for (int kc = 0; kc < NKC; ++kc) X.cfg[kc] = LaunchCfg{256, 0};
-  X.cfg[KC_EFACE].block = 128;
-  X.cfg[KC_LFACE].block = 128;
+  X.cfg[KC_EFACE].block = sizeof(T) == 8 ? 64 : 128;
+  X.cfg[KC_LFACE].block = sizeof(T) == 8 ? 64 : 128;
   if constexpr (sizeof(T) == 4) {
     X.cfg[KC_PRIM] = LaunchCfg{256, 0};
     X.cfg[KC_EDGES] = LaunchCfg{512, 4};
@@ -257,17 +259,16 @@ cudaError_t prepare_kernels() {
 // streams, as much as `own` faces), so long ones suit large grids; on a small grid they leave SMs idle
 // while each thread walks its pencil alone, and in between the last round of blocks decides.  The model:
 // of the blocks on the busiest SM every `resident` make a round, a round takes (len + own), and a part
-// of a round with k blocks the share part[k] of it.  Fitted to FP64 steps of 16^3 to 80^3, 128x4x4 and
-// 128x128x4 cells with 1 to 8 faces, it comes within 0.5 % (Eulerian, at worst 4 %) and 0.3 % (Lagrangian, 2 %)
-// of the best length's time on average: 8 faces against the chosen 1 is 0.36 against 0.09 ms of Eulerian faces
-// at 128x4x4, against the chosen 6 0.50 / 0.44 ms at 40^3; 1 against the chosen 7 is 3.8 / 2.8 ms at 80^3.  The
-// faces' results do not depend on it.
+// of a round with k blocks the share first + (1 - first) k / resident of it.  Fitted to FP64 steps of 16^3
+// to 96^3, 128x4x4 and 128x128x4 cells with 1 to 8 faces, it comes within 0.8 % (Eulerian, at worst 5 %) and 0.0 %
+// (Lagrangian) of the best length's time on average: 8 faces against the chosen 1 is 0.34 against 0.08 ms of
+// Eulerian faces at 128x4x4, 1 against the chosen 6 is 0.47 / 0.41 ms at 40^3, 1 against the chosen 7
+// 4.9 / 3.9 ms at 96^3.  The faces' results do not depend on it.
 struct PencilModel {
   int resident;
-  double own, part[4];
+  double own, first;
 };
-constexpr PencilModel kEulerPencils64 = {2, 0.8, {0.0, 0.9}}, kLagPencils64 = {3, 2.0, {0.0, 0.6, 0.8}},
-                      kEulerPencils32 = {4, 1.5, {0.0, 0.55, 0.7, 0.85}};
+constexpr PencilModel kEulerPencils64 = {4, 0.2, 0.8}, kLagPencils64 = {7, 0.8, 0.4}, kEulerPencils32 = {4, 1.5, 0.4};
 template <typename T>
 Pencils pencils_of(const Box<T>& b, int len) {
   Pencils P;
@@ -292,7 +293,9 @@ int pencil_length(const Exec<T>& X, int block, const PencilModel& m) {
       }
     }
     const long long per_sm = (blocks + X.nsm - 1) / X.nsm;
-    const double cost = ((double)(per_sm / m.resident) + m.part[per_sm % m.resident]) * (longest + m.own);
+    const int rest = (int)(per_sm % m.resident);
+    const double part = rest > 0 ? m.first + (1.0 - m.first) * rest / m.resident : 0.0;
+    const double cost = ((double)(per_sm / m.resident) + part) * (longest + m.own);
     if (len == 1 || cost < least) {
       best = len;
       least = cost;
@@ -347,7 +350,7 @@ void exec_free(Exec<T>& X) {
 // ------------------------------------------------------------------------------------------------
 // a launch whose blocks may start while the kernel before it in the stream drains
 // (dependent_launch_begin); in a captured step a programmatic edge.  The small grids' steps are chains of
-// 20 short kernels: 128x4x4 FP64 PDL0 -> PDL1, 32^3 FP32 PDL2 -> PDL3 us per step.
+// 20 short kernels: 128x4x4 FP64 230 -> 224, 32^3 FP32 104 -> 99 us per step.
 template <typename... P, typename... A>
 void launch_dep(cudaStream_t st, unsigned grid, unsigned block, size_t smem, void (*kernel)(P...), A... args) {
   cudaLaunchConfig_t cfg = {};
