@@ -360,6 +360,18 @@ __device__ __forceinline__ long long& pencil_word(int k) {
   return reinterpret_cast<long long*>(pencil_smem_raw)[k * blockDim.x + threadIdx.x];
 }
 
+// The element at an unsigned 32-bit byte offset: one add to a base that all threads share instead of an index
+// widened and scaled for each access (FP32 256^3 step: Lagrangian faces 3.25 -> 3.14 ms).  4 GiB of one field
+// are 2^29 cells (2^30 in FP32), whose fields together, 330 bytes a cell and more, no device holds.
+template <typename T>
+__device__ __forceinline__ T& at_byte(T* p, unsigned byte) {
+  return *reinterpret_cast<T*>(reinterpret_cast<char*>(p) + byte);
+}
+template <typename T>
+__device__ __forceinline__ const T& at_byte(const T* p, unsigned byte) {
+  return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(p) + byte);
+}
+
 // The fluxes of one Eulerian face f of direction D from its Riemann solution q* = (V_n, V_t1, V_t2,
 // B_t1, B_t2, P) and the face field B_n (the non-advective parts of Sec. 2, reading A12), and the
 // two EMF contributions E = B x U of Sec. 2.5.
@@ -856,13 +868,14 @@ __device__ __forceinline__ void lag_face(const Box<T>& B, int D, idx_t t) {
   // the upwind average as q + kA A + kB B on either side
   const T kA = o0 == 0 ? kc.p : -kc.r, kB = o0 == 0 ? kc.r : -kc.p;
   const int nv = B.nv;
-  idx_t st[5];
+  unsigned st[5];
 #pragma unroll
-  for (int o = 0; o < 5; ++o) st[o] = o0 == 0 ? cell[o] : cell[o + 1];
+  for (int o = 0; o < 5; ++o) st[o] = (unsigned)(o0 == 0 ? cell[o] : cell[o + 1]) * (unsigned)sizeof(T);
+  const unsigned fb = (unsigned)f * (unsigned)sizeof(T);
   auto flux = [&](const T* u, int v) {
-    const T qc = u[st[2]];
-    const Dev<T> P = dev_of(u[st[0]], u[st[1]], qc, u[st[3]], u[st[4]]);
-    B.fo[D].f[v][f] = vn * fma(kB, P.B, fma(kA, P.A, qc));
+    const T qc = at_byte(u, st[2]);
+    const Dev<T> P = dev_of(at_byte(u, st[0]), at_byte(u, st[1]), qc, at_byte(u, st[3]), at_byte(u, st[4]));
+    at_byte(B.fo[D].f[v], fb) = vn * fma(kB, P.B, fma(kA, P.A, qc));
   };
 #pragma unroll
   for (int v = 0; v < 7; ++v) {
