@@ -844,13 +844,14 @@ template <typename T>
 struct AvgCoef {
   T p, r;
 };
+// The factor of A and B goes into y as its square root k: (k - k y)^2 and (k y)(k - k y); y k comes from
+// tau k / h, formed once per thread (avg_scale).
 template <typename T>
-__device__ __forceinline__ AvgCoef<T> avg_coef(T y) {
-  const T u = sub_t(in_register(T(1)), y);
-  T hu;
-  if constexpr (sizeof(T) == 8) hu = mul_t(u, in_register(1.0 / 6.0));
-  else hu = scale_down_b<1>(u);
-  return AvgCoef<T>{mul_t(y, hu), mul_t(u, hu)};
+__device__ __forceinline__ T avg_scale() { return sizeof(T) == 8 ? T(0.40824829046386301637) : T(0.70710678118654752440); }
+template <typename T>
+__device__ __forceinline__ AvgCoef<T> avg_coef(T yk) {
+  const T v = sub_t(in_register(avg_scale<T>()), yk);
+  return AvgCoef<T>{mul_t(yk, v), mul_t(v, v)};
 }
 // the average next to the right edge of a cell less the cell's value, and the average next to the left
 // edge of a cell of value d
@@ -858,6 +859,13 @@ template <typename T>
 __device__ __forceinline__ T inc_right(Dev<T> P, AvgCoef<T> k) { return fma(k.r, P.B, mul_t(k.p, P.A)); }
 template <typename T>
 __device__ __forceinline__ T inc_left(T d, Dev<T> P, AvgCoef<T> k) { return fma(-k.r, P.A, fma(-k.p, P.B, d)); }
+// a row times four averages of inc_right: applied to A and B first, which leaves one average (10 instructions
+// instead of 12; for inc_left, with d as a third, it would be 14)
+template <typename T>
+__device__ __forceinline__ T row_right(T a, Dev<T> P, T b, Dev<T> Q, T c, Dev<T> R, T d, Dev<T> S, AvgCoef<T> k) {
+  auto dot = [&](T p, T q, T r, T s) { return fma(a, p, fma(b, q, fma(c, r, mul_t(d, s)))); };
+  return inc_right(Dev<T>{dot(P.A, Q.A, R.A, S.A), dot(P.B, Q.B, R.B, S.B)}, k);
+}
 
 // ------------------------------------------------------------------------------------------------
 // Sec. 2.4 + App. A: Roe-type face state, eigenvectors and the characteristic Riemann solution.
@@ -889,7 +897,7 @@ struct FaceSide {
 // is the sum over the averages themselves, at the same count of instructions, and its rounding is that
 // of the differences between the cells, not of their values.
 template <typename T>
-__device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>& r, T Bn, T tau_h, T qs[6]) {
+__device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>& r, T Bn, T tau_k, T qs[6]) {
   const T INV_SQRT2 = T(0.70710678118654752440), HALF = in_register(T(0.5));
   const T iden = rcp_t(add_t(l.w[5], r.w[5]));
   const T al = mul_t(l.w[5], iden), ar = mul_t(r.w[5], iden);  // the normalised weights
@@ -903,10 +911,10 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
   const T irho = mul_t(rs, rs), sqr = mul_t(rho, rs);
   const T gp = mul_t(gam, p);
   const T c2 = mul_t(gp, irho);
-  const T ca2 = mul_t(mul_t(Bn, Bn), irho);
+  const T ca = mul_t(abs_b(Bn), rs), ca2 = mul_t(ca, ca);
   const T bp2 = fma(Bt1, Bt1, mul_t(Bt2, Bt2));
   const T b2 = mul_t(bp2, irho);  // b_perp^2
-  const T s = add_t(add_t(c2, ca2), b2), Z = sub_t(sub_t(c2, ca2), b2);
+  const T ab2 = add_t(ca2, b2), s = add_t(c2, ab2), Z = sub_t(c2, ab2);
   const T sq2 = fma(Z, Z, mul_t(b2, four_b(c2)));
   // the directions of B_perp; the degenerate case keeps |B_perp| itself
   T by = INV_SQRT2, bz = INV_SQRT2, bper;
@@ -918,7 +926,7 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
   } else {
     bper = sqrt_t(bp2);
   }
-  const T rc = rsqrt_n(c2), c = mul_t(c2, rc);
+  const T rc = rsqrt_n(c2), c = mul_t(c2, rc), crs = mul_t(c, rs);
   T sq = T(0), af = INV_SQRT2, as = INV_SQRT2;
   {
     const T isq = rsqrt_n(sq2), sqn = mul_t(sq2, isq);
@@ -926,7 +934,7 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
       sq = sqn;
       const T big2 = fma(half_nn(abs_b(Z)), isq, HALF);  // in [1/2, 1]
       const T rb = rsqrt_n(big2), big = mul_t(big2, rb);
-      const T small = mul_t(mul_t(mul_t(c, bper), mul_t(rs, isq)), rb);
+      const T small = mul_t(mul_t(crs, bper), mul_t(isq, rb));
       const bool fast = !sign_bit_b(Z);
       af = fast ? big : small;
       as = fast ? small : big;
@@ -934,12 +942,12 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
   }
   const T cf2 = half_nn(add_t(s, sq));
   const T rcf = rsqrt_n(cf2);
-  const T cf = mul_t(cf2, rcf), ca = mul_t(abs_b(Bn), rs);
+  const T cf = mul_t(cf2, rcf);
   const T cs = mul_t(mul_t(c, ca), rcf);
   const bool neg = sign_bit_b(Bn) && gt_nn(abs_b(Bn), T(0));  // sign(0) = +1
   const T bys = neg ? neg_b(by) : by, bzs = neg ? neg_b(bz) : bz;
 
-  const AvgCoef<T> ka = avg_coef(mul_t(ca, tau_h)), kf = avg_coef(mul_t(cf, tau_h)), ks = avg_coef(mul_t(cs, tau_h));
+  const AvgCoef<T> ka = avg_coef(mul_t(ca, tau_k)), kf = avg_coef(mul_t(cf, tau_k)), ks = avg_coef(mul_t(cs, tau_k));
 
   // the right cell's values less the left cell's
   T d[6];
@@ -950,21 +958,19 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
   // beyond their components along B_perp
   T hv, hb;
   {
-    T ql[5], qr[5];
+    const T rbz = mul_t(rs, bz), rby = mul_t(rs, by);
+    T qr[5];
 #pragma unroll
-    for (int m = 1; m < 5; ++m) {
-      ql[m] = inc_right(l.P[m], ka);
-      qr[m] = inc_left(d[m], r.P[m], ka);
-    }
-    const T vl = fma(bys, ql[2], -mul_t(bzs, ql[1])), vr = fma(bys, qr[2], -mul_t(bzs, qr[1]));
-    const T bl = fma(bz, ql[3], -mul_t(by, ql[4])), br = fma(bz, qr[3], -mul_t(by, qr[4]));
-    const T sp = fma(rs, bl, vl), sm = fma(-rs, br, vr);
+    for (int m = 1; m < 5; ++m) qr[m] = inc_left(d[m], r.P[m], ka);
+    const T sp = row_right(bys, l.P[2], -bzs, l.P[1], rbz, l.P[3], -rby, l.P[4], ka);
+    const T sm = fma(bys, qr[2], fma(-bzs, qr[1], fma(-rbz, qr[3], mul_t(rby, qr[4]))));
     hv = scale_down_b<1>(add_t(sp, sm));
     hb = mul_t(half_nn(sqr), sub_t(sp, sm));
   }
-  // the magnetosonic waves on (v_n, v_par sgn(B_n), B_par, p): the +c_f wave has
-  // L = (lf, -ls, as i2sc, af i2r), R = (af cf, -as cs, as sc, af gp), the +c_s wave
-  // L = (ls, lf, -af i2sc, as i2r), R = (as cs, af cf, -af sc, as gp)
+  // the magnetosonic waves on (v_n, v_par sgn(B_n), B_par, p): with the rows times 2 c^2 and the columns
+  // divided by it, the +c_f wave has L = (af cf, -as cs, as c / sqrt(rho), af / rho), R = (lf, -ls,
+  // as sqrt(rho) / 2c, af rho / 2), the +c_s wave L = (as cs, af cf, -af c / sqrt(rho), as / rho),
+  // R = (ls, lf, -af sqrt(rho) / 2c, as rho / 2)
   auto along = [&](T a, T b) { return fma(by, a, mul_t(bz, b)); };
   auto along_s = [&](T a, T b) { return fma(bys, a, mul_t(bzs, b)); };
   const Dev<T> lv = {along_s(l.P[1].A, l.P[2].A), along_s(l.P[1].B, l.P[2].B)};
@@ -973,27 +979,26 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
   const Dev<T> rb = {along(r.P[3].A, r.P[4].A), along(r.P[3].B, r.P[4].B)};
   const T dv = along_s(d[1], d[2]), db = along(d[3], d[4]);
   const T af_cf = mul_t(af, cf), as_cs = mul_t(as, cs);
-  const T hrc = half_nn(rc), i2c2 = mul_t(hrc, rc), i2sc = mul_t(rs, hrc), i2r = mul_t(i2c2, irho);
+  const T hrc = half_nn(rc), i2c2 = mul_t(hrc, rc);
   const T lf = mul_t(af_cf, i2c2), ls = mul_t(as_cs, i2c2);
   auto pair = [&](AvgCoef<T> k, T l0, T l1, T l2, T l3, T& dif, T& sum) {
-    const T sp = fma(l0, inc_right(l.P[0], k),
-                     fma(l1, inc_right(lv, k), fma(l2, inc_right(lb, k), mul_t(l3, inc_right(l.P[5], k)))));
+    const T sp = row_right(l0, l.P[0], l1, lv, l2, lb, l3, l.P[5], k);
     const T sm = fma(-l0, inc_left(d[0], r.P[0], k),
                      fma(-l1, inc_left(dv, rv, k), fma(l2, inc_left(db, rb, k), mul_t(l3, inc_left(d[5], r.P[5], k)))));
     dif = sub_t(sp, sm);
     sum = add_t(sp, sm);
   };
   T difF, sumF, difS, sumS;
-  pair(kf, lf, -ls, mul_t(as, i2sc), mul_t(af, i2r), difF, sumF);
-  pair(ks, ls, lf, -mul_t(af, i2sc), mul_t(as, i2r), difS, sumS);
-  const T vpar = fma(af_cf, difS, -mul_t(as_cs, difF));
-  const T bpar = mul_t(mul_t(sqr, c), fma(as, sumF, -mul_t(af, sumS)));
-  qs[0] = fma(af_cf, difF, fma(as_cs, difS, l.q[0]));
+  pair(kf, af_cf, -as_cs, mul_t(as, crs), mul_t(af, irho), difF, sumF);
+  pair(ks, as_cs, af_cf, -mul_t(af, crs), mul_t(as, irho), difS, sumS);
+  const T vpar = fma(lf, difS, -mul_t(ls, difF));
+  const T bpar = mul_t(mul_t(sqr, hrc), fma(as, sumF, -mul_t(af, sumS)));
+  qs[0] = fma(lf, difF, fma(ls, difS, l.q[0]));
   qs[1] = fma(bys, vpar, fma(-bzs, hv, l.q[1]));
   qs[2] = fma(bzs, vpar, fma(bys, hv, l.q[2]));
   qs[3] = fma(by, bpar, fma(bz, hb, l.q[3]));
   qs[4] = fma(bz, bpar, fma(-by, hb, l.q[4]));
-  qs[5] = fma(gp, fma(af, sumF, mul_t(as, sumS)), l.q[5]);
+  qs[5] = fma(half_nn(rho), fma(af, sumF, mul_t(as, sumS)), l.q[5]);
 }
 // the same from parabolas in the paper's form, whose values are L + A/2 with A = Delta q + q6/3 and
 // B = Delta q - q6/3
@@ -1012,7 +1017,7 @@ __device__ __forceinline__ void riemann(const T wl[6], const T wr[6], T Bn, cons
     return f;
   };
   FaceSide<T> l = side(wl, pl), r = side(wr, pr);
-  riemann(l, r, Bn, tau_h, qs);
+  riemann(l, r, Bn, tau_h * avg_scale<T>(), qs);
 }
 
 // ------------------------------------------------------------------------------------------------

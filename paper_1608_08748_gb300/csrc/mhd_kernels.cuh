@@ -379,8 +379,8 @@ template <typename T>
 __device__ __forceinline__ void store_face_fluxes(const FaceOut<T>& fo, idx_t f, T Bn, const T qs[6]) {
   const T Vn = qs[0], Vt1 = qs[1], Vt2 = qs[2], Bt1 = qs[3], Bt2 = qs[4], P = qs[5];
   const T Bn2 = mul_t(Bn, Bn);
-  const T pstar = fma(T(0.5), fma(Bt1, Bt1, fma(Bt2, Bt2, Bn2)), P);
-  const T Fn = sub_t(pstar, Bn2), F1 = -mul_t(Bn, Bt1), F2 = -mul_t(Bn, Bt2);
+  const T Fn = fma(T(0.5), fma(Bt1, Bt1, fma(Bt2, Bt2, -Bn2)), P);  // p* - B_n^2
+  const T F1 = -mul_t(Bn, Bt1), F2 = -mul_t(Bn, Bt2);
   fo.f[0][f] = Fn;
   fo.f[1][f] = F1;
   fo.f[2][f] = F2;
@@ -407,7 +407,7 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, int D, idx_
   const Geom& g = B.g;
   const Line L = line_of_pencil(B, B.pe, D, p);
   const int f0 = L.f0, nfp = L.nfp;
-  const T tau_h = tau_h_of(B);
+  const T tau_k = mul_t(tau_h_of(B), avg_scale<T>());
   const bool inside = f0 >= 3 && f0 + nfp + 2 <= L.n;
   auto cell_at = [&](int i) -> idx_t {
     if (inside) return MHD_CELL(g, L.base + i * L.stride);
@@ -485,7 +485,7 @@ __device__ __forceinline__ void euler_pencil_window(const Box<T>& B, int D, idx_
       r.w[3] = r.q[3];
       r.w[4] = r.q[4];
       T qs[6];
-      riemann(l, r, Bn, tau_h, qs);
+      riemann(l, r, Bn, tau_k, qs);
       store_face_fluxes(B.fo[D], L.face(g, i), Bn, qs);
       l = r;
     }
@@ -504,7 +504,7 @@ __device__ __forceinline__ void euler_pencil(const Box<double>& B, int D, idx_t 
   const Geom& g = B.g;
   const Line L = line_of_pencil(B, B.pe, D, p);
   const int f0 = L.f0, nfp = live ? L.nfp : 0;
-  const double tau_h = tau_h_of(B);
+  const double tau_k = mul_t(tau_h_of(B), avg_scale<double>());
   const double* qv[6] = {B.w.v[D], B.w.v[D1], B.w.v[D2], B.w.B[D1], B.w.B[D2], B.w.p};
   auto cell_at = [&](int i) { return L.cell(g, i); };
   Step4Ring ring(EULER_SLOTS, 6);
@@ -574,7 +574,7 @@ __device__ __forceinline__ void euler_pencil(const Box<double>& B, int D, idx_t 
       r.w[5] = B.w.sr[cr];
       const double Bn = B.s.b[D][cr];
       double qs[6];
-      riemann(l, r, Bn, tau_h, qs);
+      riemann(l, r, Bn, tau_k, qs);
       store_face_fluxes(B.fo[D], L.face(g, i), Bn, qs);
     }
 #pragma unroll
@@ -841,7 +841,7 @@ __device__ __forceinline__ void lag_face(const Box<T>& B, int D, idx_t t) {
   const FastDiv d0 = D == 0 ? g.dn1[0] : g.dn[0], d1 = D == 1 ? g.dn1[1] : g.dn[1];
   const unsigned r0 = fdiv((unsigned)t, d0);
   const int i = (int)((unsigned)t - r0 * d0.d), k = (int)fdiv(r0, d1), j = (int)(r0 - (unsigned)k * d1.d);
-  const T tau_h = tau_h_of(B);
+  const T tau_k = mul_t(tau_h_of(B), avg_scale<T>());
   const int nx = g.n[0], ny = g.n[1], n = g.n[D];
   const int a = D == 0 ? i : D == 1 ? j : k;
   const idx_t stride = D == 0 ? 1 : (D == 1 ? nx : nx * ny);
@@ -861,7 +861,7 @@ __device__ __forceinline__ void lag_face(const Box<T>& B, int D, idx_t t) {
   T rl = B.s.rho[cl], rr = B.s.rho[cr];
   T isl = rsqrt_t(rl), isr = rsqrt_t(rr);
   const T vn = mul_t(fma(B.s.m[D][cr], isr, mul_t(B.s.m[D][cl], isl)), rcp_t(fma(rr, isr, mul_t(rl, isl))));
-  const AvgCoef<T> kc = avg_coef(mul_t(abs_b(vn), tau_h));
+  const AvgCoef<T> kc = avg_coef(mul_t(abs_b(vn), tau_k));
   const T* q[7] = {B.s.rho, B.s.m[0], B.s.m[1], B.s.m[2], B.s.E, B.s.eint, B.s.rh2};
   const idx_t f = fidx(g, i, j, k);
   const int o0 = vn >= T(0) ? 0 : 1;  // upwind cell: stencil cells o0 .. o0 + 4
@@ -912,7 +912,7 @@ __device__ __forceinline__ void lag_pencil(const Box<double>& B, int D, idx_t p,
   const Geom& g = B.g;
   const Line L = line_of_pencil(B, B.pl, D, p);
   const int f0 = L.f0, nfp = live ? L.nfp : 0;
-  const double tau_h = tau_h_of(B);
+  const double tau_k = mul_t(tau_h_of(B), avg_scale<double>());
   auto cell_at = [&](int i) { return L.cell(g, i); };
   constexpr int VN = 0, KP = LAG_FACES, KR = 2 * LAG_FACES, CA = 3 * LAG_FACES, CB = CA + LAG_CELLS, CQ = CB + LAG_CELLS;
   Step4Ring ring(LAG_SLOTS, LAG_CELLS);
@@ -936,7 +936,7 @@ __device__ __forceinline__ void lag_pencil(const Box<double>& B, int D, idx_t p,
     const double vn = mul_t(add_t(al, ar), rcp_t(add_t(bl, br)));
     al = ar;
     bl = br;
-    const AvgCoef<double> kc = avg_coef(mul_t(abs_b(vn), tau_h));
+    const AvgCoef<double> kc = avg_coef(mul_t(abs_b(vn), tau_k));
     pencil_slot(VN + k) = vn;
     pencil_slot(KP + k) = kc.p;
     pencil_slot(KR + k) = kc.r;
