@@ -723,14 +723,15 @@ struct FixStep4 {
   long long num, s0, h3, ql, qr;  // (ql, qr) = q_{-1}, q_{+1}
   int E;
 };
-// Steps 1 and 2 of the cell in the middle of q_{-2} .. q_{+2}: 3 A and 3 B.  All is done with the sign of
+// Steps 1 and 2 of the cell in the middle of q_{-2} .. q_{+2}: 3 A and 3 B (left: q_0 - q_{-1}, for the
+// Riemann solve).  All is done with the sign of
 // q_0 - q_{-1} taken off: where q_{+1} - q_0 is then negative the cell is an extremum, and else the
 // cell's own slope and A and B are not negative, and a neighbour's slope counts only where it is not.  Returns
 // whether Step 4 may act (never false where it does): D- >= 0 >= D+, and by the high words |num| > 3 |s0| / 20
 // and |s0| > mn / 128.  A wide stencil, where the largest exponent is more than 5 above that of the cell and of one
 // of its neighbours (the results are at most a few times the smaller of the two differences, so the cut
 // would show), or with an infinity or a NaN, is done as a whole in FP64.
-__device__ __forceinline__ bool fix_dev(const FixCell c[5], Dev<double>& P, FixStep4& st) {
+__device__ __forceinline__ bool fix_dev(const FixCell c[5], Dev<double>& P, double& left, FixStep4& st) {
   const int near = max_i(c[2].e, min_i(c[1].e, c[3].e));
   const int E = max_i(max_i(max_i(c[0].e, c[1].e), max_i(c[3].e, c[4].e)), c[2].e);
   const bool wide = E > near + 5 || E == 0x7ff;
@@ -748,6 +749,7 @@ __device__ __forceinline__ bool fix_dev(const FixCell c[5], Dev<double>& P, FixS
   const bool mono = d[2] >= 0;
   P.A = fix_to_double(mono ? mA : 0, neg, E);
   P.B = fix_to_double(mono ? mB : 0, neg, E);
+  left = fix_to_double((unsigned long long)d[1], neg, E);
   const long long Dm = d[1] - d[0], Dp = d[2] - d[3];  // D- and -D+
   st = FixStep4{Dm + Dp, d[1] + d[2], 3 * h0, q[1], q[3], E};
   const int ml = hi_word(q[1]), mr = hi_word(q[3]);
@@ -758,6 +760,7 @@ __device__ __forceinline__ bool fix_dev(const FixCell c[5], Dev<double>& P, FixS
   if (wide) {
     const Dev<double> W = dev_of(fix_value(c[0]), fix_value(c[1]), fix_value(c[2]), fix_value(c[3]), fix_value(c[4]));
     P = Dev<double>{mul_t(3.0, W.A), mul_t(3.0, W.B)};
+    left = sub_t(fix_value(c[2]), fix_value(c[1]));
     return false;
   }
   return cand;
@@ -766,22 +769,25 @@ __device__ __forceinline__ long long fix_min_abs(const FixStep4& st) {
   const unsigned long long l = uabs64(st.ql), r = uabs64(st.qr);
   return (long long)(l < r ? l : r);
 }
-// Step 4's blend from there (the integers convert on the FP64 pipe, once per 32 gathered cells): hbar =
+// Step 4's blend from there (converted on the integer pipes, where a conversion on the FP64 pipe would cost it
+// an instruction: 128^3 step 13.7 -> 13.6 ms): hbar =
 // (20/3) num / s0 - 1 clamped to [0, 1], 3 A += hbar (3 h - 3 A).
 __device__ __forceinline__ Dev<double> fix_step4(Dev<double> P, long long n, long long s, long long h3, long long mn,
                                                  int E) {
-  const double num = (double)n, s0 = (double)s;
+  const double num = fix_to_double((unsigned long long)n, 0, 1081), s0 = fix_to_double((unsigned long long)s, 0, 1081);
   double hb = fma(mul_t(in_register(20.0 / 3.0), num), rcp_nr(s0), -in_register(1.0));
   hb = min_nn(hb, 1.0);
-  if (sign_bit_b(hb) || !gt_nn(s0, mul_t(in_register(0.01), (double)mn))) hb = 0.0;
+  // |s0| > mn / 100 exactly: from 2^53 on 100 |s0| is above 2^59, the bound of mn
+  if (sign_bit_b(hb) || !(s >= (1ll << 53) || 100 * s > mn)) hb = 0.0;
   const double h = with_sign_b(fix_to_double((unsigned long long)h3, 0, E), P.A);  // A = 0: h = 0
   return Dev<double>{fma(hb, sub_t(h, P.A), P.A), fma(hb, sub_t(h, P.B), P.B)};
 }
 // the deviations of the cell in the middle of five values, by the same steps
 __device__ __forceinline__ Dev<double> fix_dev_of(const FixCell c[5]) {
   Dev<double> P;
+  double left;
   FixStep4 st;
-  if (fix_dev(c, P, st)) P = fix_step4(P, st.num, st.s0, st.h3, fix_min_abs(st), st.E);
+  if (fix_dev(c, P, left, st)) P = fix_step4(P, st.num, st.s0, st.h3, fix_min_abs(st), st.E);
   return Dev<double>{P.A * (1.0 / 3.0), P.B * (1.0 / 3.0)};
 }
 
@@ -896,8 +902,9 @@ struct FaceSide {
 // All waves act on the averages less the left cell's values q_l, and q* = q_l + sum R s: with R L = I that
 // is the sum over the averages themselves, at the same count of instructions, and its rounding is that
 // of the differences between the cells, not of their values.
+// d: the right cell's values less the left cell's
 template <typename T>
-__device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>& r, T Bn, T tau_k, T qs[6]) {
+__device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>& r, const T d[6], T Bn, T tau_k, T qs[6]) {
   const T INV_SQRT2 = T(0.70710678118654752440), HALF = in_register(T(0.5));
   const T iden = rcp_t(add_t(l.w[5], r.w[5]));
   const T al = mul_t(l.w[5], iden), ar = mul_t(r.w[5], iden);  // the normalised weights
@@ -949,10 +956,6 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
 
   const AvgCoef<T> ka = avg_coef(mul_t(ca, tau_k)), kf = avg_coef(mul_t(cf, tau_k)), ks = avg_coef(mul_t(cs, tau_k));
 
-  // the right cell's values less the left cell's
-  T d[6];
-#pragma unroll
-  for (int m = 0; m < 6; ++m) d[m] = sub_t(r.q[m], l.q[m]);
   // the Alfven waves, on the components across B_perp: v = -bz v_t1 + by v_t2 (times sgn(B_n)),
   // b = (bz B_t1 - by B_t2) / sqrt(rho); first, so that the tangential coefficients are not needed
   // beyond their components along B_perp
@@ -999,6 +1002,13 @@ __device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>&
   qs[3] = fma(by, bpar, fma(bz, hb, l.q[3]));
   qs[4] = fma(bz, bpar, fma(-by, hb, l.q[4]));
   qs[5] = fma(half_nn(rho), fma(af, sumF, mul_t(as, sumS)), l.q[5]);
+}
+template <typename T>
+__device__ __forceinline__ void riemann(const FaceSide<T>& l, const FaceSide<T>& r, T Bn, T tau_k, T qs[6]) {
+  T d[6];
+#pragma unroll
+  for (int m = 0; m < 6; ++m) d[m] = sub_t(r.q[m], l.q[m]);
+  riemann(l, r, d, Bn, tau_k, qs);
 }
 // the same from parabolas in the paper's form, whose values are L + A/2 with A = Delta q + q6/3 and
 // B = Delta q - q6/3

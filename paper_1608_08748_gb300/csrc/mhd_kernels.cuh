@@ -342,20 +342,23 @@ constexpr size_t pencil_smem_bytes(int slots, int block) {
   return (size_t)slots * block * sizeof(double) + (size_t)(block / 32) * Step4Ring::BYTES;
 }
 // the deviations of the middle cell of c (live: this lane has one): Steps 1 and 2 at once, into the slots,
-// Step 4 into the ring
-__device__ __forceinline__ void ring_dev(const FixCell c[5], bool live, Step4Ring& ring, int slotA, int slotB) {
+// Step 4 into the ring; returns q_0 - q_{-1}
+__device__ __forceinline__ double ring_dev(const FixCell c[5], bool live, Step4Ring& ring, int slotA, int slotB) {
   Dev<double> P;
+  double left;
   FixStep4 st;
-  const bool cand = fix_dev(c, P, st);
+  const bool cand = fix_dev(c, P, left, st);
   pencil_slot(slotA) = P.A;
   pencil_slot(slotB) = P.B;
   ring.push(live && cand, slotA, st);
+  return left;
 }
 
 // The FP64 Eulerian pencils keep of each primitive v the last cells in rings of slots: the values of four
 // (10 v .. 10 v + 3), the integers of five (10 v + 4 .. 10 v + 8) and their exponents, 11 bits each, in one
-// word (10 v + 9); the new cell's deviations in the slots 60 + v (A) and 66 + v (B).
-constexpr int EULER_SLOTS = 10 * 6 + 12;
+// word (10 v + 9); the new cell's deviations in the slots 60 + v (A) and 66 + v (B), its value less the cell's on
+// its left in 72 + v (from the integers, which the integer pipes have time for: 128^3 step 13.9 -> 13.7 ms).
+constexpr int EULER_SLOTS = 10 * 6 + 18;
 __device__ __forceinline__ long long& pencil_word(int k) {
   return reinterpret_cast<long long*>(pencil_smem_raw)[k * blockDim.x + threadIdx.x];
 }
@@ -548,7 +551,7 @@ __device__ __forceinline__ void euler_pencil(const Box<double>& B, int D, idx_t 
       pencil_slot(10 * v + w4) = q;
       pencil_word(10 * v + 4 + w5[4]) = c[4].n;
       pencil_word(10 * v + 9) = es;
-      ring_dev(c, on, ring, 60 + v, 66 + v);
+      pencil_slot(72 + v) = ring_dev(c, on, ring, 60 + v, 66 + v);
     }
     ring.flush();
 #pragma unroll
@@ -573,8 +576,10 @@ __device__ __forceinline__ void euler_pencil(const Box<double>& B, int D, idx_t 
       r.w[4] = r.q[4];
       r.w[5] = B.w.sr[cr];
       const double Bn = B.s.b[D][cr];
-      double qs[6];
-      riemann(l, r, Bn, tau_k, qs);
+      double d[6], qs[6];
+#pragma unroll
+      for (int v = 0; v < 6; ++v) d[v] = pencil_slot(72 + v);
+      riemann(l, r, d, Bn, tau_k, qs);
       store_face_fluxes(B.fo[D], L.face(g, i), Bn, qs);
     }
 #pragma unroll

@@ -57,12 +57,13 @@ int main() {
     int top = 0;
     for (int i = 0; i < 5; ++i) top = std::max(top, c[i].e);
     Dev<double> P;
+    double left;
     FixStep4 st;
-    const bool cand = fix_dev(c, P, st);
+    const bool cand = fix_dev(c, P, left, st);
     if (top > std::max(c[2].e, std::min(c[1].e, c[3].e)) + 5) {  // as a whole in FP64
       const Dev<double> W = dev_of(q[0], q[1], q[2], q[3], q[4]);
       ++wide;
-      wide_bad += cand || P.A != 3 * W.A || P.B != 3 * W.B;
+      wide_bad += cand || P.A != 3 * W.A || P.B != 3 * W.B || left != q[2] - q[1];
       continue;
     }
     const Q u = std::ldexp(1.0, top - 1081);
@@ -78,6 +79,7 @@ int main() {
     const Q Dp = d3 - d2, Dm = d1 - d0, s0 = d1 + d2, mn = std::min(mag(q[1]), mag(q[3]));
     if (mag(mag(s0) - mn / 100) < 1e-9 * mn || (Dp != 0 && mag(Dp) < 8 * u) || (Dm != 0 && mag(Dm) < 8 * u)) continue;
     ++n;
+    bad += !(mag(left - d1) <= u + (Q)std::ldexp(1.0, -53) * mag(d1));
     Q hb = 0;
     if (mag(s0) > mn / 100 && Dp * Dm <= 0) {
       hb = (Q)20 / 3 * (Dm - Dp) / s0 - 1;
@@ -100,9 +102,10 @@ int main() {
     FixCell c[5];
     for (int j = 0; j < 5; ++j) c[j] = fix_cell(2 + std::sin(2 * M_PI * (i * 0.37 + j) / 40));
     Dev<double> P;
+    double left;
     FixStep4 st;
     ++smooth;
-    kept += fix_dev(c, P, st);
+    kept += fix_dev(c, P, left, st);
   }
   // infinities and NaNs go the FP64 way; constants give exactly 0, ramps of exact steps exactly their step
   const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
@@ -121,9 +124,10 @@ int main() {
     FixCell c[5], r[5];
     for (int i = 0; i < 5; ++i) c[i] = fix_cell(x), r[i] = fix_cell(-1.75 + 0.5 * i);
     Dev<double> P, R;
+    double left;
     FixStep4 st;
-    special += fix_dev(c, P, st) || P.A != 0 || P.B != 0;
-    special += fix_dev(r, R, st) || R.A != 1.5 || R.B != 1.5;
+    special += fix_dev(c, P, left, st) || P.A != 0 || P.B != 0;
+    special += fix_dev(r, R, left, st) || R.A != 1.5 || R.B != 1.5;
   }
   std::printf("%ld %ld %ld %ld %ld %ld %ld %ld %ld\n", n, acts, bad, missed, wide, wide_bad, smooth, kept, special);
 }
