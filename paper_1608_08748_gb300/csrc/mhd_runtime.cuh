@@ -200,7 +200,11 @@ inline unsigned grid_of(const Tiles& t, const LaunchCfg& c, int nsm) {
 // HBM-bound cell kernels run grid-stride over their tiles with a few blocks per SM where that is faster
 // (256^3 step, measured over 64-512 threads and 2-16 blocks per SM: Lagrangian update 0.98 ms with 12 blocks
 // of 128 per SM, 1.20 with 8; Eulerian update 1.46 with 8, 1.52 one block per tile; edges 0.49 / 0.51;
-// post stage 0.93 / 0.95; primitives 0.53 ms one block per tile, 0.60 with 4 blocks of 512).
+// post stage 0.93 / 0.95; primitives 0.53 ms one block per tile, 0.60 with 4 blocks of 512).  The instances over
+// many boxes take more registers (64 against 40 in the Lagrangian update, so 8 blocks of 128 fill an SM, and 12
+// would leave a half-empty round) and a search for the box of each tile, which a grid-stride block shares
+// (32 boxes of 32^3 to 96^3: Lagrangian update 0.65 ms with 8 blocks, 0.86 with 12; primitives 0.296 with 8 blocks
+// of 256, 0.326 one block per tile).
 template <typename T>
 void default_cfgs(Exec<T>& X) {
   for (int kc = 0; kc < NKC; ++kc) X.cfg[kc] = LaunchCfg{256, 0};
@@ -212,6 +216,10 @@ void default_cfgs(Exec<T>& X) {
     X.cfg[KC_EUPD] = LaunchCfg{128, 8};
     X.cfg[KC_LUPD] = LaunchCfg{128, 12};
     X.cfg[KC_POST] = LaunchCfg{128, 8};
+    if (X.nb > 1) {
+      X.cfg[KC_PRIM] = LaunchCfg{256, 8};
+      X.cfg[KC_LUPD] = LaunchCfg{128, 8};
+    }
   }
 }
 
