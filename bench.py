@@ -43,22 +43,21 @@ BYTES_PER_CELL_UPDATE = {8: 1032, 4: 516}
 # the copy bandwidth used when the measured peaks are not available
 HBM_FALLBACK_GBS = 6800.0
 # algorithmic FP64 flops of one Eulerian face, counted from the kernel source with an FMA as two
-# flops and a division, square root or reciprocal square root as one (compares and selects not
-# counted): the parabolas of the six primitives of one new cell, streamed along the pencil (6 x 32:
-# differences, halved slope, edge value and second difference 11, Steps 2-5 18, the Step 4 test 3),
-# the Riemann solve (Roe average, speeds and eigenvector rows 116; the three wave pairs'
-# domain-of-dependence averages with L q and R s 244) and the fluxes (25)
-FLOPS_PER_EULER_FACE = 577
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one Eulerian face launch at 128^3,
-# the mean of the x, y and z launches of one ncu capture of this kernel (358.1, 256.2, 260.9 MB;
+# flops and a division, square root or reciprocal square root as one (compares, selects and exact
+# scalings by powers of two not counted): the Riemann solve 270 (Roe state 19, speeds and alphas 41,
+# the averages' coefficients 12, Alfven waves 45, components along B_perp 30, magnetosonic rows and
+# sums 98, q* 25) and the fluxes 20.  The parabolas run on the integer pipes and are not counted
+# (Step 4's blend, in FP64 on a tenth of them, neither).
+FLOPS_PER_EULER_FACE = 290
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one Eulerian face launch at 128^3, which
+# takes the three directions (550.4 + 360.5 MB, the mean of three launches of one ncu capture;
 # profiles/kb_metrics_turbulence_128_fp64.md; set to None whenever the kernel changes)
-EULER_FACE_TRAFFIC_BYTES = 291.7e6
-# FP32 bulk: FP32 flops of one Eulerian face (fadd + fmul + 2 ffma executed per face, 795-796 in
-# the three directions of one ncu capture of kb_euler_pencil<float> at 128^3) and the DRAM bytes of
-# one 256^3 launch: the mean of the 128^3 capture's x, y, z launches (175.7, 110.0, 114.0 MB) times
-# 8, the ratio of the faces processed (profiles/kb_metrics_turbulence_128_fp32bulk.md)
-FP32_FLOPS_PER_EULER_FACE = 796
-EULER_FACE_TRAFFIC_BYTES_FP32 = 133.2e6 * 8
+EULER_FACE_TRAFFIC_BYTES = 910.9e6
+# FP32 bulk: FP32 flops of one Eulerian face (fadd + fmul + 2 ffma executed per face: 105 + 134 + 2 x 123)
+# and the DRAM bytes of one 256^3 launch (2142 + 1486 MB), both from one ncu capture of
+# kb_euler_pencil<float> at 256^3 (profiles/kb_metrics_turbulence_256_fp32bulk.md)
+FP32_FLOPS_PER_EULER_FACE = 484
+EULER_FACE_TRAFFIC_BYTES_FP32 = 3627.7e6
 
 
 def hbm_peak():
