@@ -1408,6 +1408,9 @@ __device__ __forceinline__ bool chem_cell_pairs(const Phys& ph, const float ts_p
 //   x = log10(T / 1e4); T, k1' and k4 as in chem_cell, from the state after the chemistry update;
 //   the change is limited to at most half of rho eps (the explicit step of a cooling time shorter
 //   than tau would drive rho eps negative).
+// Bound by the FP64 pipe.  f(T) without logarithms, the quotients that stay finite by rcp_nr, the exponentials by
+// exp_tang (its arguments outside +-707, where it takes the library's, are rare): post stage of a 128^3 FP64 step
+// 3.05 -> 2.49 ms, with ions 4.05 -> 3.60 ms; the same worst error against the oracle (2.8e-14).
 template <bool IONS>
 __device__ MHD_NOINLINE double heatcool_delta(const Phys& ph, double rho, double eint, double rh2,
                                                  double rhp, double tau) {
@@ -1419,32 +1422,32 @@ __device__ MHD_NOINLINE double heatcool_delta(const Phys& ph, double rho, double
   const double nH2 = 0.5 * rh2, n = rho;
   double den3 = fma(3.0, nH, 5.0 * nH2);
   if (IONS) den3 = fma(6.0, rhp, den3);
-  const double T = ((2.0 * P0) * eint) / (den3 * ChemConst::KB);
+  const double T = ((2.0 * P0) * eint) / (den3 * ChemConst::KB), iT = rcp_nr(T);
   const double x = log10(T * 1e-4);
   // k1' and k4 (App. D, as in chem_cell)
   const double t2 = T * 0.01, s2 = sqrt(t2);
-  const double k1p = 3e-17 * s2 / (((1.0 + 0.4 * s2) + 0.2 * t2) + 0.08 * (t2 * t2));
+  const double k1p = (3e-17 * s2) * rcp_nr(((1.0 + 0.4 * s2) + 0.2 * t2) + 0.08 * (t2 * t2));
   const double Ls = (ph.lshield > 0.0 ? ph.lshield : ph.dx) * ChemConst::PC;
   const double NH = nH * Ls, NH2 = nH2 * Ls;
-  const double fdust = exp(-(ph.taud * (NH + NH2)));
+  const double fdust = exp_tang(-(ph.taud * (NH + NH2)));
   const double xs = NH2 * ph.ixnorm;
   const double u = 1.0 + xs * ph.ibdop;
   const double isx = rsqrt(1.0 + xs);
-  const double fsh = 0.965 / (u * u) + (0.035 * isx) * exp(-8.5e-4 * ((1.0 + xs) * isx));
+  const double fsh = 0.965 * rcp_nr(u * u) + (0.035 * isx) * exp_tang(-8.5e-4 * ((1.0 + xs) * isx));
   const double k4 = (3.3 * 1.7e-11) * fsh * fdust;
   // Gamma_1
   const double ncr = exp10(4.0 - 0.416 * x - 0.327 * x * x);
   const double G1 = 7.2e-12 * (k1p * n * nH) / (1.0 + ncr / n);
   // Lambda_2
-  const double LH2 = T > 1087.0 ? 3.9e-19 * exp(-6118.0 / T) : exp10(-19.24 + 0.474 * x - 1.247 * x * x);
+  const double LH2 = T > 1087.0 ? 3.9e-19 * exp_tang(-6118.0 * iT) : exp10(-19.24 + 0.474 * x - 1.247 * x * x);
   const double LL2 = (pow(nH2, 0.77) + 1.2 * pow(nH, 0.77)) *
-                     (T > 4031.0 ? 1.38e-22 * exp(-9243.0 / T) : exp10(-22.9 - 0.553 * x - 1.148 * x * x));
+                     (T > 4031.0 ? 1.38e-22 * exp_tang(-9243.0 * iT) : exp10(-22.9 - 0.553 * x - 1.148 * x * x));
   const double L2 = nH2 * LH2 / (1.0 + LH2 / LL2);
   // Lambda_3
-  const double LH3 = 1.1e-13 * exp(-6744.0 / T);
-  const double a = 1.0 + 1.0 / (KB_EV * T), a0 = 1.0 + 1.0 / (KB_EV * 4500.0);
-  const double lnf = (0.5 * log(T) + log(a)) + a, lnf0 = (0.5 * log(4500.0) + log(a0)) + a0;
-  const double kH2 = (6.29e-15 * 1.38) * exp(lnf - lnf0);
+  const double LH3 = 1.1e-13 * exp_tang(-6744.0 * iT);
+  // f(T) / f(4500 K) of f = sqrt(T) a e^a, a = 1 + 1 / (k_B T)
+  const double a = 1.0 + (1.0 / KB_EV) * iT, a0 = 1.0 + 1.0 / (KB_EV * 4500.0);
+  const double kH2 = ((6.29e-15 * 1.38) / (6.7082039324993690892 * a0)) * (s2 * a) * exp_tang(a - a0);  // sqrt(45)
   const double LL3 = 8.18e-13 * ((nH + nH2) * kH2);
   const double L3 = nH2 * LH3 / (1.0 + LH3 / LL3);
   // Gamma_4
