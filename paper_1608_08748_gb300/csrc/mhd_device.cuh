@@ -730,11 +730,12 @@ struct FixStep4 {
 // whether Step 4 may act (never false where it does): D- >= 0 >= D+, and by the high words |num| > 3 |s0| / 20
 // and |s0| > mn / 128.  A wide stencil, where the largest exponent is more than 5 above that of the cell and of one
 // of its neighbours (the results are at most a few times the smaller of the two differences, so the cut
-// would show), or with an infinity or a NaN, is done as a whole in FP64.
+// would show), or with an infinity, a NaN or a value of 2^1019 or more (3 A could overflow), is done as a whole in
+// FP64.
 __device__ __forceinline__ bool fix_dev(const FixCell c[5], Dev<double>& P, double& left, FixStep4& st) {
   const int near = max_i(c[2].e, min_i(c[1].e, c[3].e));
   const int E = max_i(max_i(max_i(c[0].e, c[1].e), max_i(c[3].e, c[4].e)), c[2].e);
-  const bool wide = E > near + 5 || E == 0x7ff;
+  const bool wide = E > near + 5 || E >= 0x7fa;
   long long q[5], d[4];
 #pragma unroll
   for (int k = 0; k < 5; ++k) q[k] = c[k].n >> min_i(E - c[k].e, 63);

@@ -111,8 +111,10 @@ int main() {
   const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
   long special = 0;
   for (int at = 0; at < 5; ++at)
-    for (double x : {inf, -inf, nan}) {
+    for (double x : {inf, -inf, nan, 5e306, 1e308, -1.7e308}) {
       double q[5] = {1, 2, 4, 5, 7};
+      if (x == 5e306)
+        for (double& v : q) v *= 2e306;
       q[at] = x;
       FixCell c[5];
       for (int i = 0; i < 5; ++i) c[i] = fix_cell(q[i]);
